@@ -570,12 +570,12 @@ rom_status rom_fom_create(int Nr, int Ntheta, double r_cmb, double r_earth, doub
                           double dt, rom_fom_t* out);
 rom_status rom_fom_destroy(rom_fom_t f);
 
-/* rom_fom_set_passes -- 1 (default): one fused pass per step that reads
- * and writes every state value once (8 bytes per unknown and realization
- * in FP32), ping-ponging between the caller's buffers and a library-owned
- * second set (allocated on the first run that needs it, sized by M); 2: a
- * velocity pass then a stress pass in place (12 bytes).  Both compute the
- * same arithmetic.  ROM_E_INVAL for another value. */
+/* rom_fom_set_passes -- 1 (default): fused passes that ping-pong between the
+ * caller's buffers and a library-owned second set (allocated on the first
+ * run that needs it, sized by M), two steps per pass in FP32 (4 bytes per
+ * unknown, realization and step), one in FP64 (16 bytes); 2: a velocity pass
+ * then a stress pass in place (12 bytes in FP32).  The values agree bit for
+ * bit in FP32.  ROM_E_INVAL for another value. */
 rom_status rom_fom_set_passes(rom_fom_t f, int passes);
 
 /* Unknowns per realization: velocity Nr (Ntheta - 1), sigma_rp
@@ -592,8 +592,9 @@ rom_status rom_fom_dims(rom_fom_t f, int* nv, int* n1, int* n2);
  * T (M periods, or NULL for no forcing) drives velocity unknown src.
  * recv (device int[nrecv], velocity unknowns) are recorded after every step
  * with (n + 1) mod r == 0 into traces[(rec nrecv + k) M + m] (NULL: none).
- * The run is a CUDA graph of 64 steps, captured on the first call for a
- * given set of buffers and arguments and replayed; it is asynchronous on
+ * Every 64 steps are one launch of a CUDA graph, captured on the first call
+ * for a given set of buffers and arguments and replayed; the fused form
+ * launches the remaining steps one pass at a time.  Asynchronous on
  * `stream` (the first fused run allocates the second buffer set).  A handle is not re-entrant across concurrent streams.  Errors:
  * ROM_E_INVAL (host buffers, bad indices), ROM_E_UNSUPPORTED (prec other than
  * ROM_FP32 / ROM_FP64), ROM_E_CUDA.

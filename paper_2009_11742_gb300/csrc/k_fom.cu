@@ -19,17 +19,18 @@
 //     V[k * M + m], k = i (Nt - 1) + (j - 1);  S1[k * M + m], k = (i - 1)(Nt - 1) + (j - 1);
 //     S2[k * M + m], k = i (Nt - 2) + (j - 1).
 // A warp reads whole M-vectors of its stencil neighbours, so every access
-// is coalesced and the stencil's reuse stays in L1/L2.  The run is bound by
-// HBM: 12 M bytes per unknown per step in FP32 (read V, S and write V in the
-// velocity pass; read V, S and write S in the stress pass).
+// is coalesced and the stencil's reuse stays in L1/L2.
 //
-// Per step: velocity kernel, point source, receiver record (on record
-// steps), stress kernel, and a one-thread tick of the device step counter.  The kernels
-// read the step from that counter, so a CUDA graph of kFomGraphSteps steps is
-// captured once per argument set and replayed; steps past nsteps are no-ops.
+// Two forms.  The fused form (default) marches blocks through the grid and
+// advances one or two steps per pass over the state (fom_march_kernel).  The
+// two-pass form runs a velocity kernel, the point source, the receiver
+// record, a stress kernel and a one-thread tick of the device step counter
+// per step, in place.  Both evaluate the stencils through the functions
+// below, so their values agree bit for bit.
 #include <cuda_runtime.h>
 #include <math.h>
 
+#include <initializer_list>
 #include <map>
 #include <mutex>
 #include <new>
@@ -43,7 +44,6 @@ namespace romk {
 
 constexpr int kFomThreads = 256;
 constexpr int kFomGraphSteps = 64;
-constexpr int kFomSegRows = 32;  // radial rows per block of the fused pass
 
 struct FomCtl {
     long long step, nsteps, n0;
@@ -75,12 +75,30 @@ struct FomArgs {
     const FomCtl* ctl;
     int Nr, Nt, M, src, nrecv, r, wavelet;
     double dt, rho;
-    // fused single pass: second buffer set (ping-pong by step parity), the
-    // source's grid point and the radial rows per block
-    T* V2;
-    T* S12;
-    T* S22;
-    int fused, src_i, src_j, seg_rows;
+};
+
+// One pass of the fused form: the state of step n = base + off is read from
+// the `o` buffers, that of step n + 1 (or n + 2) written to the `n` buffers;
+// base and n0 come from ctl (a pass of the graph) or are off and n0 alone.
+template <typename T>
+struct FomPass {
+    FomTables<T> tb;
+    const T* Vo;
+    const T* S1o;
+    const T* S2o;
+    T* Vn;
+    T* S1n;
+    T* S2n;
+    const T* Tper;
+    const int* recv;
+    T* traces;
+    const FomCtl* ctl;
+    long long off, n0;
+    int Nr, Nt, M, nrecv, r, wavelet;
+    int src_i, src_j;   // the source's grid point
+    int seg_rows;       // radial rows per block
+    int nmarch;         // blocks that march; those beyond record receivers
+    double dt, rho;
 };
 
 // Vector of VW consecutive realizations (16-byte loads when VW > 1).
@@ -104,6 +122,29 @@ __device__ __forceinline__ void fom_store(T* p, const T (&x)[VW]) {
 #pragma unroll
     for (int q = 0; q < VW; ++q) e[q] = x[q];
     *reinterpret_cast<typename FomVec<T, VW>::type*>(p) = v;
+}
+
+// The stencils, with every operation written out so that each caller (an
+// owner or a halo recomputing it, one or two steps a pass, either form)
+// rounds the same way.
+__device__ __forceinline__ float fom_fma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double fom_fma(double a, double b, double c) { return __fma_rn(a, b, c); }
+__device__ __forceinline__ float fom_mul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double fom_mul(double a, double b) { return __dmul_rn(a, b); }
+template <typename T>
+__device__ __forceinline__ T fom_vel(T v, T dt, T cp, T s1u, T cm, T s1d, T ir, T pp, T s2r, T pm, T s2l) {
+    const T radial = fom_fma(cp, s1u, -fom_mul(cm, s1d));
+    const T polar = fom_fma(pp, s2r, -fom_mul(pm, s2l));
+    return fom_fma(dt, fom_fma(ir, polar, radial), v);
+}
+// s += c (a x - b y): sigma_rp with c = dt, sigma_tp with c = dt / r.
+template <typename T>
+__device__ __forceinline__ T fom_str(T s, T c, T a, T x, T b, T y) {
+    return fom_fma(c, fom_fma(a, x, -fom_mul(b, y)), s);
+}
+template <typename T>
+__device__ __forceinline__ T fom_src(T v, T csrc, int wavelet, long long n, double dt, T Tm) {
+    return fom_fma(csrc, (T)wavelet_eval(wavelet, n, dt, Tm), v);
 }
 
 // Thread layout of the two passes: persistent blocks stride over tiles of
@@ -146,7 +187,7 @@ __global__ void __launch_bounds__(kFomThreads) fom_velocity_kernel(const FomArgs
             fom_load<T, VW>(v + m, y);
 #pragma unroll
             for (int q = 0; q < VW; ++q)
-                y[q] = y[q] + dt * (cp * x1p[q] - cm * x1m[q] + ir * (pp * x2p[q] - pm * x2m[q]));
+                y[q] = fom_vel(y[q], dt, cp, x1p[q], cm, x1m[q], ir, pp, x2p[q], pm, x2m[q]);
             fom_store<T, VW>(v + m, y);
         }
     }
@@ -161,7 +202,7 @@ __global__ void __launch_bounds__(kFomThreads) fom_source_kernel(const FomArgs<T
     const T c = (T)(a.dt / a.rho);
     T* v = a.V + (size_t)a.src * a.M;
     for (int m = blockIdx.x * blockDim.x + threadIdx.x; m < a.M; m += gridDim.x * blockDim.x)
-        v[m] = v[m] + c * (T)wavelet_eval(a.wavelet, a.ctl->n0 + n, a.dt, a.Tper[m]);
+        v[m] = fom_src(v[m], c, a.wavelet, a.ctl->n0 + n, a.dt, a.Tper[m]);
 }
 
 template <typename T>
@@ -170,111 +211,269 @@ __global__ void __launch_bounds__(kFomThreads) fom_record_kernel(const FomArgs<T
     if (n >= a.ctl->nsteps || ((n + 1) % a.r) != 0) return;
     const long long rec = (n + 1) / a.r - 1;
     const int tot = a.nrecv * a.M;
-    const T* V = (a.fused && !(n & 1)) ? a.V2 : a.V;  // the buffer this step wrote
     for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < tot; idx += gridDim.x * blockDim.x) {
         const int kk = idx / a.M, m = idx - kk * a.M;
-        a.traces[(rec * a.nrecv + kk) * a.M + m] = V[(long long)a.recv[kk] * a.M + m];
+        a.traces[(rec * a.nrecv + kk) * a.M + m] = a.V[(long long)a.recv[kk] * a.M + m];
     }
 }
 
-// Fused single pass of one step.  Reads the old state and writes the new
-// one into the other buffer set (step parity picks which), so neighbouring
-// blocks never see each other's writes within a step.  Block = a strip of
-// TJ = blockDim.y - 1 polar columns (thread row ty; ty = TJ is a halo column
-// whose new velocity the strip's last stress sigma_tp needs) times a segment
-// of seg_rows radial rows, marched outward in r: the lower sigma_rp face and
-// the previous row's new velocity stay in registers, the row's new velocity
-// goes through shared memory to the left neighbour.  The segment starts one
-// row early to recompute the new velocity below it.  Every state value is
-// read once and written once per step (plus the halo column and row), 8 M
-// bytes per unknown in FP32, against 12 M for the two passes.  The halo
-// values are computed by the same arithmetic as their owners' (forcing
-// included), so they are bitwise the owners' values.
-template <typename T, int VW>
-__global__ void __launch_bounds__(kFomThreads) fom_fused_kernel(const FomArgs<T> a) {
-    const long long n = a.ctl->step;
-    if (n >= a.ctl->nsteps) return;
-    const bool odd = (n & 1) != 0;
-    const T* __restrict__ Vo = odd ? a.V2 : a.V;
-    const T* __restrict__ S1o = odd ? a.S12 : a.S1;
-    const T* __restrict__ S2o = odd ? a.S22 : a.S2;
-    T* __restrict__ Vn = odd ? a.V : a.V2;
-    T* __restrict__ S1n = odd ? a.S1 : a.S12;
-    T* __restrict__ S2n = odd ? a.S2 : a.S22;
+// Receiver records of a pass: V^n as it was found (the record of step n - 1)
+// and, of a pass over two steps, V^{n+1}, which the march keeps on chip, from
+// the old state by the same arithmetic.
+template <typename T, int NS>
+__device__ __forceinline__ void fom_march_record(const FomPass<T>& a, long long n, long long n0) {
+    const bool rec0 = n > 0 && n % a.r == 0;
+    const bool rec1 = NS == 2 && (n + 1) % a.r == 0;
+    if (!rec0 && !rec1) return;
     const int Nt1 = a.Nt - 1, Nt2 = a.Nt - 2, M = a.M;
-    const int TJ = (int)blockDim.y - 1;
+    const T dt = (T)a.dt;
+    const long long tot = (long long)a.nrecv * M;
+    const long long nthr = (long long)(gridDim.x - a.nmarch) * kFomThreads;
+    const int tid = (int)(threadIdx.y * blockDim.x + threadIdx.x);
+    for (long long idx = (long long)(blockIdx.x - a.nmarch) * kFomThreads + tid; idx < tot; idx += nthr) {
+        const int kk = (int)(idx / M), m = (int)(idx - (long long)kk * M);
+        const long long u = a.recv[kk];
+        const T v = a.Vo[u * M + m];
+        if (rec0) a.traces[(n / a.r - 1) * tot + idx] = v;
+        if (rec1) {
+            const int i = (int)(u / Nt1), j = (int)(u - (long long)i * Nt1) + 1;
+            const T s1u = i + 1 < a.Nr ? a.S1o[((size_t)i * Nt1 + (j - 1)) * M + m] : T(0);
+            const T s1d = i >= 1 ? a.S1o[((size_t)(i - 1) * Nt1 + (j - 1)) * M + m] : T(0);
+            const T s2r = j <= Nt2 ? a.S2o[((size_t)i * Nt2 + (j - 1)) * M + m] : T(0);
+            const T s2l = j >= 2 ? a.S2o[((size_t)i * Nt2 + (j - 2)) * M + m] : T(0);
+            T vn = fom_vel(v, dt, a.tb.cr_p[i], s1u, a.tb.cr_m[i], s1d, a.tb.inv_rh[i], a.tb.pt_p[j], s2r,
+                           a.tb.pt_m[j], s2l);
+            if (a.Tper && i == a.src_i && j == a.src_j)
+                vn = fom_src(vn, (T)(a.dt / a.rho), a.wavelet, n0 + n, a.dt, a.Tper[m]);
+            a.traces[((n + 1) / a.r - 1) * tot + idx] = vn;
+        }
+    }
+}
+
+// Rows in flight per thread (512 x 2048, M = 32: 62.8 us a step with 3, 63.2
+// with 4), and resident blocks per SM (two-step pass: 128 registers a thread;
+// 3 blocks of 80 spill: 123 us).
+template <int NS>
+__host__ __device__ constexpr int fom_stages() { return NS == 2 ? 3 : 2; }
+template <int NS>
+__host__ __device__ constexpr int fom_occupancy() { return NS == 2 ? 2 : 4; }
+constexpr int kFomMaxSeg = 128;  // radial rows per block, at most
+
+// Asynchronous copy of B bytes to shared memory, zeros beyond src_bytes.
+template <int B, typename T>
+__device__ __forceinline__ void fom_cp_async(T* dst, const T* src, int src_bytes) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)),
+                 "l"(src), "n"(B), "r"(src_bytes)
+                 : "memory");
+}
+
+// One pass of the fused form over NS = 1 or 2 steps.  Reads the old state
+// from one buffer set and writes the new one to the other, so that
+// neighbouring blocks never see each other's writes.  A block takes a strip
+// of polar columns times a segment of seg_rows radial rows and marches
+// outward in r; thread row ty holds one column, threadIdx.x the realizations
+// in groups of VW.  The lower sigma_rp face and the previous row's new
+// velocity stay in registers; a row's new velocity goes through shared memory
+// to the column's neighbours.  Two steps run one row apart: once step n has
+// row i, its sigma_rp face i, and with them every input of step n + 1 at row
+// i - 1, is there.  Nothing of step n + 1's input touches memory.
+//  * Columns: strip s owns j in [s TJ + 1, s TJ + TJ].  NS = 1 needs one halo
+//    column on the right (sigma_tp takes the next column's new velocity).
+//    NS = 2 needs two there and one on the left, whose sigma_tp of step n the
+//    neighbour recomputes from the velocity in shared memory.
+//  * Rows: NS = 1 starts one row early to have the velocity below its first
+//    sigma_rp, NS = 2 two rows early, and reads one row past its end.
+// Halo values are computed by the owners' arithmetic (forcing included), so
+// they equal the owners' values bit for bit.
+// A thread's next rows are copied ahead into its own shared-memory slots, and
+// the row factors are staged there: with both read from global memory in the
+// loop a two-step pass was bound by their latency (96 us a step below).
+// Bound: memory.  NS = 1 moves 8 M bytes per unknown and step in FP32, NS = 2
+// half of that: 512 x 2048 grid, M = 32, 142 us a step with one step a pass
+// (85 % of the HBM copy rate), 61 us with two (98 %); M = 1, which stays in
+// L2, 25.4 and 5.8 us.  FP64 (NS = 1) is bound by the FP64 units, for which
+// the halo's extra work would be a loss.
+template <typename T, int VW, int NS>
+__global__ void __launch_bounds__(kFomThreads, fom_occupancy<NS>()) fom_march_kernel(const FomPass<T> a) {
+    const long long n = a.off + (a.ctl ? a.ctl->step : 0);
+    const long long n0 = a.ctl ? a.ctl->n0 : a.n0;
+    if ((int)blockIdx.x >= a.nmarch) {
+        fom_march_record<T, NS>(a, n, n0);
+        return;
+    }
+    constexpr int LH = NS - 1;                    // halo columns on the left
+    constexpr int STAGES = fom_stages<NS>();
+    constexpr int B = VW * (int)sizeof(T);
+    const int Nt1 = a.Nt - 1, Nt2 = a.Nt - 2, M = a.M, Nr = a.Nr;
+    const int by = (int)blockDim.y;
+    const int TJ = by - (2 * NS - 1);
     const int nstrip = (Nt1 + TJ - 1) / TJ;
     const int strip = (int)blockIdx.x % nstrip, seg = (int)blockIdx.x / nstrip;
     const int ia = seg * a.seg_rows;
-    const int ib = min(a.Nr, ia + a.seg_rows);
+    const int ib = min(Nr, ia + a.seg_rows);
     const int ty = threadIdx.y, tx = threadIdx.x;
-    const int j = strip * TJ + ty + 1;            // polar index of this thread's column
-    const bool act = j <= Nt1;                    // a velocity column
-    const bool own = act && ty < TJ;              // written by this block
+    const int j = strip * TJ + 1 - LH + ty;       // polar index of this thread's column
+    const bool act = j >= 1 && j <= Nt1;          // a velocity column
+    const bool own = act && ty >= LH && ty < LH + TJ;
+    const bool has_s2 = act && j <= Nt2, has_l = act && j >= 2;
     const T dt = (T)a.dt;
     const T pp = act ? a.tb.pt_p[j] : T(0), pm = act ? a.tb.pt_m[j] : T(0);
-    const bool has_s2 = own && j <= Nt2;
     const T wp = has_s2 ? a.tb.w_p[j] : T(0), wm = has_s2 ? a.tb.w_m[j] : T(0);
+    const T wpl = NS == 2 && has_l ? a.tb.w_p[j - 1] : T(0), wml = NS == 2 && has_l ? a.tb.w_m[j - 1] : T(0);
     const bool src_col = a.Tper && act && j == a.src_j;
-    const T csrc = (T)(a.dt / a.rho);
     extern __shared__ __align__(16) unsigned char fom_smem[];
-    T* row = reinterpret_cast<T*>(fom_smem);      // [blockDim.y][blockDim.x * VW] new velocity
-    const int i0 = ia > 0 ? ia - 1 : 0;
+    // [row parity][step][thread][VW] new velocity
+    T* row = reinterpret_cast<T*>(fom_smem);
+    constexpr int rstep = kFomThreads * VW;
+    T* slots = row + 2 * NS * rstep;              // [STAGES][V, S1, S2 right, S2 left][thread][VW]
+    T* rtab = slots + STAGES * 4 * rstep;         // [row i0 - 1 ..][cr_p, cr_m, 1/r, dt/r, q_u, q_d, -, -]
+    const int self = (ty * (int)blockDim.x + tx) * VW;
+    const int right = (min(ty + 1, by - 1) * (int)blockDim.x + tx) * VW;
+    const int left = (max(ty - 1, 0) * (int)blockDim.x + tx) * VW;
+    const int i0 = max(0, ia - NS);
+    const int iend = NS == 2 ? ib : ib - 1;       // last row of step n (row Nr is all zeros)
+    for (int k = ty * (int)blockDim.x + tx; k < iend - i0 + 2; k += kFomThreads) {
+        const int i = i0 - 1 + k;
+        const bool in = i >= 0 && i < Nr;         // zero factors outside the grid
+        T* e = rtab + 8 * k;
+        const T ir = in ? a.tb.inv_rh[i] : T(0);
+        e[0] = in ? a.tb.cr_p[i] : T(0);
+        e[1] = in ? a.tb.cr_m[i] : T(0);
+        e[2] = ir;
+        e[3] = fom_mul(dt, ir);
+        e[4] = in ? a.tb.q_u[i] : T(0);
+        e[5] = in ? a.tb.q_d[i] : T(0);
+    }
     const int chunk = (int)blockDim.x * VW;
+    const size_t rv = (size_t)Nt1 * M, r2 = (size_t)Nt2 * M;  // elements per row
     for (int mb = 0; mb < M; mb += chunk) {       // same trip count in every thread
         const int m0 = mb + tx * VW;
         const bool lane = act && m0 < M;
-        T prev_s1[VW], prev_v[VW];
+        const bool put = own && m0 < M, put2 = put && has_s2;
+        // addresses of inactive lanes stay on a valid element
+        const int jc = act ? j : 1, mc = m0 < M ? m0 : 0;
+        const size_t ov = (size_t)(jc - 1) * M + mc, o2 = (size_t)(min(jc, Nt2) - 1) * M + mc;
+        T s1d[VW], vp[VW];                        // step n: sigma_rp face i, new velocity of row i - 1
+        T t1d[VW], t2r[VW], t2l[VW], wprev[VW];   // step n + 1: face i - 1, sigma_tp of row i - 1, velocity of i - 2
 #pragma unroll
-        for (int q = 0; q < VW; ++q) prev_s1[q] = prev_v[q] = T(0);
-        if (lane && i0 >= 1) fom_load<T, VW>(S1o + ((size_t)(i0 - 1) * Nt1 + (j - 1)) * M + m0, prev_s1);
-        for (int i = i0; i < ib; ++i) {
-            T s1u[VW], s2r[VW], s2l[VW], vo[VW], vn[VW];
-#pragma unroll
-            for (int q = 0; q < VW; ++q) s1u[q] = s2r[q] = s2l[q] = vo[q] = T(0);
-            if (lane) {
-                if (i + 1 <= a.Nr - 1) fom_load<T, VW>(S1o + ((size_t)i * Nt1 + (j - 1)) * M + m0, s1u);
-                if (j <= Nt2) fom_load<T, VW>(S2o + ((size_t)i * Nt2 + (j - 1)) * M + m0, s2r);
-                if (j >= 2) fom_load<T, VW>(S2o + ((size_t)i * Nt2 + (j - 2)) * M + m0, s2l);
-                fom_load<T, VW>(Vo + ((size_t)i * Nt1 + (j - 1)) * M + m0, vo);
+        for (int q = 0; q < VW; ++q) s1d[q] = vp[q] = t1d[q] = t2r[q] = t2l[q] = wprev[q] = T(0);
+        if (lane && i0 >= 1) fom_load<T, VW>(a.S1o + (size_t)(i0 - 1) * rv + ov, s1d);
+        // rows are copied STAGES - 1 ahead into the thread's own slots
+        const T* gv = a.Vo + (size_t)i0 * rv + ov;
+        const T* g1 = a.S1o + (size_t)i0 * rv + ov;
+        const T* g2 = a.S2o + (size_t)i0 * r2 + o2;
+        const T* g2l = has_l ? a.S2o + (size_t)i0 * r2 + (size_t)(jc - 2) * M + mc : g2;
+        const int bv = lane ? B : 0, b2r = lane && has_s2 ? B : 0, b2l = lane && has_l ? B : 0;
+        int inext = i0, snext = 0, scur = 0;
+        auto fetch = [&]() {
+            if (inext <= iend) {
+                T* d = slots + snext * 4 * rstep + self;
+                const bool in = inext < Nr, face = inext + 1 < Nr;
+                fom_cp_async<B>(d, in ? gv : a.Vo, in ? bv : 0);
+                fom_cp_async<B>(d + rstep, face ? g1 : a.Vo, face ? bv : 0);
+                fom_cp_async<B>(d + 2 * rstep, in ? g2 : a.Vo, in ? b2r : 0);
+                fom_cp_async<B>(d + 3 * rstep, in ? g2l : a.Vo, in ? b2l : 0);
+                gv += rv;
+                g1 += rv;
+                g2 += r2;
+                g2l += r2;
+                snext = snext + 1 == STAGES ? 0 : snext + 1;
             }
-            const T cp = a.tb.cr_p[i], cm = a.tb.cr_m[i], ir = a.tb.inv_rh[i];
+            ++inext;
+            asm volatile("cp.async.commit_group;" ::: "memory");
+        };
 #pragma unroll
-            for (int q = 0; q < VW; ++q) vn[q] = vo[q] + dt * (cp * s1u[q] - cm * prev_s1[q] + ir * (pp * s2r[q] - pm * s2l[q]));
-            if (lane && src_col && i == a.src_i) {
+        for (int k = 0; k < STAGES - 1; ++k) fetch();
+        // outputs of row i (NS = 1) or i - 1 (NS = 2)
+        T* hv = a.Vn + (size_t)i0 * rv + ov - (NS - 1) * rv;
+        T* h1 = a.S1n + (size_t)i0 * rv + ov - NS * rv;
+        T* h2 = a.S2n + (size_t)i0 * r2 + o2 - (NS - 1) * r2;
+        __syncthreads();                          // rtab is there; the last chunk's rows are read
+        for (int i = i0; i <= iend; ++i) {
+            T* rb = row + (i & 1) * NS * rstep;
+            fetch();
+            asm volatile("cp.async.wait_group %0;" ::"n"(STAGES - 1) : "memory");
+            const T* d = slots + scur * 4 * rstep + self;
+            scur = scur + 1 == STAGES ? 0 : scur + 1;
+            T vo[VW], s1u[VW], s2r[VW], s2l[VW], vn[VW], s1n[VW], w[VW];
+            fom_load<T, VW>(d, vo);
+            fom_load<T, VW>(d + rstep, s1u);
+            fom_load<T, VW>(d + 2 * rstep, s2r);
+            fom_load<T, VW>(d + 3 * rstep, s2l);
+            const T* e = rtab + 8 * (i - i0 + 1);
+            const T c = e[3];
+#pragma unroll
+            for (int q = 0; q < VW; ++q)
+                vn[q] = fom_vel(vo[q], dt, e[0], s1u[q], e[1], s1d[q], e[2], pp, s2r[q], pm, s2l[q]);
+            if (src_col && i == a.src_i && m0 < M) {
 #pragma unroll
                 for (int q = 0; q < VW; ++q)
-                    vn[q] = vn[q] + csrc * (T)wavelet_eval(a.wavelet, a.ctl->n0 + n, a.dt, a.Tper[m0 + q]);
+                    vn[q] = fom_src(vn[q], (T)(a.dt / a.rho), a.wavelet, n0 + n, a.dt, a.Tper[m0 + q]);
             }
-            if (i >= ia) {                        // block-uniform
-                if (own && m0 < M) fom_store<T, VW>(Vn + ((size_t)i * Nt1 + (j - 1)) * M + m0, vn);
+            fom_store<T, VW>(rb + self, vn);
+            // the face below row i (of the first row: not used, or face 0, whose factors are 0)
 #pragma unroll
-                for (int q = 0; q < VW; ++q) row[(ty * blockDim.x + tx) * VW + q] = vn[q];
-                __syncthreads();
-                if (own && m0 < M) {
-                    if (i >= 1) {
-                        const T qu = a.tb.q_u[i], qd = a.tb.q_d[i];
-                        T s1[VW];
+            for (int q = 0; q < VW; ++q) s1n[q] = fom_str(s1d[q], dt, e[4], vn[q], e[5], vp[q]);
+            if (NS == 2) {
+                // step n + 1 at row i - 1 (the first rows' values are not used)
 #pragma unroll
-                        for (int q = 0; q < VW; ++q) s1[q] = prev_s1[q] + dt * (qu * vn[q] - qd * prev_v[q]);
-                        fom_store<T, VW>(S1n + ((size_t)(i - 1) * Nt1 + (j - 1)) * M + m0, s1);
-                    }
-                    if (has_s2) {
-                        T s2[VW];
+                for (int q = 0; q < VW; ++q)
+                    w[q] = fom_vel(vp[q], dt, e[-8], s1n[q], e[-7], t1d[q], e[-6], pp, t2r[q], pm, t2l[q]);
+                if (src_col && i - 1 == a.src_i && m0 < M) {
 #pragma unroll
-                        for (int q = 0; q < VW; ++q) {
-                            const T vr = row[((ty + 1) * blockDim.x + tx) * VW + q];
-                            s2[q] = s2r[q] + dt * ir * (wp * vr - wm * vn[q]);
-                        }
-                        fom_store<T, VW>(S2n + ((size_t)i * Nt2 + (j - 1)) * M + m0, s2);
+                    for (int q = 0; q < VW; ++q)
+                        w[q] = fom_src(w[q], (T)(a.dt / a.rho), a.wavelet, n0 + n + 1, a.dt, a.Tper[m0 + q]);
+                }
+                fom_store<T, VW>(rb + rstep + self, w);
+            }
+            __syncthreads();                      // rows are double-buffered by parity: one barrier a row
+            T vr[VW];
+            fom_load<T, VW>(rb + right, vr);
+            if (NS == 1) {
+                if (i >= ia) {
+                    if (put) fom_store<T, VW>(hv, vn);
+                    if (put && i >= 1) fom_store<T, VW>(h1, s1n);
+                    if (put2) {
+#pragma unroll
+                        for (int q = 0; q < VW; ++q) s2r[q] = fom_str(s2r[q], c, wp, vr[q], wm, vn[q]);
+                        fom_store<T, VW>(h2, s2r);
                     }
                 }
-                __syncthreads();
+            } else {
+                if (i > ia) {
+                    if (put) fom_store<T, VW>(hv, w);
+                    if (put && i >= 2) {
+                        T s1[VW];
+#pragma unroll
+                        for (int q = 0; q < VW; ++q) s1[q] = fom_str(t1d[q], dt, e[-4], w[q], e[-3], wprev[q]);
+                        fom_store<T, VW>(h1, s1);
+                    }
+                    if (put2) {
+                        T wr[VW];
+                        fom_load<T, VW>(rb + rstep + right, wr);
+#pragma unroll
+                        for (int q = 0; q < VW; ++q) wr[q] = fom_str(t2r[q], e[-5], wp, wr[q], wm, w[q]);
+                        fom_store<T, VW>(h2, wr);
+                    }
+                }
+                // sigma_tp of row i after step n, this column's and the left one's
+                T vl[VW];
+                fom_load<T, VW>(rb + left, vl);
+#pragma unroll
+                for (int q = 0; q < VW; ++q) {
+                    t2r[q] = fom_str(s2r[q], c, wp, vr[q], wm, vn[q]);
+                    t2l[q] = fom_str(s2l[q], c, wpl, vn[q], wml, vl[q]);
+                    t1d[q] = s1n[q];
+                    wprev[q] = w[q];
+                }
             }
+            hv += rv;
+            h1 += rv;
+            h2 += r2;
 #pragma unroll
             for (int q = 0; q < VW; ++q) {
-                prev_s1[q] = s1u[q];
-                prev_v[q] = vn[q];
+                s1d[q] = s1u[q];
+                vp[q] = vn[q];
             }
         }
     }
@@ -306,7 +505,7 @@ __global__ void __launch_bounds__(kFomThreads) fom_stress_kernel(const FomArgs<T
                 fom_load<T, VW>(vd + m, xd);
                 fom_load<T, VW>(s + m, y);
 #pragma unroll
-                for (int q = 0; q < VW; ++q) y[q] = y[q] + dt * (qu * xu[q] - qd * xd[q]);
+                for (int q = 0; q < VW; ++q) y[q] = fom_str(y[q], dt, qu, xu[q], qd, xd[q]);
                 fom_store<T, VW>(s + m, y);
             }
         } else {
@@ -325,7 +524,7 @@ __global__ void __launch_bounds__(kFomThreads) fom_stress_kernel(const FomArgs<T
                 fom_load<T, VW>(vl + m, xl);
                 fom_load<T, VW>(s + m, y);
 #pragma unroll
-                for (int q = 0; q < VW; ++q) y[q] = y[q] + dt * ir * (wp * xr[q] - wm * xl[q]);
+                for (int q = 0; q < VW; ++q) y[q] = fom_str(y[q], fom_mul(dt, ir), wp, xr[q], wm, xl[q]);
                 fom_store<T, VW>(s + m, y);
             }
         }
@@ -334,6 +533,21 @@ __global__ void __launch_bounds__(kFomThreads) fom_stress_kernel(const FomArgs<T
 
 __global__ void fom_tick_kernel(FomCtl* ctl) {
     if (ctl->step < ctl->nsteps) ctl->step = ctl->step + 1;
+}
+
+__global__ void fom_advance_kernel(FomCtl* ctl, int steps) { ctl->step = ctl->step + steps; }
+
+// Record of the final velocity of a fused run.
+template <typename T>
+__global__ void __launch_bounds__(kFomThreads) fom_last_record_kernel(const T* __restrict__ V,
+                                                                      const int* __restrict__ recv, int nrecv,
+                                                                      int M, T* __restrict__ out) {
+    const long long tot = (long long)nrecv * M;
+    for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < tot;
+         idx += (long long)gridDim.x * blockDim.x) {
+        const int kk = (int)(idx / M), m = (int)(idx - (long long)kk * M);
+        out[idx] = V[(long long)recv[kk] * M + m];
+    }
 }
 
 __global__ void fom_set_kernel(FomCtl* ctl, long long nsteps, long long n0) {
@@ -369,25 +583,127 @@ FomTables<T> tables_of(const rom_fom_s* f) {
     return {b, b + L, b + 2 * L, b + 3 * L, b + 4 * L, b + 5 * L, b + 6 * L, b + 7 * L, b + 8 * L};
 }
 
+// Launch shape of a run: 16-byte vectors along m when every row starts on a
+// 16-byte boundary; a block is bx realization groups x by polar points.
+struct FomShape {
+    bool wide;
+    int bx, by;
+};
 template <typename T>
-cudaError_t capture_steps(rom_fom_s* f, const FomArgs<T>& a, long long nv, long long ns,
-                          cudaGraphExec_t* out) {
-    // 16-byte vectors along m when every row starts on a 16-byte boundary
+FomShape fom_shape(int M, std::initializer_list<const void*> bufs) {
     constexpr int VWIDE = 16 / (int)sizeof(T);
-    bool wide = a.M % VWIDE == 0;
-    for (const void* p : {(const void*)a.V, (const void*)a.S1, (const void*)a.S2, (const void*)a.V2,
-                          (const void*)a.S12, (const void*)a.S22})
-        wide = wide && ((uintptr_t)p % 16 == 0);
-    const int vw = wide ? VWIDE : 1;
-    // block: bx realization groups x by polar points; persistent grid of
-    // blocks_per_sm blocks on every SM striding over the tiles
-    int bx = 1;
-    while (bx * vw < a.M && bx < 32) bx *= 2;
-    const int by = kFomThreads / bx;
-    const dim3 blk(bx, by, 1);
+    FomShape s{M % VWIDE == 0, 1, 0};
+    for (const void* p : bufs) s.wide = s.wide && ((uintptr_t)p % 16 == 0);
+    const int vw = s.wide ? VWIDE : 1;
+    while (s.bx * vw < M && s.bx < 32) s.bx *= 2;
+    s.by = kFomThreads / s.bx;
+    return s;
+}
+
+int fom_sm_count() {
     int dev = 0, nsm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    return nsm > 0 ? nsm : 1;
+}
+
+unsigned fom_blocks(long long work) {
+    const long long b = (work + kFomThreads - 1) / kFomThreads;
+    return (unsigned)(b < 1 ? 1 : (b > 1024 ? 1024 : b));
+}
+
+// Radial rows per block.  A block's time is its rows (seg plus the NS + 1 it
+// recomputes or looks ahead) and about two rows' worth of start-up; the blocks
+// run in waves of the resident ones.  Short segments fill the GPU when a grid
+// or M is small, long ones waste fewer rows.  Measured, us a step, FP32 on
+// 512 x 2048: M = 1 (9 strips) 6.4 / 5.8 / 7.2 / 12.2 at 8 / 16 / 32 / 64
+// rows, M = 32 (71 strips) 73 / 67 / 65 / 63 / 61 at 8 / 16 / 32 / 64 / 128;
+// the rule takes 16 and 128.
+template <int NS>
+int fom_seg_rows(int Nr, int nstrip, int nsm) {
+    const long long slots = (long long)nsm * fom_occupancy<NS>();
+    long long best = 0;
+    int seg = 1;
+    for (int s = 1; s <= kFomMaxSeg && s <= Nr; ++s) {
+        const long long waves = ((long long)nstrip * ((Nr + s - 1) / s) + slots - 1) / slots;
+        const long long t = waves * (s + NS + 3);
+        if (s == 1 || t < best) { best = t; seg = s; }
+    }
+    return seg;
+}
+
+template <typename T, int NS>
+cudaError_t launch_march(FomPass<T> a, const FomShape& s, int nsm, cudaStream_t st) {
+    constexpr int VWIDE = 16 / (int)sizeof(T);
+    const int TJ = s.by - (2 * NS - 1);
+    const int nstrip = (a.Nt - 1 + TJ - 1) / TJ;
+    a.seg_rows = fom_seg_rows<NS>(a.Nr, nstrip, nsm);
+    a.nmarch = nstrip * ((a.Nr + a.seg_rows - 1) / a.seg_rows);
+    const unsigned grid = (unsigned)a.nmarch + (a.traces ? fom_blocks((long long)a.nrecv * a.M) : 0u);
+    const dim3 blk(s.bx, s.by, 1);
+    const size_t smem = ((size_t)(2 * NS + 4 * fom_stages<NS>()) * kFomThreads * (s.wide ? VWIDE : 1) +
+                         (size_t)8 * (a.seg_rows + NS + 3)) * sizeof(T);
+    const void* fn = s.wide ? (const void*)fom_march_kernel<T, VWIDE, NS> : (const void*)fom_march_kernel<T, 1, NS>;
+    if (smem > 48 * 1024) cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (s.wide) fom_march_kernel<T, VWIDE, NS><<<grid, blk, smem, st>>>(a);
+    else fom_march_kernel<T, 1, NS><<<grid, blk, smem, st>>>(a);
+    return cudaGetLastError();
+}
+
+// Passes over `count` steps from step a.off on, two steps a pass in FP32.
+// The buffers alternate from pass to pass; with an odd number of passes the
+// result ends in the second set (*odd).  Of the FP32 splits of `count` into
+// two-step and one-step passes the one with the fewest passes of an even
+// number is taken (count = 1 alone has none), so no copy follows.
+template <typename T>
+cudaError_t march_steps(FomPass<T> a, const FomShape& s, int nsm, int count, cudaStream_t st, bool* odd) {
+    int pairs = sizeof(T) == 4 ? count / 2 : 0;
+    if ((count - pairs) % 2 != 0 && pairs > 0) --pairs;
+    const int passes = count - pairs;
+    cudaError_t e = cudaSuccess;
+    for (int p = 0; p < passes && e == cudaSuccess; ++p) {
+        const bool two = p < pairs;
+        if (two) e = launch_march<T, sizeof(T) == 4 ? 2 : 1>(a, s, nsm, st);
+        else e = launch_march<T, 1>(a, s, nsm, st);
+        a.off += two ? 2 : 1;
+        T *v = const_cast<T*>(a.Vo), *s1 = const_cast<T*>(a.S1o), *s2 = const_cast<T*>(a.S2o);
+        a.Vo = a.Vn; a.S1o = a.S1n; a.S2o = a.S2n;
+        a.Vn = v; a.S1n = s1; a.S2n = s2;
+    }
+    *odd = passes % 2 != 0;
+    return e;
+}
+
+cudaError_t end_capture(cudaStream_t cap, cudaError_t e, cudaGraphExec_t* out) {
+    cudaGraph_t g = nullptr;
+    const cudaError_t e2 = cudaStreamEndCapture(cap, &g);
+    if (e == cudaSuccess) e = e2;
+    if (e == cudaSuccess) e = cudaGraphInstantiate(out, g, 0);
+    if (g) cudaGraphDestroy(g);
+    return e;
+}
+
+// The fused form's graph: kFomGraphSteps steps from step ctl->step on.
+template <typename T>
+cudaError_t capture_march(rom_fom_s* f, FomPass<T> a, const FomShape& s, int nsm, cudaGraphExec_t* out) {
+    cudaError_t e = cudaStreamBeginCapture(f->cap, cudaStreamCaptureModeThreadLocal);
+    if (e != cudaSuccess) return e;
+    bool odd = false;
+    a.off = 0;
+    e = march_steps<T>(a, s, nsm, kFomGraphSteps, f->cap, &odd);
+    if (e == cudaSuccess) {
+        fom_advance_kernel<<<1, 1, 0, f->cap>>>(f->ctl, kFomGraphSteps);
+        e = cudaGetLastError();
+    }
+    return end_capture(f->cap, e, out);
+}
+
+// The two-pass form's graph: kFomGraphSteps steps, steps past nsteps idle.
+template <typename T>
+cudaError_t capture_steps(rom_fom_s* f, const FomArgs<T>& a, const FomShape& s, int nsm, cudaGraphExec_t* out) {
+    constexpr int VWIDE = 16 / (int)sizeof(T);
+    const dim3 blk(s.bx, s.by, 1);
+    // persistent grids: the resident blocks of every SM stride over the tiles
     auto grid_for = [&](const void* fn, long long tiles) {
         int per = 0;
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, kFomThreads, 0) != cudaSuccess || per < 1)
@@ -395,42 +711,122 @@ cudaError_t capture_steps(rom_fom_s* f, const FomArgs<T>& a, long long nv, long 
         const long long g = (long long)nsm * per;
         return (unsigned)(tiles < g ? (tiles < 1 ? 1 : tiles) : g);
     };
-    const long long gx = (a.Nt - 1 + by - 1) / by;
-    const void* fv = wide ? (const void*)fom_velocity_kernel<T, VWIDE> : (const void*)fom_velocity_kernel<T, 1>;
-    const void* fs = wide ? (const void*)fom_stress_kernel<T, VWIDE> : (const void*)fom_stress_kernel<T, 1>;
+    const long long gx = (a.Nt - 1 + s.by - 1) / s.by;
+    const void* fv = s.wide ? (const void*)fom_velocity_kernel<T, VWIDE> : (const void*)fom_velocity_kernel<T, 1>;
+    const void* fs = s.wide ? (const void*)fom_stress_kernel<T, VWIDE> : (const void*)fom_stress_kernel<T, 1>;
     const unsigned gv = grid_for(fv, (long long)a.Nr * gx);
     const unsigned gs = grid_for(fs, (long long)(2 * a.Nr - 1) * gx);
-    auto blocks = [&](long long work) {
-        const long long b = (work + kFomThreads - 1) / kFomThreads;
-        return (unsigned)(b < 1 ? 1 : (b > 1024 ? 1024 : b));
-    };
-    // fused pass: strips of by - 1 polar columns x segments of seg_rows radial rows
-    const unsigned gfused = (unsigned)(((a.Nt - 1 + by - 2) / (by - 1)) * ((a.Nr + a.seg_rows - 1) / a.seg_rows));
-    const size_t fsmem = (size_t)by * bx * vw * sizeof(T);
     cudaError_t e = cudaStreamBeginCapture(f->cap, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return e;
-    for (int s = 0; s < kFomGraphSteps && e == cudaSuccess && a.fused; ++s) {
-        if (wide) fom_fused_kernel<T, VWIDE><<<gfused, blk, fsmem, f->cap>>>(a);
-        else fom_fused_kernel<T, 1><<<gfused, blk, fsmem, f->cap>>>(a);
-        if (a.traces) fom_record_kernel<T><<<blocks((long long)a.nrecv * a.M), kFomThreads, 0, f->cap>>>(a);
-        fom_tick_kernel<<<1, 1, 0, f->cap>>>(const_cast<FomCtl*>(a.ctl));
-        e = cudaGetLastError();
-    }
-    for (int s = 0; s < kFomGraphSteps && e == cudaSuccess && !a.fused; ++s) {
-        if (wide) fom_velocity_kernel<T, VWIDE><<<gv, blk, 0, f->cap>>>(a);
+    for (int k = 0; k < kFomGraphSteps && e == cudaSuccess; ++k) {
+        if (s.wide) fom_velocity_kernel<T, VWIDE><<<gv, blk, 0, f->cap>>>(a);
         else fom_velocity_kernel<T, 1><<<gv, blk, 0, f->cap>>>(a);
-        if (a.Tper) fom_source_kernel<T><<<blocks(a.M), kFomThreads, 0, f->cap>>>(a);
-        if (a.traces) fom_record_kernel<T><<<blocks((long long)a.nrecv * a.M), kFomThreads, 0, f->cap>>>(a);
-        if (wide) fom_stress_kernel<T, VWIDE><<<gs, blk, 0, f->cap>>>(a);
+        if (a.Tper) fom_source_kernel<T><<<fom_blocks(a.M), kFomThreads, 0, f->cap>>>(a);
+        if (a.traces) fom_record_kernel<T><<<fom_blocks((long long)a.nrecv * a.M), kFomThreads, 0, f->cap>>>(a);
+        if (s.wide) fom_stress_kernel<T, VWIDE><<<gs, blk, 0, f->cap>>>(a);
         else fom_stress_kernel<T, 1><<<gs, blk, 0, f->cap>>>(a);
         fom_tick_kernel<<<1, 1, 0, f->cap>>>(const_cast<FomCtl*>(a.ctl));
         e = cudaGetLastError();
     }
-    cudaGraph_t g = nullptr;
-    const cudaError_t e2 = cudaStreamEndCapture(f->cap, &g);
-    if (e == cudaSuccess) e = e2;
-    if (e == cudaSuccess) e = cudaGraphInstantiate(out, g, 0);
-    if (g) cudaGraphDestroy(g);
+    return end_capture(f->cap, e, out);
+}
+
+// The checked arguments of one rom_fom_run call.
+struct FomRun {
+    void *V, *S1, *S2, *V2, *S12, *S22;
+    const void* T;
+    const int* recv;
+    void* traces;
+    int M, nsteps;
+    long n0;
+    int src, wavelet, nrecv, r;
+    bool fused;
+};
+
+// The graph of a run's buffers and arguments, captured on its first use.
+template <typename F>
+cudaError_t cached_graph(rom_fom_s* f, const std::vector<long long>& key, cudaStream_t st, F capture,
+                         cudaGraphExec_t* out) {
+    auto it = f->graphs.find(key);
+    if (it == f->graphs.end()) {
+        cudaGraphExec_t ge = nullptr;
+        const cudaError_t e = capture(&ge);
+        if (e != cudaSuccess) return e;
+        if (f->graphs.size() >= 16) {  // keep the cache small
+            cudaStreamSynchronize(st);
+            for (auto& kv : f->graphs) cudaGraphExecDestroy(kv.second);
+            f->graphs.clear();
+        }
+        it = f->graphs.emplace(key, ge).first;
+    }
+    *out = it->second;
+    return cudaSuccess;
+}
+
+template <typename T>
+cudaError_t run_fom(rom_fom_s* f, const FomRun& q, cudaStream_t st) {
+    const size_t nv = (size_t)f->Nr * (f->Nt - 1), n1 = (size_t)(f->Nr - 1) * (f->Nt - 1),
+                 n2 = (size_t)f->Nr * (f->Nt - 2);
+    const int nsm = fom_sm_count();
+    const FomShape s = fom_shape<T>(q.M, {q.V, q.S1, q.S2, q.V2, q.S12, q.S22});
+    const std::vector<long long> key = {(long long)(uintptr_t)q.V, (long long)(uintptr_t)q.S1,
+                                        (long long)(uintptr_t)q.S2, q.M, q.src, (long long)(uintptr_t)q.T,
+                                        q.wavelet, (long long)(uintptr_t)q.recv, q.nrecv, q.traces ? q.r : 0,
+                                        (long long)(uintptr_t)q.traces, (long long)sizeof(T), q.fused,
+                                        (long long)(uintptr_t)q.V2};
+    cudaGraphExec_t ge = nullptr;
+    cudaError_t e = cudaSuccess;
+    if (!q.fused) {
+        const FomArgs<T> a = {tables_of<T>(f), static_cast<T*>(q.V), static_cast<T*>(q.S1), static_cast<T*>(q.S2),
+                              static_cast<const T*>(q.T), q.recv, static_cast<T*>(q.traces), f->ctl, f->Nr, f->Nt,
+                              q.M, q.src, q.nrecv, q.r, q.wavelet, f->dt, f->rho};
+        e = cached_graph(f, key, st, [&](cudaGraphExec_t* g) { return capture_steps<T>(f, a, s, nsm, g); }, &ge);
+        if (e != cudaSuccess) return e;
+        fom_set_kernel<<<1, 1, 0, st>>>(f->ctl, q.nsteps, q.n0);
+        e = cudaGetLastError();
+        for (int k = 0; k < (q.nsteps + kFomGraphSteps - 1) / kFomGraphSteps && e == cudaSuccess; ++k)
+            e = cudaGraphLaunch(ge, st);
+        return e;
+    }
+    FomPass<T> a{};
+    a.tb = tables_of<T>(f);
+    a.Vo = static_cast<T*>(q.V), a.S1o = static_cast<T*>(q.S1), a.S2o = static_cast<T*>(q.S2);
+    a.Vn = static_cast<T*>(q.V2), a.S1n = static_cast<T*>(q.S12), a.S2n = static_cast<T*>(q.S22);
+    a.Tper = static_cast<const T*>(q.T);
+    a.recv = q.recv;
+    a.traces = static_cast<T*>(q.traces);
+    a.n0 = q.n0;
+    a.Nr = f->Nr, a.Nt = f->Nt, a.M = q.M;
+    a.nrecv = q.nrecv, a.r = q.r, a.wavelet = q.wavelet;
+    a.src_i = q.src >= 0 ? q.src / (f->Nt - 1) : -1;
+    a.src_j = q.src >= 0 ? q.src % (f->Nt - 1) + 1 : -1;
+    a.dt = f->dt, a.rho = f->rho;
+    // whole groups of kFomGraphSteps steps by graph, the rest launched
+    const int reps = q.nsteps / kFomGraphSteps;
+    if (reps > 0) {
+        FomPass<T> g = a;
+        g.ctl = f->ctl;
+        e = cached_graph(f, key, st, [&](cudaGraphExec_t* x) { return capture_march<T>(f, g, s, nsm, x); }, &ge);
+        if (e != cudaSuccess) return e;
+        fom_set_kernel<<<1, 1, 0, st>>>(f->ctl, q.nsteps, q.n0);
+        e = cudaGetLastError();
+        for (int k = 0; k < reps && e == cudaSuccess; ++k) e = cudaGraphLaunch(ge, st);
+    }
+    bool odd = false;
+    a.off = (long long)reps * kFomGraphSteps;
+    if (e == cudaSuccess) e = march_steps<T>(a, s, nsm, q.nsteps - reps * kFomGraphSteps, st, &odd);
+    if (e == cudaSuccess && odd) {
+        e = cudaMemcpyAsync(q.V, q.V2, nv * q.M * sizeof(T), cudaMemcpyDeviceToDevice, st);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(q.S1, q.S12, n1 * q.M * sizeof(T), cudaMemcpyDeviceToDevice, st);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(q.S2, q.S22, n2 * q.M * sizeof(T), cudaMemcpyDeviceToDevice, st);
+    }
+    if (e == cudaSuccess && a.traces && q.nsteps % q.r == 0) {
+        // a pass records the velocity it finds: the last step's record is left
+        fom_last_record_kernel<T><<<fom_blocks((long long)q.nrecv * q.M), kFomThreads, 0, st>>>(
+            static_cast<const T*>(q.V), q.recv, q.nrecv, q.M,
+            a.traces + (size_t)(q.nsteps / q.r - 1) * q.nrecv * q.M);
+        e = cudaGetLastError();
+    }
     return e;
 }
 
@@ -602,57 +998,8 @@ rom_status rom_fom_run(rom_fom_t f, void* V, void* S1, void* S2, int M, int nste
         S12 = w + al((size_t)nv * M * es);
         S22 = w + al((size_t)nv * M * es) + al((size_t)(f->Nr - 1) * (f->Nt - 1) * M * es);
     }
-    const int src_i = src >= 0 ? (int)(src / (f->Nt - 1)) : -1;
-    const int src_j = src >= 0 ? (int)(src % (f->Nt - 1)) + 1 : -1;
-    const std::vector<long long> key = {(long long)(uintptr_t)V, (long long)(uintptr_t)S1,
-                                        (long long)(uintptr_t)S2, M, src, (long long)(uintptr_t)T,
-                                        wavelet, (long long)(uintptr_t)recv, nrecv, traces ? r : 0,
-                                        (long long)(uintptr_t)traces, prec, fused,
-                                        (long long)(uintptr_t)V2};
-    auto it = f->graphs.find(key);
-    if (it == f->graphs.end()) {
-        cudaGraphExec_t ge = nullptr;
-        cudaError_t e;
-        if (prec == ROM_FP64) {
-            FomArgs<double> a = {tables_of<double>(f), static_cast<double*>(V), static_cast<double*>(S1),
-                                 static_cast<double*>(S2), static_cast<const double*>(T), recv,
-                                 static_cast<double*>(traces), f->ctl, f->Nr, f->Nt, M, src, nrecv,
-                                 traces ? r : 1, wavelet, f->dt, f->rho,
-                                 static_cast<double*>(V2), static_cast<double*>(S12), static_cast<double*>(S22),
-                                 fused ? 1 : 0, src_i, src_j, kFomSegRows};
-            e = capture_steps<double>(f, a, nv, ns, &ge);
-        } else {
-            FomArgs<float> a = {tables_of<float>(f), static_cast<float*>(V), static_cast<float*>(S1),
-                                static_cast<float*>(S2), static_cast<const float*>(T), recv,
-                                static_cast<float*>(traces), f->ctl, f->Nr, f->Nt, M, src, nrecv,
-                                traces ? r : 1, wavelet, f->dt, f->rho,
-                                static_cast<float*>(V2), static_cast<float*>(S12), static_cast<float*>(S22),
-                                fused ? 1 : 0, src_i, src_j, kFomSegRows};
-            e = capture_steps<float>(f, a, nv, ns, &ge);
-        }
-        if (e != cudaSuccess) {
-            set_last_error(cudaGetErrorString(e));
-            return ROM_E_CUDA;
-        }
-        if (f->graphs.size() >= 16) {  // keep the cache small
-            cudaStreamSynchronize(st);
-            for (auto& kv : f->graphs) cudaGraphExecDestroy(kv.second);
-            f->graphs.clear();
-        }
-        it = f->graphs.emplace(key, ge).first;
-    }
-    fom_set_kernel<<<1, 1, 0, st>>>(f->ctl, nsteps, n0);
-    cudaError_t e = cudaGetLastError();
-    const int reps = (nsteps + kFomGraphSteps - 1) / kFomGraphSteps;
-    for (int k = 0; k < reps && e == cudaSuccess; ++k) e = cudaGraphLaunch(it->second, st);
-    if (e == cudaSuccess && fused && (nsteps & 1)) {
-        // an odd number of fused steps leaves the result in the second buffer set
-        e = cudaMemcpyAsync(V, V2, (size_t)nv * M * es, cudaMemcpyDeviceToDevice, st);
-        if (e == cudaSuccess)
-            e = cudaMemcpyAsync(S1, S12, (size_t)(f->Nr - 1) * (f->Nt - 1) * M * es, cudaMemcpyDeviceToDevice, st);
-        if (e == cudaSuccess)
-            e = cudaMemcpyAsync(S2, S22, (size_t)f->Nr * (f->Nt - 2) * M * es, cudaMemcpyDeviceToDevice, st);
-    }
+    FomRun q{V, S1, S2, V2, S12, S22, T, recv, traces, M, nsteps, n0, src, wavelet, nrecv, traces ? r : 1, fused};
+    const cudaError_t e = prec == ROM_FP64 ? run_fom<double>(f, q, st) : run_fom<float>(f, q, st);
     if (e != cudaSuccess) {
         set_last_error(cudaGetErrorString(e));
         return ROM_E_CUDA;

@@ -773,8 +773,8 @@ class Fom:
             self.h = None
 
     def set_passes(self, passes):
-        """1: fused single pass (default, 8 B per unknown and realization
-        in FP32); 2: velocity pass then stress pass (12 B)."""
+        """1: fused passes (default; FP32: two steps a pass, 4 B per unknown,
+        realization and step); 2: velocity pass then stress pass (12 B)."""
         _chk(rom_fom_set_passes(self.h, passes), "rom_fom_set_passes")
 
     def vindex(self, i, j):

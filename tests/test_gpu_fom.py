@@ -136,9 +136,9 @@ def test_fom_rank2_equals_rank1_bitwise(rom):
 @pytest.mark.parametrize("passes", [1, 2])
 def test_fom_chunked_equals_one_run_and_zero(rom, passes):
     """n0 continues the forcing clock: 71 + 129 steps equal 200 steps
-    bitwise (the 64-step graph is replayed with steps past the end idle; an
-    odd count ends in the fused pass's second buffer set and is copied
-    back); zero state without forcing stays exactly zero."""
+    bitwise (the two-pass form replays its 64-step graph with steps past
+    the end idle; an odd FP64 count ends in the fused form's second buffer
+    set and is copied back); zero state without forcing stays exactly zero."""
     Nr, Nt, M = 12, 20, 3
     f = rom.Fom(Nr, Nt, dt=stable_dt(Nr, Nt))
     f.set_passes(passes)
@@ -170,6 +170,30 @@ def test_fom_fused_equals_two_passes(rom):
         outs.append(gpu_run(rom, f, X0, N, "fp32", src=src, T=T, recv=[src, f.vindex(Nr - 1, 5)], r=3))
     for k in range(4):
         assert rel(outs[0][k], outs[1][k]) <= 1e-6, k
+
+
+@pytest.mark.parametrize("Nr,Nt,M,nsteps", [
+    (2, 3, 1, 1), (2, 3, 4, 2), (3, 4, 2, 3), (5, 33, 33, 5), (9, 260, 1, 6), (40, 31, 32, 7), (33, 90, 36, 64),
+    (150, 256, 3, 67), (131, 515, 1, 130), (300, 64, 160, 9)])
+def test_fom_fused_bitwise_two_passes(rom, Nr, Nt, M, nsteps):
+    """Every split of a run into one- and two-step passes, at the edges of
+    strips, segments and realization groups, records on every step: the fused
+    form equals the two-pass form bit for bit, state and records."""
+    f = rom.Fom(Nr, Nt, dt=0.01)
+    X0 = case(Nr, Nt, M, seed=Nr + nsteps)
+    T = np.linspace(60.0, 80.0, M)
+    outs = []
+    for passes in (1, 2):
+        f.set_passes(passes)
+        for src in sorted({0, f.nv // 2, f.nv - 1}):
+            for r in (1, 2, 3):
+                if r <= nsteps:
+                    outs.append(gpu_run(rom, f, X0, nsteps, "fp32", src=src, T=T, n0=7000, r=r,
+                                        recv=[0, src, f.nv - 1]))
+    half = len(outs) // 2
+    for a, b in zip(outs[:half], outs[half:]):
+        for x, y in zip(a, b):
+            assert np.array_equal(x, y)
 
 
 def test_fom_rejects_bad_arguments(rom):
