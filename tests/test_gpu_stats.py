@@ -47,6 +47,34 @@ def test_stats_with_ties_and_signed_zeros(rom):
     check(rom, x)
 
 
+@pytest.mark.parametrize("M", [1, 31, 32, 33, 64, 65, 128, 129, 256, 257, 511, 512, 513, 1023, 1025, 2048, 2049, 4095])
+@pytest.mark.parametrize("R", [1, 7, 33])
+def test_stats_sort_widths(rom, M, R):
+    """Both sides of every sort width and tile shape, values over the whole
+    range of exponents (the mean's bound: FP64 summation-order rounding)."""
+    rng = np.random.default_rng(M * 100 + R)
+    x = rng.standard_normal((5, M, R)) * 10.0 ** rng.integers(-30, 8, (5, M, R))
+    check(rom, x.astype(np.float32))
+
+
+def test_stats_extreme_scales(rom):
+    """All-zero, denormal and largest-magnitude columns, and columns with an
+    infinity (kept in order; their mean is not finite)."""
+    rng = np.random.default_rng(3)
+    x = rng.standard_normal((4, 70, 3))
+    x[0] = 0.0
+    x[1] *= 1e-42
+    x[2] *= 1e37
+    check(rom, x.astype(np.float32))
+    x = x.astype(np.float32)
+    x[3, 5, :] = np.inf
+    x[3, 9, 1] = -np.inf
+    mean, q = rom.trace_stats(torch.as_tensor(x, device="cuda"), PS)
+    with np.errstate(invalid="ignore"):
+        np.testing.assert_array_equal(q.cpu().numpy(), oracle.trace_stats(x, PS)[1])
+    assert not np.isfinite(mean[3].cpu().numpy()).any()
+
+
 def test_stats_of_simulated_traces(rom):
     """Traces from a rank-2 run (the intended use)."""
     from paper_2009_11742_gb300 import inputs
