@@ -127,7 +127,8 @@ rom_status rom_get_dims(rom_t h, int* Kv, int* Ks, int* R, double* dt);
 
 /* Kernel selection for the rank-2 FP32 path (the FP64 path always uses the
  * one-block kernel):
- *  ROM_KERNEL_AUTO      planner's choice (default: two-block);
+ *  ROM_KERNEL_AUTO      planner's choice (default: two-block above Kp = 128,
+ *                       one CTA per column block, without clusters, up to it);
  *  ROM_KERNEL_ONE_BLOCK one column block per cluster, every CTA owns 32 rows
  *                       of both V and S;
  *  ROM_KERNEL_TWO_BLOCK two column blocks per cluster half a step apart,
@@ -145,7 +146,7 @@ rom_status rom_set_kernel(rom_t h, int kernel);
 /* The launch plan the handle would use for M realizations at precision prec
  * (ROM_FP32 or ROM_FP64): kernel variant (1 one-block, 2 two-block, 3
  * dataflow, 4 two-block with the streaming companion of rom_set_companion on
- * the last columns), cluster size, columns per column block and number of
+ * the last columns, 5 one CTA per column block), cluster size, columns per column block and number of
  * clusters of the main kernel (outputs may be NULL).  ROM_E_UNSUPPORTED for
  * another precision or if no kernel fits. */
 rom_status rom_get_plan(rom_t h, int prec, int M, int* variant, int* cluster_size,
@@ -191,7 +192,7 @@ rom_status rom_get_companion(rom_t h, int M, int* cluster_size, int* nclusters, 
  * rom_run_rank2_ex calls with the same precision and M use it while the
  * kernel choice (rom_set_kernel) and the tensor-core width
  * (rom_set_tc_columns) are automatic.  Candidates:
- *   ROM_FP32  the two-block and the one-block kernels, each with the cluster
+ *   ROM_FP32  the one-CTA kernel (up to Kp = 128); the two-block and the one-block kernels, each with the cluster
  *             count capped at the co-resident maximum, half and a quarter of
  *             it (wider column blocks on fewer clusters); and, when the
  *             two-block kernel fills every cluster that fits, the same with

@@ -180,16 +180,17 @@ __device__ __forceinline__ void rs32_stage(float (&v)[16], int lane, int o) {
 
 // Receiver traces y = C V^{n+1} of one block (Sec. 4.5.2): out[c R + jj] for
 // this CTA's nj receiver rows Cown (row-major, Kp wide) and the nc columns of
-// the new V in Xb (column-major, Kp rows).  A warp takes a tile of 4
+// the new V in Xb (columns xstride apart, Kp rows), dealt out to nwarps warps.  A warp takes a tile of 4
 // receivers x 4 columns over the whole K: each lane sums 4-wide stripes of k
 // into 16 independent accumulators, then a 32-lane reduce-scatter (fixed
 // order) leaves entry lane / 2 of the tile in lanes 2e and 2e + 1.
 __device__ __forceinline__ void split_traces(const float* __restrict__ Cown, const float* __restrict__ Xb,
                                              int Kp, int nj, int nc, int warp, int lane,
-                                             float* __restrict__ out, int R) {
+                                             float* __restrict__ out, int R, int xstride,
+                                             int nwarps) {
     const int tcn = (nc + 3) >> 2;
     const int ntile = ((nj + 3) >> 2) * tcn;
-    for (int t = warp; t < ntile; t += kSplitWarps) {
+    for (int t = warp; t < ntile; t += nwarps) {
         const int tj = t / tcn;
         const int j0 = 4 * tj, c0 = 4 * (t - tj * tcn);
         float acc[16];
@@ -201,7 +202,7 @@ __device__ __forceinline__ void split_traces(const float* __restrict__ Cown, con
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 load4(Cown + (size_t)min(j0 + u, nj - 1) * Kp + k, cv[u]);
-                load4(Xb + (size_t)min(c0 + u, nc - 1) * Kp + k, xv[u]);
+                load4(Xb + (size_t)min(c0 + u, nc - 1) * xstride + k, xv[u]);
             }
 #pragma unroll
             for (int u = 0; u < 4; ++u)
@@ -342,7 +343,7 @@ __device__ __forceinline__ void split_body(cg::cluster_group& cluster, const Ran
                     const int rec = (n + 1) / a.r - 1;
                     const int nj = min(a.rpc, a.R - s * a.rpc);  // this CTA's receivers
                     split_traces(Cown, Xb, Kp, nj > 0 ? nj : 0, ncol(b), warp, lane,
-                                 traces + ((size_t)rec * a.Mtot + gc0(b)) * a.R + s * a.rpc, a.R);
+                                 traces + ((size_t)rec * a.Mtot + gc0(b)) * a.R + s * a.rpc, a.R, Kp, kSplitWarps);
                 }
             }
         }

@@ -254,7 +254,7 @@ __global__ void __launch_bounds__(kStrThreads, 1) rank2_stream_kernel(const Rank
                     const int nj = min(rpc, a.R - sl * rpc);
                     if (nj <= 0) break;
                     split_traces(Cp + (size_t)sl * rpc * Kp, Vf, Kp, nj, ncol, warp, lane,
-                                 traces + ((size_t)rec * a.Mtot + col0) * a.R + sl * rpc, a.R);
+                                 traces + ((size_t)rec * a.Mtot + col0) * a.R + sl * rpc, a.R, Kp, kSplitWarps);
                 }
             }
         }

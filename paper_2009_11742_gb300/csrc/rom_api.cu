@@ -388,9 +388,14 @@ rom_status get_plan(rom_s* h, int prec, int M, bool rank1, Rank2Plan* plan) {
     // FP32 with more than one realization: the two-block split-role kernel,
     // unless the caller pinned the one-block kernel.
     const bool two_block = prec != ROM_FP64 && !rank1 && h->kernel_choice != ROM_KERNEL_ONE_BLOCK;
-    if (two_block && h->kernel_choice == ROM_KERNEL_DATAFLOW) {
+    // Small models run one CTA per column block unless the caller pinned a
+    // cluster kernel or a companion: no cluster barrier in the step, the same
+    // bits (see rank2_cta.cuh for both sides' times).
+    if (prec != ROM_FP64 && h->Kp <= 128 && h->kernel_choice == ROM_KERNEL_AUTO && h->comp_cs <= 0)
+        ok = plan_rank2_cta_f32(h->Kp, M, h->R, plan);
+    if (!ok && two_block && h->kernel_choice == ROM_KERNEL_DATAFLOW) {
         ok = plan_rank2_dataflow_f32(h->Kp, M, h->R, plan);
-    } else if (two_block) {
+    } else if (!ok && two_block) {
         ok = plan_rank2_split_f32(h->Kp, M, h->R, plan);
         // the streaming companion on the SMs the split kernel's clusters
         // leave idle (automatic kernel choice only)
@@ -601,6 +606,7 @@ rom_status launch_simt_with_plan(rom_s* h, const RunBufs& b, int M, int nsteps, 
         return launch_with_companion(h, a, plan, st);
     }
     cudaError_t e = prec == ROM_FP64   ? launch_rank2_simt_f64(a, plan, st)
+                    : plan.variant == 5 ? launch_rank2_cta_f32(a, plan, st)
                     : plan.variant >= 2 ? launch_rank2_split_f32(a, plan, st)
                                         : launch_rank2_simt_f32(a, plan, st);
     if (e != cudaSuccess) return cuda_fail(e, "rank2 launch");
@@ -827,6 +833,7 @@ rom_status rom_autotune(rom_t h, int prec, int M, int probe_steps, double* best_
     } else {
         Rank2Plan p0;
         int nact = 0;
+        if (h->Kp <= 128 && h->comp_cs <= 0 && plan_rank2_cta_f32(h->Kp, M, h->R, &p0)) simt.push_back(p0);
         if (plan_rank2_split_f32(h->Kp, M, h->R, &p0)) nact = p0.max_active_clusters;
         else if (plan_rank2_simt_f32(h->Kp, M, h->R, false, &p0)) nact = p0.max_active_clusters;
         const int budgets[3] = {nact, nact / 2, nact / 4};

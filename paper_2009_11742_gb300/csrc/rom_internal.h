@@ -104,7 +104,7 @@ struct Rank2Plan {
     int max_active_clusters;
     size_t smem;
     bool resident; // operators kept in registers for the whole run
-    int variant;   // 1: one-block, 2: two-block split-role, 3: two-block dataflow
+    int variant;   // 1: one-block, 2: two-block split-role, 3: two-block dataflow, 5: one CTA
     bool c_global; // one-block: the CTA's receiver rows are read from global memory (too many to stage)
     int nrt;       // one-block kernel: 32-row tiles per CTA (2 when Kp > 512)
     // streaming companion (two-block variant only): the last comp_cols
@@ -127,6 +127,9 @@ bool plan_rank2_simt_f64(int Kp, int M, int R, bool rank1, Rank2Plan* plan, int 
 bool plan_rank2_split_f32(int Kp, int M, int R, Rank2Plan* plan, int cluster_budget = 0);
 bool plan_rank2_dataflow_f32(int Kp, int M, int R, Rank2Plan* plan);
 cudaError_t launch_rank2_split_f32(const Rank2Args& a, const Rank2Plan& plan, cudaStream_t st);
+// One-CTA kernel (FP32, Kp <= 128): no cluster, both operators in registers.
+bool plan_rank2_cta_f32(int Kp, int M, int R, Rank2Plan* plan);
+cudaError_t launch_rank2_cta_f32(const Rank2Args& a, const Rank2Plan& plan, cudaStream_t st);
 // The work-list kernel (FP32, any Kp <= 1024, clusters of cs CTAs): the
 // co-resident clusters at `smem` bytes of dynamic shared memory (0: the
 // size does not fit), and the launch of ncl clusters (a.group / items /
