@@ -71,7 +71,8 @@ static bool plan_two_block(int Kp, int M, int R, Rank2Plan* p, int cluster_budge
 }
 
 template <bool DF>
-static cudaError_t launch_two_block(const Rank2Args& a_in, const Rank2Plan& p, cudaStream_t st) {
+static cudaError_t launch_two_block(const Rank2Args& a_in, const Rank2Plan& p, cudaStream_t st,
+                                    cudaEvent_t started = nullptr) {
     Rank2Args a = a_in;
     a.Wv = p.Wv;
     a.Wa = p.Wa;
@@ -85,6 +86,7 @@ static cudaError_t launch_two_block(const Rank2Args& a_in, const Rank2Plan& p, c
     cudaError_t e = prepare_kernel<float>(fn, p.smem);
     if (e != cudaSuccess) return e;
     ClusterLaunch L(p.cs, p.nclusters, kThreads, p.smem, st);
+    if (started) L.record_started(started);
     void* args[] = {(void*)&a};
     return L.launch(fn, args);
 }
@@ -92,8 +94,8 @@ static cudaError_t launch_two_block(const Rank2Args& a_in, const Rank2Plan& p, c
 bool plan_rank2_split_f32(int Kp, int M, int R, Rank2Plan* p, int budget) { return plan_two_block<false>(Kp, M, R, p, budget); }
 
 bool plan_rank2_dataflow_f32(int Kp, int M, int R, Rank2Plan* p) { return plan_two_block<true>(Kp, M, R, p); }
-cudaError_t launch_rank2_split_f32(const Rank2Args& a, const Rank2Plan& p, cudaStream_t st) {
-    return p.variant == 3 ? launch_two_block<true>(a, p, st) : launch_two_block<false>(a, p, st);
+cudaError_t launch_rank2_split_f32(const Rank2Args& a, const Rank2Plan& p, cudaStream_t st, cudaEvent_t started) {
+    return p.variant == 3 ? launch_two_block<true>(a, p, st) : launch_two_block<false>(a, p, st, started);
 }
 
 }  // namespace romk

@@ -14,7 +14,7 @@ namespace romk {
 // so it is neither copied nor moved.
 struct ClusterLaunch {
     cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute attr[1] = {};
+    cudaLaunchAttribute attr[2] = {};
     ClusterLaunch(int cs, int nclusters, int threads, size_t smem, cudaStream_t st = nullptr) {
         attr[0].id = cudaLaunchAttributeClusterDimension;
         attr[0].val.clusterDim.x = cs;
@@ -26,6 +26,13 @@ struct ClusterLaunch {
         cfg.stream = st;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
+    }
+    // Record `ev` once every block of the launch has started.
+    void record_started(cudaEvent_t ev) {
+        attr[1].id = cudaLaunchAttributeLaunchCompletionEvent;
+        attr[1].val.launchCompletionEvent.event = ev;
+        attr[1].val.launchCompletionEvent.flags = 0;
+        cfg.numAttrs = 2;
     }
     ClusterLaunch(const ClusterLaunch&) = delete;
     ClusterLaunch& operator=(const ClusterLaunch&) = delete;

@@ -126,7 +126,9 @@ bool plan_rank2_simt_f64(int Kp, int M, int R, bool rank1, Rank2Plan* plan, int 
 // with per-block mbarriers fed by asynchronous stores (bounded waits).
 bool plan_rank2_split_f32(int Kp, int M, int R, Rank2Plan* plan, int cluster_budget = 0);
 bool plan_rank2_dataflow_f32(int Kp, int M, int R, Rank2Plan* plan);
-cudaError_t launch_rank2_split_f32(const Rank2Args& a, const Rank2Plan& plan, cudaStream_t st);
+// started (variant 2; may be null): an event recorded once every block has started.
+cudaError_t launch_rank2_split_f32(const Rank2Args& a, const Rank2Plan& plan, cudaStream_t st,
+                                   cudaEvent_t started = nullptr);
 // One-CTA kernel (FP32, Kp <= 128): no cluster, both operators in registers.
 bool plan_rank2_cta_f32(int Kp, int M, int R, Rank2Plan* plan);
 cudaError_t launch_rank2_cta_f32(const Rank2Args& a, const Rank2Plan& plan, cudaStream_t st);
