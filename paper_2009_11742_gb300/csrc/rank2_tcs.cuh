@@ -10,18 +10,22 @@
 //     state column j as 2^(eX_j - 7) (x0 + 2^-8 x1 + 2^-16 x2), with integer
 //     digits in [-128, 128] (exact in BF16) and |A| < 2^eA_r over the row,
 //     |X| < 2^eX_j over the whole column (all Kp rows of the cluster);
-//   * the six digit products of weight 1, 2^-8 and 2^-16 go to four TMEM
-//     accumulators: T0 = sum a0 x0 (|T0| <= Kp 2^14 <= 2^24), T1a / T1b =
-//     sum a0 x1 + a1 x0 over k < 512 / k >= 512 (each <= 2^24), and
-//     T2 = sum a0 x2 + a1 x1 + a2 x0.  Products of integers below 2^7 in
-//     magnitude are exact, and every partial sum of T0 and T1 is an integer
-//     of magnitude at most 2^24, so the tensor core computes them exactly;
-//     T2 carries weight 2^-16, so whatever it rounds is below 2^-32 of the
-//     result;
+//   * the six digit products of weight 1, 2^-8 and 2^-16 each have a TMEM
+//     accumulator of their own.  Products of integers of magnitude at most
+//     2^7 are exact, and every partial sum is an integer of magnitude at most
+//     Kp 2^14 <= 2^24, so the tensor core rounds nothing;
+//   * the products that share an operator digit are one MMA: the state digit
+//     tiles lie one after the other in a stage, so a0 [x0 x1 x2] has N = 3 W,
+//     a1 [x0 x1] N = 2 W and a2 [x0] N = W, side by side in TMEM.  Each
+//     operator tile is then read from shared memory once per k step instead
+//     of six reads of three tiles; shared-memory bandwidth bounds the phase;
 //   * the readers load the accumulators once per half-step and form
-//     A.X = 2^(eA_r + eX_j - 14) (T0 + 2^-8 (T1a + T1b) + 2^-16 T2) in FP32
-//     with round-to-nearest; the terms of weight 2^-24 and below that the
-//     digits leave out are not biased either.
+//     A.X = 2^(eA_r + eX_j - 14) (T0 + 2^-8 T1 + 2^-16 T2) in FP32 with
+//     round-to-nearest, T0 = a0 x0, T1 = a0 x1 + a1 x0, T2 = a0 x2 + a1 x1 +
+//     a2 x0; the terms of weight 2^-24 and below that the digits leave out
+//     are not biased either.
+// K = M = 1024 in blocks of 80: 41.1 us a step against 48.8 with six MMAs a k
+// step; in blocks of 32 to 48 27.3 to 31.0 against 39.9 to 43.1.
 // The state's column exponent needs the column maximum over all rows, which
 // the CTAs of a cluster agree on through distributed shared memory with one
 // extra cluster barrier per half-step.  Work split, pipeline and bounded
@@ -77,13 +81,10 @@ __device__ __forceinline__ int bound_exponent(float mx) {
     return e;
 }
 
-// Column stride of the accumulators in tensor memory; after the four
-// accumulators the new state of each readout warp (W columns in all) is
-// parked between the update and the slicing.  Allocation: next power of two.
-__host__ __device__ constexpr int tcs_acc_stride(int W) { return ((W + 31) / 32) * 32; }
-__host__ __device__ constexpr uint32_t tcs_tmem_cols(int W) {
-    return 4 * tcs_acc_stride(W) + W <= 128 ? 128u : (4 * tcs_acc_stride(W) + W <= 256 ? 256u : 512u);
-}
+// Accumulator columns in tensor memory: a0x0, a0x1, a0x2, a1x0, a1x1, a2x0,
+// W columns each.  The new state waits in a0x0's columns between the update,
+// which has read them, and the slicing.
+__host__ __device__ constexpr uint32_t tcs_tmem_cols(int W) { return 6 * W <= 256 ? 256u : 512u; }
 
 __host__ __device__ inline size_t tcs_stage_bytes(int W) {
     return (size_t)kTcsTerms * kATileBytes + (size_t)kTcsTerms * W * kTileRowBytes;
@@ -127,17 +128,15 @@ __device__ __forceinline__ void tmem_ld8_nowait(uint32_t taddr, uint32_t (&r)[8]
                  : "memory");
 }
 // Wait for outstanding tensor-memory loads; the registers pass through the
-// statement so that no use of them is scheduled before the wait.
-__device__ __forceinline__ void tmem_wait_ld4(uint32_t (&a)[8], uint32_t (&b)[8], uint32_t (&c)[8],
-                                              uint32_t (&d)[8]) {
-    asm volatile("tcgen05.wait::ld.sync.aligned;"
-                 : "+r"(a[0]), "+r"(a[1]), "+r"(a[2]), "+r"(a[3]), "+r"(a[4]), "+r"(a[5]), "+r"(a[6]),
-                   "+r"(a[7]), "+r"(b[0]), "+r"(b[1]), "+r"(b[2]), "+r"(b[3]), "+r"(b[4]), "+r"(b[5]),
-                   "+r"(b[6]), "+r"(b[7]), "+r"(c[0]), "+r"(c[1]), "+r"(c[2]), "+r"(c[3]), "+r"(c[4]),
-                   "+r"(c[5]), "+r"(c[6]), "+r"(c[7]), "+r"(d[0]), "+r"(d[1]), "+r"(d[2]), "+r"(d[3]),
-                   "+r"(d[4]), "+r"(d[5]), "+r"(d[6]), "+r"(d[7])
-                 :
-                 : "memory");
+// statements so that no use of them is scheduled before the wait.
+__device__ __forceinline__ void reg_pin8(uint32_t (&a)[8]) {
+    asm volatile("" : "+r"(a[0]), "+r"(a[1]), "+r"(a[2]), "+r"(a[3]), "+r"(a[4]), "+r"(a[5]), "+r"(a[6]), "+r"(a[7])
+                 :: "memory");
+}
+__device__ __forceinline__ void tmem_wait_ld6(uint32_t (&a)[6][8]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int k = 0; k < 6; ++k) reg_pin8(a[k]);
 }
 
 __device__ __forceinline__ void tmem_st8(uint32_t taddr, const float (&v)[8]) {
@@ -159,27 +158,24 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, float (&v)[8]) {
     for (int q = 0; q < 8; ++q) v[q] = __uint_as_float(r[q]);
 }
 
-// The six digit products of one 16-deep k-step, issued from one asm block:
-// d0 += a0 x0, d1 += a0 x1 + a1 x0, d2 += a0 x2 + a1 x1 + a2 x0.  The
-// operands are given as the low words of their SW128 descriptors (the high
-// word, hi, is the same for every tile); acc0 / acc1 = 0 start d0 and d2 /
-// d1 afresh.
-__device__ __forceinline__ void tcs_mma6(uint32_t d0, uint32_t d1, uint32_t d2, uint32_t hi, uint32_t a0,
-                                         uint32_t a1, uint32_t a2, uint32_t x0, uint32_t x1, uint32_t x2,
-                                         uint32_t idesc, uint32_t acc0, uint32_t acc1) {
+// The digit products of one 16-deep k-step as three MMAs: d += a0 [x0 x1 x2],
+// d + 3 W += a1 [x0 x1], d + 5 W += a2 [x0].  No two of them share an
+// accumulator, so their order is free.  The operands are given as the low
+// words of their SW128 descriptors (the high word, hi, is the same for every
+// tile); acc = 0 starts the accumulators afresh.
+template <int W>
+__device__ __forceinline__ void tcs_mma3(uint32_t d, uint32_t hi, uint32_t a0, uint32_t a1, uint32_t a2, uint32_t x,
+                                         uint32_t acc) {
     asm volatile(
-        "{\n\t.reg .pred p0, p1;\n\t.reg .b64 da0, da1, da2, dx0, dx1, dx2;\n\t"
-        "setp.ne.b32 p0, %11, 0;\n\tsetp.ne.b32 p1, %12, 0;\n\t"
-        "mov.b64 da0, {%4, %3};\n\tmov.b64 da1, {%5, %3};\n\tmov.b64 da2, {%6, %3};\n\t"
-        "mov.b64 dx0, {%7, %3};\n\tmov.b64 dx1, {%8, %3};\n\tmov.b64 dx2, {%9, %3};\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], da0, dx0, %10, p0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%1], da0, dx1, %10, p1;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%1], da1, dx0, %10, 1;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%2], da0, dx2, %10, p0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%2], da1, dx1, %10, 1;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%2], da2, dx0, %10, 1;\n\t}"
-        ::"r"(d0), "r"(d1), "r"(d2), "r"(hi), "r"(a0), "r"(a1), "r"(a2), "r"(x0), "r"(x1), "r"(x2),
-          "r"(idesc), "r"(acc0), "r"(acc1)
+        "{\n\t.reg .pred p;\n\t.reg .b64 da0, da1, da2, dx;\n\t"
+        "setp.ne.b32 p, %11, 0;\n\t"
+        "mov.b64 da0, {%4, %3};\n\tmov.b64 da1, {%5, %3};\n\tmov.b64 da2, {%6, %3};\n\tmov.b64 dx, {%7, %3};\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], da0, dx, %8, p;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%1], da1, dx, %9, p;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%2], da2, dx, %10, p;\n\t}"
+        ::"r"(d), "r"(d + 3 * W), "r"(d + 5 * W), "r"(hi), "r"(a0), "r"(a1), "r"(a2), "r"(x),
+          "r"(mma_idesc(kFmtBF16, kTcRows, 3 * W)), "r"(mma_idesc(kFmtBF16, kTcRows, 2 * W)),
+          "r"(mma_idesc(kFmtBF16, kTcRows, W)), "r"(acc)
         : "memory");
 }
 
@@ -237,7 +233,6 @@ __device__ __forceinline__ void reader_bar_sync() {
 template <int W, bool XR>
 __global__ void __launch_bounds__(kTcsThreads, 1) rank2_tcs_kernel(const TcArgs a) {
     constexpr int WH = W / 2;                       // columns per readout warp
-    constexpr int AST = tcs_acc_stride(W);          // accumulator column stride
     constexpr uint32_t NCOLS = tcs_tmem_cols(W);
     static_assert(W % 16 == 0 && W >= 32 && W <= 80 && WH % 8 == 0, "unsupported block width");
     cg::cluster_group cluster = cg::this_cluster();
@@ -253,8 +248,6 @@ __global__ void __launch_bounds__(kTcsThreads, 1) rank2_tcs_kernel(const TcArgs 
     // scratch fits in the stage ring (decided identically on the host)
     const bool chip_tr = a.traces && a.R <= kTcsTraceR &&
                          tcs_trace_scratch_bytes(W) <= (size_t)STAGES * tcs_stage_bytes(W);
-    const int KC_T1B = 512 / kTcsKC;                // first chunk accumulated into T1b
-    const bool two_t1 = Kp > 512;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const float dt = (float)a.dt;
     const long long limit = a.spin_limit;
@@ -353,7 +346,6 @@ __global__ void __launch_bounds__(kTcsThreads, 1) rank2_tcs_kernel(const TcArgs 
     cluster.sync();
     tc_fence_after();
     const uint32_t tbase = *tslot;
-    const uint32_t idesc = mma_idesc(kFmtBF16, kTcRows, (uint32_t)W);
     const uint32_t xtile = (uint32_t)W * kTileRowBytes;
     const uint32_t chunk_bytes = kTcsTerms * kATileBytes + kTcsTerms * xtile;
 
@@ -425,7 +417,7 @@ __global__ void __launch_bounds__(kTcsThreads, 1) rank2_tcs_kernel(const TcArgs 
                     bool ok = true;
                     const uint64_t dring = sw128_desc(cvta_shared(smem));
                     const uint32_t dhi = (uint32_t)(dring >> 32), dlo = (uint32_t)dring;
-                    const uint32_t ta = kATileBytes >> 4, tx = xtile >> 4;
+                    const uint32_t ta = kATileBytes >> 4;
                     const uint32_t tstage = (uint32_t)(stage_bytes >> 4);
                     for (int kc = 0; kc < NKC; ++kc) {
                         const int s = s_mma;
@@ -434,18 +426,11 @@ __global__ void __launch_bounds__(kTcsThreads, 1) rank2_tcs_kernel(const TcArgs 
                         tc_fence_after();
                         const uint32_t la = dlo + (uint32_t)s * tstage;
                         const uint32_t lx = la + kTcsTerms * ta;
-                        const bool t1b = two_t1 && kc >= KC_T1B;
-                        const uint32_t d0 = tbase;
-                        const uint32_t d1 = tbase + (uint32_t)((t1b ? 2 : 1) * AST);
-                        const uint32_t d2 = tbase + (uint32_t)(3 * AST);
-                        const bool first0 = kc == 0;
-                        const bool first1 = kc == (t1b ? KC_T1B : 0);
 #pragma unroll
                         for (int ks = 0; ks < 4; ++ks) {  // four 16-deep K steps per 128-byte chunk
                             const uint32_t o = 2u * ks;     // 32 bytes
-                            tcs_mma6(d0, d1, d2, dhi, la + o, la + ta + o, la + 2 * ta + o, lx + o, lx + tx + o,
-                                     lx + 2 * tx + o, idesc, (first0 && ks == 0) ? 0u : 1u,
-                                     (first1 && ks == 0) ? 0u : 1u);
+                            tcs_mma3<W>(tbase, dhi, la + o, la + ta + o, la + 2 * ta + o, lx + o,
+                                        kc == 0 && ks == 0 ? 0u : 1u);
                         }
                         mma_commit(&empty[s]);
                         ++it_mma;
@@ -456,11 +441,11 @@ __global__ void __launch_bounds__(kTcsThreads, 1) rank2_tcs_kernel(const TcArgs 
                 __syncwarp();
             }
             {
-                // ---- readers: one readout of the four accumulators, the fused
+                // ---- readers: one readout of the accumulators, the fused
                 //      forcing and Kahan update, the column maxima of the new
                 //      state.  The old rows and carries are loaded two 8-column
                 //      groups ahead (the first two while the MMAs run); the new
-                //      rows wait in spare tensor-memory columns for the slicing.
+                //      rows wait in the columns of a0 x0 for the slicing.
                 int gotl = 0;
                 if (lane == 0) gotl = (*abort_flag == 0) && mbarrier_wait(dready, (uint32_t)(hs & 1), limit, abort_flag);
                 have = __shfl_sync(0xffffffffu, gotl, 0) != 0;
@@ -471,32 +456,34 @@ __global__ void __launch_bounds__(kTcsThreads, 1) rank2_tcs_kernel(const TcArgs 
                 const uint32_t tl = tbase + ((uint32_t)(32 * quad) << 16) + (uint32_t)jbase;
                 // one 8-column group: readout, update, new state parked in TMEM,
                 // loads of the group two ahead into the same buffers
-                // accumulator registers of one group, double-buffered: the next
-                // group's loads are issued before the current group's update
-                struct Acc8 { uint32_t r0[8], r1a[8], r1b[8], r2[8]; };
-                auto acc_issue = [&](const int g, Acc8& t) {
+                // accumulators of one group: the next group's loads are issued
+                // before the current group's update and summed by weight (T0,
+                // T1, T2) when they have arrived
+                struct Acc8 { float t[3][8]; };
+                uint32_t raw[6][8];
+                auto acc_issue = [&](const int g) {
                     if (!have) return;
-                    const int i0 = 8 * g;
-                    tmem_ld8_nowait(tl + (uint32_t)i0, t.r0);
-                    tmem_ld8_nowait(tl + (uint32_t)(AST + i0), t.r1a);
-                    if (two_t1) tmem_ld8_nowait(tl + (uint32_t)(2 * AST + i0), t.r1b);
-                    tmem_ld8_nowait(tl + (uint32_t)(3 * AST + i0), t.r2);
+#pragma unroll
+                    for (int k = 0; k < 6; ++k) tmem_ld8_nowait(tl + (uint32_t)(k * W + 8 * g), raw[k]);
                 };
                 auto acc_wait = [&](Acc8& t) {
 #pragma unroll
+                    for (int k = 0; k < 6; ++k)
+#pragma unroll
+                        for (int q = 0; q < 8; ++q)
+                            if (!have) raw[k][q] = 0u;
+                    if (have) tmem_wait_ld6(raw);
+#pragma unroll
                     for (int q = 0; q < 8; ++q) {
-                        if (!have) { t.r0[q] = 0u; t.r1a[q] = 0u; t.r2[q] = 0u; }
-                        if (!have || !two_t1) t.r1b[q] = 0u;
+                        t.t[0][q] = __uint_as_float(raw[0][q]);
+                        t.t[1][q] = __fadd_rn(__uint_as_float(raw[1][q]), __uint_as_float(raw[3][q]));
+                        t.t[2][q] = __fadd_rn(__fadd_rn(__uint_as_float(raw[2][q]), __uint_as_float(raw[4][q])),
+                                              __uint_as_float(raw[5][q]));
                     }
-                    if (have) tmem_wait_ld4(t.r0, t.r1a, t.r1b, t.r2);
                 };
                 auto group = [&](const int g, Acc8& cur, Acc8& nxt, float (&yg)[8], float (&cg_)[8]) {
                     const int i0 = 8 * g;
-                    if (g + 1 < NG) acc_issue(g + 1, nxt);
-                    const uint32_t(&r0)[8] = cur.r0;
-                    const uint32_t(&r1a)[8] = cur.r1a;
-                    const uint32_t(&r1b)[8] = cur.r1b;
-                    const uint32_t(&r2)[8] = cur.r2;
+                    if (g + 1 < NG) acc_issue(g + 1);
                     float ynew[8], scl[8], fq[8];
                     unsigned ybits[8];
 #pragma unroll
@@ -508,9 +495,8 @@ __global__ void __launch_bounds__(kTcsThreads, 1) rank2_tcs_kernel(const TcArgs 
                     // selected afterwards), so that their dependency chains interleave
 #pragma unroll
                     for (int q = 0; q < 8; ++q) {
-                        const float t1 = __fadd_rn(__uint_as_float(r1a[q]), __uint_as_float(r1b[q]));
-                        const float u = __fmaf_rn(__uint_as_float(r2[q]), 1.f / 65536.f, t1 * (1.f / 256.f));
-                        const float R = __fadd_rn(__uint_as_float(r0[q]), u);
+                        const float u = __fmaf_rn(cur.t[2][q], 1.f / 65536.f, cur.t[1][q] * (1.f / 256.f));
+                        const float R = __fadd_rn(cur.t[0][q], u);
                         float inc = R * scl[q];
                         inc = half == 0 ? __fmaf_rn(grw, fq[q], inc) : inc;
                         if (XR && Xref) inc = inc + xst[(size_t)(i0 + q) * kTcsThreads + ridx];
@@ -537,13 +523,13 @@ __global__ void __launch_bounds__(kTcsThreads, 1) rank2_tcs_kernel(const TcArgs 
                         const unsigned m = colmax8(ybits, lane, cq);
                         if ((lane & 3) == 0) colmax[quad * W + jbase + i0 + cq] = m;
                     }
-                    tmem_st8(tl + (uint32_t)(4 * AST + i0), ynew);
+                    tmem_st8(tl + (uint32_t)i0, ynew);
                     if (g + 2 < NG)
                         load_group8(Y, Cy, Kown, col0 + jbase + i0 + 16, ncol - jbase - i0 - 16, rowok, yg, cg_);
                     if (g + 1 < NG) acc_wait(nxt);
                 };
                 Acc8 accA, accB;
-                acc_issue(0, accA);
+                acc_issue(0);
                 acc_wait(accA);
 #pragma unroll 1
                 for (int g = 0; g < NG; g += 2) {
@@ -629,7 +615,7 @@ __global__ void __launch_bounds__(kTcsThreads, 1) rank2_tcs_kernel(const TcArgs 
             }
             {
                 unsigned char* Xdst = half ? Xblk0 : Xblk1;  // V feeds the S half and vice versa
-                const uint32_t ts = tbase + ((uint32_t)(32 * quad) << 16) + (uint32_t)(4 * AST + chalf * WH);
+                const uint32_t ts = tbase + ((uint32_t)(32 * quad) << 16) + (uint32_t)(chalf * WH);
                 tc_fence_after();
 #pragma unroll 1
                 for (int i0 = 0; i0 < WH; i0 += 8) {
