@@ -127,8 +127,10 @@ rom_status rom_get_dims(rom_t h, int* Kv, int* Ks, int* R, double* dt);
 
 /* Kernel selection for the rank-2 FP32 path (the FP64 path always uses the
  * one-block kernel):
- *  ROM_KERNEL_AUTO      planner's choice (default: two-block above Kp = 128,
- *                       one CTA per column block, without clusters, up to it);
+ *  ROM_KERNEL_AUTO      planner's choice (default: up to Kp = 128 one CTA per
+ *                       column block, without clusters; above, one-block with
+ *                       asynchronous exchange for up to 12 columns per
+ *                       cluster, else two-block);
  *  ROM_KERNEL_ONE_BLOCK one column block per cluster, every CTA owns 32 rows
  *                       of both V and S;
  *  ROM_KERNEL_TWO_BLOCK two column blocks per cluster half a step apart,
@@ -144,7 +146,7 @@ enum { ROM_KERNEL_AUTO = 0, ROM_KERNEL_ONE_BLOCK = 1, ROM_KERNEL_TWO_BLOCK = 2,
 rom_status rom_set_kernel(rom_t h, int kernel);
 
 /* The launch plan the handle would use for M realizations at precision prec
- * (ROM_FP32 or ROM_FP64): kernel variant (1 one-block, 2 two-block, 3
+ * (ROM_FP32 or ROM_FP64): kernel variant (1 one-block in either form, 2 two-block, 3
  * dataflow, 4 two-block with the streaming companion of rom_set_companion on
  * the last columns, 5 one CTA per column block), cluster size, columns per column block and number of
  * clusters of the main kernel (outputs may be NULL).  ROM_E_UNSUPPORTED for
@@ -250,8 +252,9 @@ rom_status rom_set_tc_columns(rom_t h, int cols);
 
 /*
  * rom_set_wait_limit -- bound, in SM clock cycles, on every device-side wait
- * of the dataflow kernel (a consumer waiting for a producer's rows) and of
- * the tensor-core kernels (stage and accumulator handshakes).  A wait that
+ * of the kernels with asynchronous exchange (a consumer waiting for a
+ * producer's rows: dataflow, and one-block in its asynchronous form) and of the
+ * tensor-core kernels (stage and accumulator handshakes).  A wait that
  * runs out makes the kernel stop, leave cleanly, and record ROM_E_TIMEOUT in
  * the handle's status word (rom_sync_status).  Default
  * 4e9 cycles (about 2 s), far above any legitimate wait.
@@ -260,7 +263,8 @@ rom_status rom_set_wait_limit(rom_t h, long long cycles);
 
 /*
  * rom_debug_inject_stall -- failure injection for tests of the timeout path:
- * when on, one CTA of every cluster of ROM_KERNEL_DATAFLOW never publishes
+ * when on, one CTA of every cluster of a kernel with asynchronous exchange
+ * (ROM_KERNEL_DATAFLOW, one-block in its asynchronous form) never publishes
  * its rows, so its peers' waits run out (set a small wait limit first).  The
  * kernel then ends with ROM_E_TIMEOUT instead of hanging.  Off by default.
  */

@@ -1,0 +1,122 @@
+// Host planning / launch of the one-block kernel with asynchronous exchange
+// (FP32, Kp <= 512; FP64, Kp <= 256).
+#include <cuda_runtime.h>
+
+#include "rank2_async.cuh"
+#include "rank2_launch.cuh"
+
+namespace romk {
+
+template <typename T, int KI>
+static void* async_kernel_for(int cb) {
+    return cb == 1   ? (void*)&rank2_async_kernel<T, KI, 1>
+           : cb == 2 ? (void*)&rank2_async_kernel<T, KI, 2>
+                     : (void*)&rank2_async_kernel<T, KI, 4>;
+}
+template <typename T>
+static void* async_kernel(int KI, int cb) {
+    switch (KI) {
+        case 1: return async_kernel_for<T, 1>(cb);
+        case 2: return async_kernel_for<T, 2>(cb);
+        case 3: return async_kernel_for<T, 3>(cb);
+        case 4: return async_kernel_for<T, 4>(cb);
+        default: break;
+    }
+    if constexpr (sizeof(T) == 4) {
+        switch (KI) {
+            case 5: return async_kernel_for<T, 5>(cb);
+            case 6: return async_kernel_for<T, 6>(cb);
+            case 7: return async_kernel_for<T, 7>(cb);
+            case 8: return async_kernel_for<T, 8>(cb);
+            default: break;
+        }
+    }
+    return nullptr;
+}
+
+// The column group for w columns.  FP64 is bound by the FP64 units, so no
+// column that is not there is computed unless the wider group's cheaper
+// reduction and epilogue make up for it; FP32 takes the widest group in use.
+static int async_group(int w, bool f64) {
+    if (!f64) return w >= 3 ? 4 : w;
+    int best = 1;
+    double t = 1e30;
+    for (int cb : {4, 2, 1}) {
+        const double x = (w + cb - 1) / cb * cb * (cb == 4 ? 1.0 : cb == 2 ? 1.06 : 1.2);
+        if (x < t) {
+            t = x;
+            best = cb;
+        }
+    }
+    return best;
+}
+
+template <typename T>
+static bool plan_async(int Kp, int M, int R, Rank2Plan* p) {
+    if (Kp <= 0 || Kp % 64 != 0 || Kp > (sizeof(T) == 4 ? 512 : 256) || M <= 0) return false;
+    p->KI = Kp / 64;
+    p->cs = Kp / kRowsPerCta;
+    p->nrt = 1;
+    p->resident = true;
+    p->variant = 1;
+    p->async = true;
+    const int rpc = (R + p->cs - 1) / p->cs;
+    p->c_global = (size_t)rpc * Kp * sizeof(T) > 64 * 1024;
+    const int nC = p->c_global ? 0 : rpc;
+    int dev = 0, nsm = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    const size_t smax = (size_t)device_smem_optin();
+    auto bytes = [&](int w, int cb) { return async_smem_layout<T>(w, w / cb, Kp, nC).total; };
+    // one CTA per SM: the clusters that fit are those of the widest block
+    void* probe_fn = async_kernel<T>(p->KI, 4);
+    const size_t probe_smem = bytes(4, 4) > smax / 2 + 1024 ? bytes(4, 4) : smax / 2 + 1024;
+    if (probe_smem > smax || prepare_kernel<T>(probe_fn, probe_smem) != cudaSuccess) return false;
+    ClusterLaunch probe(p->cs, 1, kThreads, probe_smem);
+    p->max_active_clusters = probe.max_active(probe_fn);
+    if (p->max_active_clusters <= 0) return false;
+    int w = (M + p->max_active_clusters - 1) / p->max_active_clusters;
+    p->cb = async_group(w, sizeof(T) == 8);
+    w = (w + p->cb - 1) / p->cb * p->cb;
+    while (w > p->cb && bytes(w, p->cb) > smax) w -= p->cb;
+    p->Wv = p->Wa = w;
+    p->nclusters = (M + w - 1) / w;
+    p->smem = bytes(w, p->cb);
+    return p->smem <= smax;
+}
+
+template <typename T>
+static cudaError_t launch_async(const Rank2Args& a_in, const Rank2Plan& p, cudaStream_t st) {
+    Rank2Args a = a_in;
+    a.Wv = p.Wv;
+    a.Wa = p.Wa;
+    a.rpc = (a.R + p.cs - 1) / p.cs;
+    a.c_global = p.c_global ? 1 : 0;
+    void* fn = async_kernel<T>(p.KI, p.cb);
+    if (!fn || a.group) return cudaErrorInvalidValue;
+    cudaError_t e = prepare_kernel<T>(fn, p.smem);
+    if (e != cudaSuccess) return e;
+    ClusterLaunch L(p.cs, p.nclusters, kThreads, p.smem, st);
+    void* args[] = {(void*)&a};
+    return L.launch(fn, args);
+}
+
+bool plan_rank2_async(int Kp, int M, int R, bool f64, Rank2Plan* p) {
+    return f64 ? plan_async<double>(Kp, M, R, p) : plan_async<float>(Kp, M, R, p);
+}
+
+// us a step, this kernel / two-block kernel, at W columns per cluster (the
+// two-block kernel with the same M: two blocks of 4 or 8):
+//     K = 192: W = 2 1.01 / 2.54, 4 1.30 / 2.54, 8 2.12 / 2.54, 12 3.07 / 3.59
+//     K = 256: W = 2 1.19 / 2.69, 4 1.53 / 2.71, 8 2.36 / 2.71, 12 3.42 / 3.98
+//     K = 384: W = 2 1.40 / 3.21, 4 1.97 / 3.24, 8 3.05 / 3.24, 12 4.42 / 4.81
+//     K = 512: W = 2 1.92 / 4.01, 4 2.37 / 4.02, 8 3.84 / 4.03, 12 5.45 / 5.82,
+//              20 8.96 / 7.84
+// Above that the two-block kernel's 4 rows a thread (half the operand reads
+// per product) win over the shorter exchange.
+bool async_beats_two_block(int W) { return W <= 12; }
+cudaError_t launch_rank2_async(const Rank2Args& a, const Rank2Plan& p, bool f64, cudaStream_t st) {
+    return f64 ? launch_async<double>(a, p, st) : launch_async<float>(a, p, st);
+}
+
+}  // namespace romk

@@ -44,6 +44,7 @@
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
+#include "cluster_mbar.cuh"
 #include "dev_common.cuh"
 #include "rank2_simt.cuh"
 #include "rank2_split.cuh"
@@ -74,59 +75,6 @@ __host__ __device__ inline DataflowSmem dataflow_smem_layout(int Wa, int Kp, int
     s.sent = o; o += align16((size_t)(kDataflowMaxH * 2 + 4) * sizeof(unsigned));
     s.total = o;
     return s;
-}
-
-// ---- mbarrier / cluster primitives (PTX, sm_90+ semantics)
-__device__ __forceinline__ unsigned smem_addr(const void* p) {
-    return (unsigned)__cvta_generic_to_shared(p);
-}
-__device__ __forceinline__ void mbar_init(unsigned long long* bar, unsigned count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(bar)), "r"(count)
-                 : "memory");
-}
-__device__ __forceinline__ void fence_mbar_init_cluster() {
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-}
-// Arrive on a local mbarrier and add `bytes` to the transaction count its
-// current phase waits for.
-__device__ __forceinline__ void mbar_arrive_expect_tx(unsigned long long* bar, unsigned bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;"
-                 ::"r"(smem_addr(bar)), "r"(bytes)
-                 : "memory");
-}
-// Count `bytes` as arrived on the current phase of a local mbarrier without
-// an asynchronous copy (used to retire bytes a producer will never send).
-__device__ __forceinline__ void mbar_complete_tx(unsigned long long* bar, unsigned bytes) {
-    asm volatile("mbarrier.complete_tx.relaxed.cta.shared::cta.b64 [%0], %1;"
-                 ::"r"(smem_addr(bar)), "r"(bytes)
-                 : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait(unsigned long long* bar, unsigned parity) {
-    unsigned ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(smem_addr(bar)), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-
-// Bounded wait: returns false (and raises the CTA's abort flag) if the phase
-// did not complete within `limit` clock cycles or another warp aborted.
-__device__ __forceinline__ bool mbar_wait_bounded(unsigned long long* bar, unsigned parity,
-                                                  long long limit, volatile int* abort_flag) {
-    if (mbar_try_wait(bar, parity)) return true;
-    const long long t0 = clock64();
-    while (true) {
-        if (mbar_try_wait(bar, parity)) return true;
-        if (*abort_flag) return false;
-        if (clock64() - t0 > limit) {
-            *abort_flag = 1;
-            return false;
-        }
-    }
 }
 
 template <int KI>

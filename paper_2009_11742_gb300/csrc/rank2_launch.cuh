@@ -63,12 +63,13 @@ struct Rank2Kernel {
 // half-step beyond that.
 // FP32 beyond KI = 8 (K > 512) streams two 32-row operator tiles per CTA per
 // half-step (one-block kernel with nrt = 2; in 8-column groups with the 4-row
-// half-step); FP64 stops at K = 512.
+// half-step); FP64 stops at K = 512.  FP32 one-column groups (rank-1 runs)
+// exist above K = 512 only: below, the asynchronous kernel runs them.
 template <typename T, int CB>
 static void* rank2_kernel_for(int KI, bool* resident) {
     constexpr bool f64 = sizeof(T) == 8;
     *resident = !(f64 && KI > 4) && KI <= 8;
-    switch (KI) {
+    if constexpr (f64 || CB > 1) switch (KI) {
         case 1: return Rank2Kernel<T, 1, CB, true>::fn();
         case 2: return Rank2Kernel<T, 2, CB, true>::fn();
         case 3: return Rank2Kernel<T, 3, CB, true>::fn();

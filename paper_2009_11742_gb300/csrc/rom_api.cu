@@ -393,6 +393,18 @@ rom_status get_plan(rom_s* h, int prec, int M, bool rank1, Rank2Plan* plan) {
     // bits (see rank2_cta.cuh for both sides' times).
     if (prec != ROM_FP64 && h->Kp <= 128 && h->kernel_choice == ROM_KERNEL_AUTO && h->comp_cs <= 0)
         ok = plan_rank2_cta_f32(h->Kp, M, h->R, plan);
+    // The asynchronous one-block kernel: FP64 and rank-1 runs whose operators
+    // stay in registers, and FP32 blocks of few columns unless the caller
+    // pinned a kernel or a companion (the same bits as the two-block kernel).
+    const bool one_block_only = prec == ROM_FP64 || rank1;
+    const bool async_open = prec == ROM_FP64 || h->kernel_choice == ROM_KERNEL_AUTO ||
+                            (rank1 && h->kernel_choice == ROM_KERNEL_ONE_BLOCK);
+    if (!ok && async_open && (one_block_only || h->comp_cs <= 0)) {
+        Rank2Plan pa{};
+        ok = plan_rank2_async(h->Kp, M, h->R, prec == ROM_FP64, &pa) &&
+             (one_block_only || async_beats_two_block(pa.Wa));
+        if (ok) *plan = pa;
+    }
     if (!ok && two_block && h->kernel_choice == ROM_KERNEL_DATAFLOW) {
         ok = plan_rank2_dataflow_f32(h->Kp, M, h->R, plan);
     } else if (!ok && two_block) {
@@ -605,7 +617,8 @@ rom_status launch_simt_with_plan(rom_s* h, const RunBufs& b, int M, int nsteps, 
         }
         return launch_with_companion(h, a, plan, st);
     }
-    cudaError_t e = prec == ROM_FP64   ? launch_rank2_simt_f64(a, plan, st)
+    cudaError_t e = plan.async           ? launch_rank2_async(a, plan, prec == ROM_FP64, st)
+                    : prec == ROM_FP64  ? launch_rank2_simt_f64(a, plan, st)
                     : plan.variant == 5 ? launch_rank2_cta_f32(a, plan, st)
                     : plan.variant >= 2 ? launch_rank2_split_f32(a, plan, st)
                                         : launch_rank2_simt_f32(a, plan, st);
@@ -838,11 +851,13 @@ rom_status rom_autotune(rom_t h, int prec, int M, int probe_steps, double* best_
         }
     } else if (f64) {
         Rank2Plan p;
-        if (plan_rank2_simt_f64(h->Kp, M, h->R, false, &p)) { p.variant = 1; simt.push_back(p); }
+        if (plan_rank2_async(h->Kp, M, h->R, true, &p)) simt.push_back(p);
+        else if (plan_rank2_simt_f64(h->Kp, M, h->R, false, &p)) { p.variant = 1; simt.push_back(p); }
     } else {
         Rank2Plan p0;
         int nact = 0;
         if (h->Kp <= 128 && h->comp_cs <= 0 && plan_rank2_cta_f32(h->Kp, M, h->R, &p0)) simt.push_back(p0);
+        if (h->Kp > 128 && h->comp_cs <= 0 && plan_rank2_async(h->Kp, M, h->R, false, &p0)) simt.push_back(p0);
         if (plan_rank2_split_f32(h->Kp, M, h->R, &p0)) nact = p0.max_active_clusters;
         else if (plan_rank2_simt_f32(h->Kp, M, h->R, false, &p0)) nact = p0.max_active_clusters;
         const int budgets[3] = {nact, nact / 2, nact / 4};

@@ -105,6 +105,7 @@ struct Rank2Plan {
     size_t smem;
     bool resident; // operators kept in registers for the whole run
     int variant;   // 1: one-block, 2: two-block split-role, 3: two-block dataflow, 5: one CTA
+    bool async = false;  // one-block: the form with asynchronous exchange (rank2_async.cuh)
     bool c_global; // one-block: the CTA's receiver rows are read from global memory (too many to stage)
     int nrt;       // one-block kernel: 32-row tiles per CTA (2 when Kp > 512)
     // streaming companion (two-block variant only): the last comp_cols
@@ -132,6 +133,11 @@ cudaError_t launch_rank2_split_f32(const Rank2Args& a, const Rank2Plan& plan, cu
 // One-CTA kernel (FP32, Kp <= 128): no cluster, both operators in registers.
 bool plan_rank2_cta_f32(int Kp, int M, int R, Rank2Plan* plan);
 cudaError_t launch_rank2_cta_f32(const Rank2Args& a, const Rank2Plan& plan, cudaStream_t st);
+// One-block kernel with asynchronous exchange (FP32 Kp <= 512, FP64 Kp <= 256).
+bool plan_rank2_async(int Kp, int M, int R, bool f64, Rank2Plan* plan);
+// FP32: faster than the two-block kernel for W columns per cluster?
+bool async_beats_two_block(int W);
+cudaError_t launch_rank2_async(const Rank2Args& a, const Rank2Plan& plan, bool f64, cudaStream_t st);
 // The work-list kernel (FP32, any Kp <= 1024, clusters of cs CTAs): the
 // co-resident clusters at `smem` bytes of dynamic shared memory (0: the
 // size does not fit), and the launch of ncl clusters (a.group / items /
