@@ -129,16 +129,15 @@ rom_status rom_get_dims(rom_t h, int* Kv, int* Ks, int* R, double* dt);
  * one-block kernel):
  *  ROM_KERNEL_AUTO      planner's choice (default: up to Kp = 128 one CTA per
  *                       column block, without clusters; above, one-block with
- *                       asynchronous exchange for up to 12 columns per
+ *                       asynchronous exchange for up to 4 columns per
  *                       cluster, else two-block);
  *  ROM_KERNEL_ONE_BLOCK one column block per cluster, every CTA owns 32 rows
  *                       of both V and S;
- *  ROM_KERNEL_TWO_BLOCK two column blocks per cluster half a step apart,
- *                       velocity rows and stress rows on different CTAs, one
- *                       cluster barrier per half-step phase;
- *  ROM_KERNEL_DATAFLOW  the two-block schedule synchronised by per-block
- *                       mbarriers fed with asynchronous remote stores; its
- *                       waits are bounded (rom_set_wait_limit).
+ *  ROM_KERNEL_TWO_BLOCK two column blocks per cluster, velocity rows and
+ *                       stress rows on different CTAs, exchanged by
+ *                       asynchronous remote stores that feed an mbarrier per
+ *                       4 columns; its waits are bounded (rom_set_wait_limit);
+ *  ROM_KERNEL_DATAFLOW  the same kernel, without the streaming companion.
  * All compute the same leapfrog (Sec. 3.1); their results agree to FP32
  * rounding. */
 enum { ROM_KERNEL_AUTO = 0, ROM_KERNEL_ONE_BLOCK = 1, ROM_KERNEL_TWO_BLOCK = 2,
@@ -253,7 +252,8 @@ rom_status rom_set_tc_columns(rom_t h, int cols);
 /*
  * rom_set_wait_limit -- bound, in SM clock cycles, on every device-side wait
  * of the kernels with asynchronous exchange (a consumer waiting for a
- * producer's rows: dataflow, and one-block in its asynchronous form) and of the
+ * producer's rows: two-block, its companion, and one-block in its asynchronous
+ * form) and of the
  * tensor-core kernels (stage and accumulator handshakes).  A wait that
  * runs out makes the kernel stop, leave cleanly, and record ROM_E_TIMEOUT in
  * the handle's status word (rom_sync_status).  Default
@@ -264,7 +264,7 @@ rom_status rom_set_wait_limit(rom_t h, long long cycles);
 /*
  * rom_debug_inject_stall -- failure injection for tests of the timeout path:
  * when on, one CTA of every cluster of a kernel with asynchronous exchange
- * (ROM_KERNEL_DATAFLOW, one-block in its asynchronous form) never publishes
+ * (two-block, one-block in its asynchronous form) never publishes
  * its rows, so its peers' waits run out (set a small wait limit first).  The
  * kernel then ends with ROM_E_TIMEOUT instead of hanging.  Off by default.
  */

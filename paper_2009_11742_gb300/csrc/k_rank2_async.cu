@@ -106,15 +106,14 @@ bool plan_rank2_async(int Kp, int M, int R, bool f64, Rank2Plan* p) {
 }
 
 // us a step, this kernel / two-block kernel, at W columns per cluster (the
-// two-block kernel with the same M: two blocks of 4 or 8):
-//     K = 192: W = 2 1.01 / 2.54, 4 1.30 / 2.54, 8 2.12 / 2.54, 12 3.07 / 3.59
-//     K = 256: W = 2 1.19 / 2.69, 4 1.53 / 2.71, 8 2.36 / 2.71, 12 3.42 / 3.98
-//     K = 384: W = 2 1.40 / 3.21, 4 1.97 / 3.24, 8 3.05 / 3.24, 12 4.42 / 4.81
-//     K = 512: W = 2 1.92 / 4.01, 4 2.37 / 4.02, 8 3.84 / 4.03, 12 5.45 / 5.82,
-//              20 8.96 / 7.84
-// Above that the two-block kernel's 4 rows a thread (half the operand reads
-// per product) win over the shorter exchange.
-bool async_beats_two_block(int W) { return W <= 12; }
+// two-block kernel with the same M: two blocks of 4):
+//     K = 192: W = 4 1.21 / 1.39, 8 1.96 / 1.40
+//     K = 256: W = 4 1.43 / 1.59, 8 2.21 / 1.66
+//     K = 384: W = 4 1.77 / 2.12, 8 2.96 / 2.13
+//     K = 512: W = 2 1.72 / 2.59, 4 2.29 / 2.60, 8 3.71 / 2.61
+// Above 4 the two-block kernel's 4 rows a thread (half the operand reads per
+// product) win over the shorter chain of a half-step.
+bool async_beats_two_block(int W) { return W <= 4; }
 cudaError_t launch_rank2_async(const Rank2Args& a, const Rank2Plan& p, bool f64, cudaStream_t st) {
     return f64 ? launch_async<double>(a, p, st) : launch_async<float>(a, p, st);
 }

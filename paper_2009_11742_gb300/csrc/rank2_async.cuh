@@ -79,43 +79,6 @@ __host__ __device__ inline AsyncSmem async_smem_layout(int W, int G, int Kp, int
     return s;
 }
 
-__device__ __forceinline__ unsigned cluster_addr(unsigned a, int rank) {
-    unsigned r;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
-    return r;
-}
-
-// Shared-memory layout of a group's CB columns of V or S: the four rows of a
-// row quad kq of all columns together, as U 16-byte units (FP32: one per
-// column; FP64: two), so that a warp's four rows are one contiguous piece,
-// whose stores to one peer travel together (up to 64 bytes a packet; of
-// single 16-byte stores a CTA of a 16-CTA cluster takes one in 2.5 cycles or
-// more, which at four columns was most of the half-step).  Unit u stands at
-// place u ^ swz(kq), which keeps reads of one unit over consecutive quads free
-// of bank conflicts.
-template <typename T, int CB>
-struct AsyncLayout {
-    static constexpr int U = CB * (int)sizeof(T) / 4;
-    static __device__ __forceinline__ int swz(int kq) { return U > 1 ? (kq / (8 / U)) & (U - 1) : 0; }
-    // element (row k, column c of the group)
-    static __device__ __forceinline__ int at(int c, int k) {
-        const int kq = k >> 2;
-        if (sizeof(T) == 4) return (kq * U + (c ^ swz(kq))) * 4 + (k & 3);
-        return (kq * U + ((2 * c + ((k >> 1) & 1)) ^ swz(kq))) * 2 + (k & 1);
-    }
-    // rows 4 kq .. 4 kq + 3 of column c
-    static __device__ __forceinline__ void load(const T* X, int c, int kq, T (&x)[4]) {
-        const int z = swz(kq);
-        if constexpr (sizeof(T) == 4) {
-            load4(X + (kq * U + (c ^ z)) * 4, x);
-        } else {
-            const double2 p = *reinterpret_cast<const double2*>(X + (kq * U + ((2 * c) ^ z)) * 2);
-            const double2 q = *reinterpret_cast<const double2*>(X + (kq * U + ((2 * c + 1) ^ z)) * 2);
-            x[0] = p.x; x[1] = p.y; x[2] = q.x; x[3] = q.y;
-        }
-    }
-};
-
 // The lane offset (bits 2 and 1) that holds column cc of a group after the
 // reduce-scatter of 2 CB values; row r of the warp's four is at 8 r + offset.
 template <int CB>
@@ -208,34 +171,7 @@ __device__ __forceinline__ void async_traces(const T* C, const T* X, int Kp, int
     using Lay = AsyncLayout<T, CB>;
     if constexpr (sizeof(T) == 4 && CB == 4) {
         if (nj * nc > kThreads / 32) {
-            for (int j0 = 4 * warp; j0 < nj; j0 += 4 * (kThreads / 32)) {
-                float acc[16];
-#pragma unroll
-                for (int i = 0; i < 16; ++i) acc[i] = 0.f;
-#pragma unroll 1
-                for (int k = 4 * lane; k < Kp; k += 128) {
-                    float cv[4][4], xv[4][4];
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        load4(C + (size_t)min(j0 + u, nj - 1) * Kp + k, cv[u]);
-                        Lay::load(X, u, k >> 2, xv[u]);
-                    }
-#pragma unroll
-                    for (int u = 0; u < 4; ++u)
-#pragma unroll
-                        for (int w = 0; w < 4; ++w)
-#pragma unroll
-                            for (int q = 0; q < 4; ++q)
-                                acc[4 * u + w] = __fmaf_rn(cv[u][q], xv[w][q], acc[4 * u + w]);
-                }
-                rs32_stage<8>(acc, lane, 16);
-                rs32_stage<4>(acc, lane, 8);
-                rs32_stage<2>(acc, lane, 4);
-                rs32_stage<1>(acc, lane, 2);
-                acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], 1);
-                const int e = lane >> 1, jj = j0 + (e >> 2), c = e & 3;
-                if ((lane & 1) == 0 && jj < nj && c < nc) out[(size_t)c * R + jj] = acc[0];
-            }
+            for (int j0 = 4 * warp; j0 < nj; j0 += 4 * (kThreads / 32)) trace_tile(C, X, Kp, j0, nj, nc, lane, out, R);
             return;
         }
     }
@@ -451,7 +387,7 @@ __global__ void __launch_bounds__(kThreads, 1) rank2_async_kernel(const Rank2Arg
     if (!dead && nS == N)
         for (int g = 0; g < G && !dead; ++g) dead = !wait(G + g, (unsigned)((N - 1) & 1));
     if (dead && lane == 0) *abort_flag = 1;
-    // ---- drain (see the dataflow kernel): every CTA tells every other how many
+    // ---- drain (see the split kernel): every CTA tells every other how many
     // bytes it sent per mbarrier, and each retires on the phase armed last those
     // that will not come; after a complete run nothing is outstanding.
     if (lane == 0 && npeer > 0) {

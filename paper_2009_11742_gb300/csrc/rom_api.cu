@@ -406,7 +406,8 @@ rom_status get_plan(rom_s* h, int prec, int M, bool rank1, Rank2Plan* plan) {
         if (ok) *plan = pa;
     }
     if (!ok && two_block && h->kernel_choice == ROM_KERNEL_DATAFLOW) {
-        ok = plan_rank2_dataflow_f32(h->Kp, M, h->R, plan);
+        ok = plan_rank2_split_f32(h->Kp, M, h->R, plan);
+        plan->variant = 3;
     } else if (!ok && two_block) {
         ok = plan_rank2_split_f32(h->Kp, M, h->R, plan);
         // the streaming companion on the SMs the split kernel's clusters

@@ -91,7 +91,7 @@ struct Rank2Args {
 // registers), and a kernel that streams its operators from L2 with nrt
 // 32-row tiles per CTA and W columns (one-block kernel above Kp = 512, the
 // work-list kernel).
-inline double model_split_us(int Kp, int W) { return 2.24 + 0.466 * W * (Kp / 512.0); }
+inline double model_split_us(int Kp, int W) { return 0.3 + W * (0.15 + 0.00066 * Kp); }
 inline double model_streamed_us(int Kp, int nrt, int W) { return 3.5 + 0.71 * nrt * W * (Kp / 1024.0); }
 
 // Launch plan chosen by the host for a rank-2 call.
@@ -104,7 +104,7 @@ struct Rank2Plan {
     int max_active_clusters;
     size_t smem;
     bool resident; // operators kept in registers for the whole run
-    int variant;   // 1: one-block, 2: two-block split-role, 3: two-block dataflow, 5: one CTA
+    int variant;   // 1: one-block, 2: two-block split-role (3: pinned as dataflow), 5: one CTA
     bool async = false;  // one-block: the form with asynchronous exchange (rank2_async.cuh)
     bool c_global; // one-block: the CTA's receiver rows are read from global memory (too many to stage)
     int nrt;       // one-block kernel: 32-row tiles per CTA (2 when Kp > 512)
@@ -122,12 +122,10 @@ cudaError_t launch_rank2_simt_f64(const Rank2Args& a, const Rank2Plan& plan, cud
 bool plan_rank2_simt_f32(int Kp, int M, int R, bool rank1, Rank2Plan* plan, int cluster_budget = 0);
 bool plan_rank2_simt_f64(int Kp, int M, int R, bool rank1, Rank2Plan* plan, int cluster_budget = 0);
 
-// Two-block split-role FP32 kernels (velocity and stress rows on different
-// CTAs): variant 2 synchronises with a cluster barrier per phase, variant 3
-// with per-block mbarriers fed by asynchronous stores (bounded waits).
+// Split-role FP32 kernel (velocity and stress rows on different CTAs, two
+// column blocks per cluster; bounded waits).
 bool plan_rank2_split_f32(int Kp, int M, int R, Rank2Plan* plan, int cluster_budget = 0);
-bool plan_rank2_dataflow_f32(int Kp, int M, int R, Rank2Plan* plan);
-// started (variant 2; may be null): an event recorded once every block has started.
+// started (may be null): an event recorded once every block has started.
 cudaError_t launch_rank2_split_f32(const Rank2Args& a, const Rank2Plan& plan, cudaStream_t st,
                                    cudaEvent_t started = nullptr);
 // One-CTA kernel (FP32, Kp <= 128): no cluster, both operators in registers.
