@@ -49,15 +49,14 @@ cudaError_t launch_rank2_stream_f32(const Rank2Args& a_in, int csz, int cols_per
     return L.launch(fn, args);
 }
 
-// Step-time model, microseconds per leapfrog step, fitted on GB300 at
-// Kp = 512: the split kernel takes 2.24 + 0.466 W (Kp / 512) for W columns
-// per block; the companion streams 2 (Kp / csz) Kp 4 bytes per CTA per step
-// from L2 at about 71 GB/s per SM and spends about 3 us per step on its two
-// cluster barriers, the row exchange and the epilogues (measured: 10.0 us
-// with clusters of 4, 17.1 us with clusters of 2).
+// Step-time model, microseconds per leapfrog step, fitted on GB300: the split
+// kernel's (rom_internal.h); the companion streams 2 (Kp / csz) Kp 4 bytes per
+// CTA per step from L2 at about 99 GB/s per SM and spends about 1.5 us per
+// step on the exchange and the epilogues (K = 512: 6.5 us with clusters of 4,
+// 11.8 us with clusters of 2; K = 448: 5.6 and 10.7 us).
 static double model_main_us(int Kp, int W) { return model_split_us(Kp, W); }
 static double model_comp_us(int Kp, int csz) {
-    return 2.0 * (Kp / (double)csz) * Kp * 4.0 / 71e3 + 3.0;
+    return 2.0 * (Kp / (double)csz) * Kp * 4.0 / 99e3 + 1.5;
 }
 
 // Companion placement: the columns [M - comp_cols, M) go to comp_n clusters
@@ -71,16 +70,24 @@ bool plan_rank2_companion(int Kp, int M, int R, Rank2Plan* p) {
     int dev = 0, nsm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    const int idle = nsm - base.cs * base.nclusters;
-    const double t_base = model_main_us(Kp, base.Wa);
+    // one wave of main clusters: the base plan's, or with more columns than
+    // fit it the widest blocks
+    const int nmain = base.max_active_clusters, waves = (base.nclusters + nmain - 1) / nmain;
+    const int rpc = (2 * R + base.cs - 1) / base.cs;
+    int wtop = base.Wa - kSplitBlock;
+    if (waves > 1)
+        while (split_smem_layout(wtop + kSplitBlock, Kp, rpc).total <= (size_t)device_smem_optin()) wtop += kSplitBlock;
+    const int idle = nsm - base.cs * nmain;
+    const double t_base = waves * model_main_us(Kp, base.Wa);
     double best = 0.95 * t_base;
     bool found = false;
     for (int csz : {2, 4}) {
         if (!stream_supported(Kp, csz)) continue;
-        // leave a fifth of the idle SMs free: not every idle SM may take a cluster
-        const int cmax = (idle * 4 / 5) / csz;
-        for (int w = base.Wa - kSplitCB; w >= kSplitCB; w -= kSplitCB) {
-            const int main_cols = 2 * base.nclusters * w;
+        // not every idle SM may take a cluster: leave a tenth of them free, a
+        // fifth with clusters of 4
+        const int cmax = (csz == 2 ? idle * 9 / 10 : idle * 4 / 5) / csz;
+        for (int w = wtop; w >= kSplitBlock; w -= kSplitBlock) {
+            const int main_cols = 2 * nmain * w;
             const int comp_cols = M - main_cols;
             if (comp_cols <= 0) continue;
             const int comp_n = (comp_cols + kStrCols - 1) / kStrCols;
@@ -91,6 +98,8 @@ bool plan_rank2_companion(int Kp, int M, int R, Rank2Plan* p) {
                 found = true;
                 *p = base;
                 p->Wv = p->Wa = w;
+                p->nclusters = nmain;
+                p->smem = split_smem_layout(w, Kp, rpc).total;
                 p->comp_cs = csz;
                 p->comp_n = comp_n;
                 p->comp_W = (comp_cols + comp_n - 1) / comp_n;
