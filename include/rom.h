@@ -412,9 +412,9 @@ rom_status rom_autotune_batched(const rom_job* jobs, int njobs, int prec, int pr
  * that many CTAs and at most width_cap columns per item; cluster_size 0
  * selects one launch per job (width_cap ignored).  Without a pinned or
  * tuned form, an FP32 list runs the form that the library's step-time
- * models predict faster for it: the work-list launch with clusters of 2
- * and a cap of 32, or one launch per job (chosen at the list's first call
- * and kept).  prec must be ROM_FP32.  Errors: ROM_E_INVAL (null or empty
+ * models predict fastest for it: the work-list launch with clusters of 2 or
+ * 4 and a cap of 8, 16, 24 or 32, or one launch per job (chosen at the
+ * list's first call and kept).  prec must be ROM_FP32.  Errors: ROM_E_INVAL (null or empty
  * list, a null handle, M < 1, another precision, a form outside the above).
  */
 rom_status rom_set_batched_form(const rom_job* jobs, int njobs, int prec, int cluster_size, int width_cap);

@@ -6,8 +6,10 @@
 #include <string.h>
 
 #include <algorithm>
+#include <functional>
 #include <map>
 #include <mutex>
+#include <queue>
 #include <tuple>
 #include <vector>
 
@@ -1196,7 +1198,7 @@ static int batch_tc_width(int prec, int M) {
 // 16 KB, else read from global memory.
 //
 // `wl` encodes the form: cs * 1000 + wcap.
-constexpr int kWlDefault = 2 * 1000 + 32;
+constexpr int kWlDefault = 2 * 1000 + 16;
 
 static bool wl_decode(int wl, int* cs, int* wcap) {
     *cs = wl / 1000;
@@ -1230,40 +1232,69 @@ static bool wl_job_layout(const rom_s* h, int M, int cs, int wcap, size_t budget
     return true;
 }
 
+// Makespan of items of the given costs on P clusters that take the next one,
+// longest first, whenever they are free.
+static double wl_makespan(std::vector<double> cost, int P) {
+    std::sort(cost.begin(), cost.end(), std::greater<double>());
+    std::priority_queue<double, std::vector<double>, std::greater<double>> free_at;
+    double end = 0.0;
+    for (const double c : cost) {
+        double t = c;
+        if ((int)free_at.size() >= P) {
+            t += free_at.top();
+            free_at.pop();
+        }
+        free_at.push(t);
+        end = t > end ? t : end;
+    }
+    return end;
+}
+
 // The form an FP32 job list runs in when nothing pinned or tuned one: the
-// work-list launch (kWlDefault) or one launch per job (0), whichever the
-// step-time models predict faster.  Work list: its items run longest first
-// on the co-resident clusters, so a step lasts about max(longest item,
-// sum of item times / clusters).  Per job: each job on its own plan, the
+// work-list launch of the cluster size and width cap, or one launch per job
+// (0), that the step-time models predict fastest.  Work list: its items'
+// makespan.  Wide items read an operator row for more columns, but the widest
+// of the largest models can last as long as the whole list should: 16 jobs of
+// K = 64 to 768, us a step at caps of 8, 16, 24 and 32, modelled / measured:
+// clusters of 2 103 / 101, 90 / 89, 124 / 126, 124 / 126; of 4 123 / 126,
+// 99 / 103, 97 / 101, 105 / 109; per job 131.  Per job: each job on its own plan, the
 // jobs side by side, so about max(slowest job, sum of job time x SMs / SMs
-// of the GPU).  Few items (small M, say 16 operators of 16 columns) leave
-// the work list's clusters idle while the split kernel keeps its operators
-// in registers; many uneven jobs favour the list.
+// of the GPU), the sum times kPerJobLoad for SMs that no cluster fits on and
+// for uneven ends (measured over 18 random lists: 1.0 to 1.9 times the sum).
+// Few items (small M, say 16 operators of 16 columns) leave the work list's
+// clusters idle while the split kernel keeps its operators in registers.
 static int batched_default_form(const rom_job* jobs, int njobs, int dev, int nsm) {
+    constexpr double kPerJobLoad = 1.33;
     int optin = 0;
     if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) {
         cudaGetLastError();
         return kWlDefault;
     }
     const size_t budget = (size_t)optin - 1024;
-    int cs = 0, wcap = 0;
-    wl_decode(kWlDefault, &cs, &wcap);
-    double sum = 0.0, cmax = 0.0;
-    long nitems = 0;
-    size_t smem = 0;
-    for (int i = 0; i < njobs; ++i) {
-        WlJob L;
-        if (!wl_job_layout(jobs[i].h, jobs[i].M, cs, wcap, budget, &L)) return 0;
-        const double c = model_streamed_us(jobs[i].h->Kp, L.nrt, L.W);
-        sum += c * L.nblocks;
-        cmax = c > cmax ? c : cmax;
-        nitems += L.nblocks;
-        smem = L.smem > smem ? L.smem : smem;
+    int best = 0;
+    double t_wl = 0.0;
+    for (int cs : {2, 4}) {
+        for (int wcap : {8, 16, 24, 32}) {
+            std::vector<double> cost;
+            size_t smem = 0;
+            bool fits = true;
+            for (int i = 0; i < njobs && fits; ++i) {
+                WlJob L;
+                fits = wl_job_layout(jobs[i].h, jobs[i].M, cs, wcap, budget, &L);
+                if (!fits) break;
+                cost.insert(cost.end(), L.nblocks, model_wl_us(jobs[i].h->Kp, L.nrt, L.W));
+                smem = L.smem > smem ? L.smem : smem;
+            }
+            const int P = fits ? worklist_max_clusters(cs, smem) : 0;
+            if (P <= 0) continue;
+            const double t = wl_makespan(std::move(cost), P);
+            if (best == 0 || t < t_wl) {
+                t_wl = t;
+                best = cs * 1000 + wcap;
+            }
+        }
     }
-    int P = worklist_max_clusters(cs, smem);
-    if (P <= 0) return 0;
-    if (P > nitems) P = (int)nitems;
-    const double t_wl = fmax(cmax, sum / P);
+    if (best == 0) return 0;
     double tmax = 0.0, sm_us = 0.0;
     for (int i = 0; i < njobs; ++i) {
         const rom_s* h = jobs[i].h;
@@ -1271,18 +1302,19 @@ static int batched_default_form(const rom_job* jobs, int njobs, int dev, int nsm
         double t = 0.0;
         if (plan_rank2_split_f32(h->Kp, jobs[i].M, h->R, &p)) {
             t = model_split_us(h->Kp, p.Wa);
-        } else if (plan_rank2_simt_f32(h->Kp, jobs[i].M, h->R, false, &p)) {
-            const int act = p.max_active_clusters > 0 ? p.max_active_clusters : 1;
-            t = ((p.nclusters + act - 1) / act) * model_streamed_us(h->Kp, p.nrt, p.Wa);
+        } else if (plan_rank2_simt_f32(h->Kp, jobs[i].M, h->R, false, &p, 1 << 20)) {  // (clusters of Kp / 64, as there)
+            t = model_streamed_us(h->Kp, p.nrt, p.Wa);
         } else {
-            return kWlDefault;
+            return best;
         }
-        const int busy = p.nclusters < p.max_active_clusters ? p.nclusters : p.max_active_clusters;
+        const int act = p.max_active_clusters > 0 ? p.max_active_clusters : 1;
+        t *= (p.nclusters + act - 1) / act;
+        const int busy = p.nclusters < act ? p.nclusters : act;
         tmax = t > tmax ? t : tmax;
         sm_us += t * busy * p.cs;
     }
-    const double t_pj = fmax(tmax, sm_us / nsm);
-    return t_pj < t_wl ? 0 : kWlDefault;
+    const double t_pj = fmax(tmax, kPerJobLoad * sm_us / nsm);
+    return t_pj < t_wl ? 0 : best;
 }
 
 static rom_status run_batched_worklist(const rom_job* jobs, int njobs, int nsteps, int r,
@@ -1338,7 +1370,7 @@ static rom_status run_batched_worklist(const rom_job* jobs, int njobs, int nstep
             g.Kp = Kp;
             g.Wa = W;
             g.c_global = cglob;
-            cost[i] = model_streamed_us(Kp, nrt, W);
+            cost[i] = model_wl_us(Kp, nrt, W);
             nitems += nb;
         }
         // ---- the item list, longest first (ties: job order, then columns)
@@ -1654,10 +1686,10 @@ rom_status rom_autotune_batched(const rom_job* jobs, int njobs, int prec, int pr
     double best = -1.0, best_scale = 1.0;
     int best_kthr = kAutoKthr, best_tcw = 1, best_wl = 0;
     rom_status rs = ROM_OK;
-    // FP32: work-list forms (clusters of 2 or 4 CTAs, width caps 16 / 32 /
-    // 64) besides one launch per job (0)
-    const int wls[7] = {kWlDefault, 2016, 2064, 4016, 4032, 4064, 0};
-    const int nwl = prec == ROM_FP32 ? 7 : 1;
+    // FP32: work-list forms (clusters of 2 or 4 CTAs, width caps 8 / 16 /
+    // 32 / 64) besides one launch per job (0)
+    const int wls[9] = {kWlDefault, 2008, 2032, 2064, 4008, 4016, 4032, 4064, 0};
+    const int nwl = prec == ROM_FP32 ? 9 : 1;
     for (int iw = 0; iw < nwl && e == cudaSuccess && rs == ROM_OK; ++iw)
     for (int t = 0; t < nk && e == cudaSuccess && rs == ROM_OK; ++t) {
         const int wl = prec == ROM_FP32 ? wls[iw] : 0;

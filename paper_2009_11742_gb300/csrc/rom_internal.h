@@ -89,10 +89,11 @@ struct Rank2Args {
 // Step-time models, microseconds per leapfrog step of one cluster, fitted on
 // GB300: the two-block split kernel with W columns per block (operators in
 // registers), and a kernel that streams its operators from L2 with nrt
-// 32-row tiles per CTA and W columns (one-block kernel above Kp = 512, the
-// work-list kernel).
+// 32-row tiles per CTA and W columns (one-block kernel above Kp = 512).
 inline double model_split_us(int Kp, int W) { return 0.3 + W * (0.15 + 0.00066 * Kp); }
 inline double model_streamed_us(int Kp, int nrt, int W) { return 3.5 + 0.71 * nrt * W * (Kp / 1024.0); }
+// An item of the work-list kernel (clusters of 2 or 4; K = 64 to 768).
+inline double model_wl_us(int Kp, int nrt, int W) { return 2.0 + nrt * (1.05 + W * (0.15 + 0.0003 * Kp)); }
 
 // Launch plan chosen by the host for a rank-2 call.
 struct Rank2Plan {
