@@ -94,9 +94,9 @@ static bool plan_adjoint_cs(int Kp, int M, int R, AdjPlan* p, bool f64, int cs) 
 }
 
 // The split-role plan (FP32, Kp <= 512): Kp / 32 CTAs, Wv columns per block
-// (a multiple of 4), two blocks per cluster, spread over the co-resident
+// (even), two blocks per cluster, spread over the co-resident
 // clusters.
-static bool plan_adjoint_split(int Kp, int M, int R, AdjPlan* p) {
+static bool plan_adjoint_split(int Kp, int M, AdjPlan* p) {
     p->f64 = false;
     p->split = true;
     p->KI = Kp / 64;
@@ -105,25 +105,30 @@ static bool plan_adjoint_split(int Kp, int M, int R, AdjPlan* p) {
     p->cb = kSplitCB;
     const int smax = device_smem_optin();
     int wcap = 0;
-    for (int w = kSplitCB; w <= 2048; w += kSplitCB) {
-        if (adj_split_smem_layout(w, Kp, R).total > (size_t)smax) break;
+    for (int w = kSplitBlock; w <= 2048; w += kSplitBlock) {
+        if (adj_split_smem_layout(w, Kp).total > (size_t)smax) break;
         wcap = w;
     }
     if (wcap == 0) return false;
     void* fn = adjoint_split_kernel(p->KI);
     if (!fn) return false;
-    const size_t smem_probe = adj_split_smem_layout(wcap, Kp, R).total;
+    const size_t smem_probe = adj_split_smem_layout(wcap, Kp).total;
     if (prepare_kernel<float>(fn, smem_probe) != cudaSuccess) return false;
     ClusterLaunch probe(p->cs, 1, kThreads, smem_probe);
     const int nact = probe.max_active(fn);
     if (nact <= 0) return false;
     int wv = (M + 2 * nact - 1) / (2 * nact);
-    wv = ((wv + kSplitCB - 1) / kSplitCB) * kSplitCB;
-    if (wv > wcap) wv = wcap;
+    wv = ((wv + kSplitBlock - 1) / kSplitBlock) * kSplitBlock;
+    if (wv > wcap) {
+        // more than one wave, of equal width
+        const int waves = (M + 2 * nact * wcap - 1) / (2 * nact * wcap);
+        wv = (M + 2 * nact * waves - 1) / (2 * nact * waves);
+        wv = ((wv + kSplitBlock - 1) / kSplitBlock) * kSplitBlock;
+    }
     p->Wv = wv;
     p->Wa = wv;
     p->nclusters = ((M + wv - 1) / wv + 1) / 2;
-    p->smem = adj_split_smem_layout(wv, Kp, R).total;
+    p->smem = adj_split_smem_layout(wv, Kp).total;
     p->model_us = 0.0;
     return true;
 }
@@ -136,7 +141,7 @@ static bool plan_adjoint_split(int Kp, int M, int R, AdjPlan* p) {
 // one tile per CTA.
 bool plan_adjoint(int Kp, int M, int R, AdjPlan* p, bool f64) {
     if (Kp <= 0 || Kp % 64 != 0 || Kp > (f64 ? 512 : 1024) || M <= 0 || R <= 0) return false;
-    if (!f64 && Kp <= 512 && plan_adjoint_split(Kp, M, R, p)) return true;
+    if (!f64 && Kp <= 512 && plan_adjoint_split(Kp, M, p)) return true;
     if (!plan_adjoint_cs(Kp, M, R, p, f64, 0)) return false;
     if (f64 || Kp <= 512) return true;
     for (int cs : {4, 2}) {

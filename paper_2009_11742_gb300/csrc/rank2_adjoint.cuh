@@ -339,187 +339,212 @@ __global__ void __launch_bounds__(kThreads, 1) rank2_adjoint_kernel(const AdjArg
     if (bad && tid == 0 && a.status) atomicCAS(a.status, 0, 6 /* ROM_E_NONFINITE */);
 }
 
-// ---- split-role reverse kernel (FP32, Kp <= 512).  The reverse step has
-// the forward step's shape: half A updates lamV from lamS, half B updates
-// lamS from the new lamV.  So the forward split kernel's schedule
-// (rank2_split.cuh) carries over: two column blocks half a step apart,
-// V-role CTAs holding their 64 rows of Asv^T in registers and owning those
-// rows of lamV, S-role CTAs doing the same with Avs^T and lamS, each finished
-// tile pushed into the other role's operand copy, one cluster barrier per
-// phase.  Time runs backwards: block A takes reverse step n = n_hi - 1 - k in
-// phase 2k, block B in phase 2k + 1.  The V role's epilogue adds 2 C^T r,
-// which does not depend on the adjoint state: adj_source_kernel forms it for
-// the launch's range of steps beforehand, and each V-role CTA copies its own
-// rows of it one phase ahead.  The S role, whose operand copy holds the same
-// new lamV, adds its slab's share of the period gradient to a per-CTA
-// partial after each of its phases.
+// ---- split-role reverse kernel (FP32, Kp <= 512).  The reverse step has the
+// forward step's shape: half A updates lamV from lamS, half B updates lamS from
+// the new lamV.  So the forward split kernel's schedule and exchange
+// (rank2_split.cuh) carry over: V-role CTAs hold their 64 rows of Asv^T in
+// registers and own those rows of lamV, S-role CTAs do the same with Avs^T and
+// lamS, both take the columns in groups of 4, and a group's rows travel by
+// st.async, counted on the receiver's mbarrier of the group.  Time runs
+// backwards: reverse step k is step n = n_hi - 1 - k.  The V role's update adds
+// 2 C^T r, which does not depend on the adjoint state: adj_source_kernel forms
+// it for the launch's range of steps beforehand, and a lane fetches its element
+// one group ahead.  The S role, whose operand copy holds the new lamV, adds its
+// slab's share of the period gradient to a per-CTA partial: a warp takes the
+// columns c = warp (mod 8), before its rows of lamS let lamV be overwritten.
+// K = 512, M = 128, 256 steps with checkpoints every 64, whole gradient: 5.53 ms
+// with a cluster barrier a phase here, 5.03 now.
 struct AdjSplitSmem {
-    size_t X, own, comp, src, g, T, gT, dfT, total;
+    size_t X, own, comp, g, T, gT, dfT, mbar, sent, flag, total;
 };
 
-__host__ __device__ inline AdjSplitSmem adj_split_smem_layout(int Wa, int Kp, int R) {
-    (void)R;  // the source term arrives precomputed, so the layout does not depend on R
+__host__ __device__ inline AdjSplitSmem adj_split_smem_layout(int Wa, int Kp) {
     AdjSplitSmem s{};
+    const size_t W = 2 * (size_t)Wa, G = W / kSplitCB, H = (size_t)Kp / kSplitRows;
     size_t o = 0;
-    s.X = o;    o += align16((size_t)2 * Wa * Kp * sizeof(float));
-    s.own = o;  o += align16((size_t)2 * Wa * kOwnStride * sizeof(float));
-    s.comp = o; o += align16((size_t)2 * Wa * kOwnStride * sizeof(float));
-    s.src = o;  o += align16((size_t)2 * Wa * kOwnStride * sizeof(float));
+    s.X = o;    o += align16(W * Kp * sizeof(float));
+    s.own = o;  o += align16(W * kSplitRows * sizeof(float));
+    s.comp = o; o += align16(W * kSplitRows * sizeof(float));
     s.g = o;    o += align16((size_t)kSplitRows * sizeof(float));
-    s.T = o;    o += align16((size_t)2 * Wa * sizeof(float));
-    s.gT = o;   o += align16((size_t)2 * Wa * sizeof(float));
-    s.dfT = o;  o += align16((size_t)2 * kAdjTab * Wa * sizeof(float));
+    s.T = o;    o += align16(W * sizeof(float));
+    s.gT = o;   o += align16(W * sizeof(float));
+    s.dfT = o;  o += align16((size_t)kAdjTab * W * sizeof(float));
+    s.mbar = o; o += align16(G * sizeof(unsigned long long));
+    s.sent = o; o += align16((1 + H) * G * sizeof(unsigned));
+    s.flag = o; o += 16;
     s.total = o;
     return s;
 }
 
 template <int KI>
 __global__ void __launch_bounds__(kThreads, 1) rank2_adjoint_split_kernel(const AdjArgsT<float> a) {
+    using Lay = AsyncLayout<float, kSplitCB>;
+    constexpr int CB = kSplitCB, Kp = 64 * KI, H = KI, cs = 2 * KI;
+    constexpr int kGroup = Kp * CB;
+    constexpr unsigned kGroupBytes = SplitLink<KI>::kGroupBytes;
     cg::cluster_group cluster = cg::this_cluster();
-    const int cs = (int)cluster.num_blocks();
-    const int H = cs / 2;
     const int crank = (int)cluster.block_rank();
     const bool vrole = crank < H;
     const int sl = vrole ? crank : crank - H;  // row slab
     const int row0 = sl * kSplitRows;
     const int peer0 = vrole ? H : 0;           // first CTA of the other role
     const int clu = blockIdx.x / cs;
-    const int Wa = a.Wa, Kp = a.Kp, R = a.R, M = a.M;
-    const int gc0_0 = 2 * clu * a.Wv, gc0_1 = gc0_0 + a.Wv;
-    const int nc0 = max(0, min(a.Wv, M - gc0_0)), nc1 = max(0, min(a.Wv, M - gc0_1));
-    auto gc0 = [&](int b) { return b ? gc0_1 : gc0_0; };
-    auto ncol = [&](int b) { return b ? nc1 : nc0; };
+    const int W = 2 * a.Wa, Gmax = W / CB, M = a.M;
+    const int gc0 = 2 * clu * a.Wv, ncol = max(0, min(2 * a.Wv, M - gc0));
+    const int G = (ncol + CB - 1) / CB;
+    const int N = ncol > 0 ? a.n_hi - a.n_lo : 0;  // reverse steps of this range
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int j = lane & 15;
     const int q = warp * 2 + (lane >> 4);      // row quad
     const float dt = (float)a.dt;
 
     extern __shared__ __align__(16) unsigned char smem[];
-    const AdjSplitSmem L = adj_split_smem_layout(Wa, Kp, R);
-    float* X = reinterpret_cast<float*>(smem + L.X);         // [2][Wa][Kp] operand copies
-    float* own = reinterpret_cast<float*>(smem + L.own);     // [2][Wa][72] owned rows
-    float* comp = reinterpret_cast<float*>(smem + L.comp);   // [2][Wa][72] Kahan carries
-    float* srcS = reinterpret_cast<float*>(smem + L.src);    // [2][Wa][72] C^T r, by phase parity
+    const AdjSplitSmem L = adj_split_smem_layout(a.Wa, Kp);
+    float* X = reinterpret_cast<float*>(smem + L.X);         // [G] groups of the operand
+    float* own = reinterpret_cast<float*>(smem + L.own);     // [G][warp][lane]: the lane's element of the group
+    float* comp = reinterpret_cast<float*>(smem + L.comp);   // its carry
     float* gown = reinterpret_cast<float*>(smem + L.g);      // [64]
-    float* Tcol = reinterpret_cast<float*>(smem + L.T);      // [2][Wa]
-    float* gTacc = reinterpret_cast<float*>(smem + L.gT);    // [2][Wa] period-gradient partials
-    float* dfT = reinterpret_cast<float*>(smem + L.dfT);     // [2][kAdjTab][Wa] df/dT per block
+    float* Tcol = reinterpret_cast<float*>(smem + L.T);      // [W]
+    float* gTacc = reinterpret_cast<float*>(smem + L.gT);    // [W] period-gradient partials
+    float* dfT = reinterpret_cast<float*>(smem + L.dfT);     // [kAdjTab][W] df/dT
+    unsigned long long* mbar = reinterpret_cast<unsigned long long*>(smem + L.mbar);  // [G]
+    unsigned* sent_out = reinterpret_cast<unsigned*>(smem + L.sent);  // [G]
+    unsigned* sent_in = sent_out + Gmax;                              // [H][G]
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + L.flag);
 
     const int Kown = vrole ? a.Kv : a.Ks;
-    const float* own_in = vrole ? a.lamV : a.lamS;
-    const float* comp_in = vrole ? a.compV : a.compS;
-    // operand copies: V role = the full lamS of each block; the S role's are
-    // filled by the first V-role pushes
-    for (int idx = tid; idx < 2 * Wa * Kp; idx += kThreads) {
-        const int b = idx / (Wa * Kp);
-        const int rem = idx - b * Wa * Kp;
-        const int c = rem / Kp, k = rem - (rem / Kp) * Kp;
-        X[idx] = (vrole && c < ncol(b) && k < a.Ks) ? a.lamS[(size_t)(gc0(b) + c) * a.Ks + k] : 0.f;
+    float* own_g = vrole ? a.lamV : a.lamS;
+    float* comp_g = vrole ? a.compV : a.compS;
+    // operand: V role = the full lamS; the S role's arrives with the first V-role sends
+    for (int idx = tid; idx < (vrole ? G * kGroup : 0); idx += kThreads) {
+        const int c = idx / Kp, k = idx - c * Kp;
+        X[(c / CB) * kGroup + Lay::at(c % CB, k)] =
+            c < ncol && k < a.Ks ? a.lamS[(size_t)(gc0 + c) * a.Ks + k] : 0.f;
     }
-    for (int idx = tid; idx < 2 * Wa * kOwnStride; idx += kThreads) {
-        const int b = idx / (Wa * kOwnStride);
-        const int rem = idx - b * Wa * kOwnStride;
-        const int c = rem / kOwnStride, rl = rem % kOwnStride, row = row0 + rl;
-        const bool ok = rl < kSplitRows && c < ncol(b) && row < Kown;
-        own[idx] = ok ? own_in[(size_t)(gc0(b) + c) * Kown + row] : 0.f;
-        comp[idx] = ok ? comp_in[(size_t)(gc0(b) + c) * Kown + row] : 0.f;
+    auto e_row = [&](int e) { return row0 + 8 * ((e >> 5) % kSplitWarps) + 4 * ((e >> 4) & 1) + ((e >> 2) & 3); };
+    auto e_col = [&](int e) { return CB * (e / kThreads) + (e & 3); };
+    for (int e = tid; e < G * kThreads; e += kThreads) {
+        const int c = e_col(e), row = e_row(e);
+        const bool ok = c < ncol && row < Kown;
+        own[e] = ok ? own_g[(size_t)(gc0 + c) * Kown + row] : 0.f;
+        comp[e] = ok ? comp_g[(size_t)(gc0 + c) * Kown + row] : 0.f;
     }
     if (tid < kSplitRows) gown[tid] = a.g_p[row0 + tid];  // the S role's gradient slab
-    for (int idx = tid; idx < 2 * Wa; idx += kThreads) {
-        const int b = idx / Wa, c = idx % Wa;
-        const bool ok = c < ncol(b);
-        Tcol[idx] = ok ? a.Tper[gc0(b) + c] : 1.f;
-        gTacc[idx] = ok ? a.gTpart[(size_t)crank * M + gc0(b) + c] : 0.f;
+    for (int c = tid; c < W; c += kThreads) {
+        Tcol[c] = c < ncol ? a.Tper[gc0 + c] : 1.f;
+        gTacc[c] = c < ncol ? a.gTpart[(size_t)crank * M + gc0 + c] : 0.f;
+    }
+    if (tid == 0) {
+        *abort_flag = 0;
+        for (int i = 0; i < Gmax; ++i) {
+            sent_out[i] = 0u;
+            mbar_init(&mbar[i], 1u);
+        }
+        fence_mbar_init_cluster();
+        for (int i = 0; i < Gmax; ++i) mbar_arrive_expect_tx(&mbar[i], kGroupBytes);
     }
     float op[4][4 * KI];
     load_op_quad<KI>(op, vrole ? a.opA_rm : a.opB_rm, Kp, row0 + 4 * q, j);
-
-    // the own rows' C^T r of block b, reverse step n (precomputed for the
-    // range), into parity buffer pb: 16 bytes per copy, zero for absent columns
-    auto prefetch_src = [&](int b, int n, int pb) {
-        float* dst = srcS + (size_t)pb * Wa * kOwnStride;
-        for (int idx = tid; idx < Wa * (kSplitRows / 4); idx += kThreads) {
-            const int c = idx / (kSplitRows / 4), piece = idx % (kSplitRows / 4);
-            const bool ok = c < ncol(b);
-            const float* gsrc = ok ? a.src + ((size_t)(n - a.n_lo) * M + gc0(b) + c) * Kp + row0 + 4 * piece
-                                   : a.src;  // a valid address for the zero fill
-            cp_async16(dst + (size_t)c * kOwnStride + 4 * piece, gsrc, ok ? 16 : 0);
-        }
+    const SplitLink<KI> link(smem_addr(smem), (unsigned)L.X, (unsigned)L.mbar, row0, warp, lane, peer0, H);
+    // this lane's element of C^T r at step n (every row of src is Kp wide)
+    const int own_row = row0 + 4 * q + (j >> 2);
+    auto source = [&](int k, int g) {
+        const int c = CB * g + (j & 3);
+        return vrole && k < N && c < ncol
+                   ? __ldcg(a.src + ((size_t)(a.n_hi - 1 - k - a.n_lo) * M + gc0 + c) * Kp + own_row) : 0.f;
     };
-    const int NR = a.n_hi - a.n_lo;  // reverse steps of this segment
-    if (vrole && NR > 0 && ncol(0) > 0) prefetch_src(0, a.n_hi - 1, 0);
-    // every CTA's copies must be initialised before any peer pushes into them
+    // every CTA's buffers and mbarriers are there before a peer writes to them
     cluster.sync();
 
-    const int nphase = 2 * NR + 1;
-    for (int p = 0; p < nphase; ++p) {
-        int b, k;
-        if (vrole) { b = p & 1; k = (p - b) >> 1; }
-        else { b = (p & 1) ^ 1; k = (p - 1 - b) >> 1; }
-        const bool work = k >= 0 && k < NR && ncol(b) > 0;
-        const int n = a.n_hi - 1 - k;
-        float* Xb = X + (size_t)b * Wa * Kp;
-        float* ownb = own + (size_t)b * Wa * kOwnStride;
-        float* compb = comp + (size_t)b * Wa * kOwnStride;
-        if (vrole) {
-            // this phase's source term (copied during the previous phase into
-            // parity buffer p & 1), then the next phase's copies into the other
-            // buffer (read last in phase p - 1, which a cluster barrier has closed)
-            cp_async_wait_all();
-            __syncthreads();
-            const int b2 = (p + 1) & 1, k2 = (p + 1 - b2) >> 1;
-            if (k2 < NR && ncol(b2) > 0) prefetch_src(b2, a.n_hi - 1 - k2, (p + 1) & 1);
-            if (work) {
-                // half A: lamV <- lamV + dt Asv^T lamS + 2 C^T r^{n+1}
-                split_phase<KI, false, false, true>(cluster, op, Xb, ownb, compb, gown, gown, Xb, dt, Wa, Kp,
-                                                    row0, H, peer0, q, j, warp, lane, nullptr, Kown, ncol(b),
-                                                    srcS + (size_t)(p & 1) * Wa * kOwnStride);
-            }
-        } else if (work) {
-            // the block's df/dT table every kAdjTab of its steps
-            if (k % kAdjTab == 0) {
-                for (int idx = tid; idx < kAdjTab * ncol(b); idx += kThreads) {
-                    const int i = idx / ncol(b), c = idx % ncol(b);
-                    if (n - i >= a.n_lo)
-                        dfT[(b * kAdjTab + i) * Wa + c] =
-                            wavelet_dT_eval<float>(a.wavelet, (long long)a.n0 + n - i, a.dt, Tcol[b * Wa + c]);
-                }
-                __syncthreads();
-            }
-            // half B: lamS <- lamS + dt Avs^T lamV (the new lamV of block b)
-            split_phase<KI, false, false>(cluster, op, Xb, ownb, compb, gown, gown, Xb, dt, Wa, Kp, row0, H,
-                                          peer0, q, j, warp, lane, nullptr, Kown, ncol(b));
-            // period gradient of step n over this slab's rows of the same new
-            // lamV: dt (g_slab . a_V[:, c]) df/dT(t_n; T_c), fixed order
-            const float* dfn = dfT + (b * kAdjTab + (k % kAdjTab)) * Wa;
-            for (int c = warp; c < ncol(b); c += kSplitWarps) {
-                const float* av = Xb + (size_t)c * Kp + row0;
-                float sg = gown[lane] * av[lane];
-                sg = __fmaf_rn(gown[lane + 32], av[lane + 32], sg);
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) sg += __shfl_xor_sync(0xffffffffu, sg, o);
-                if (lane == 0) gTacc[b * Wa + c] = __fmaf_rn(dt * sg, dfn[c], gTacc[b * Wa + c]);
+    auto wait = [&](int g, unsigned parity) {
+        const bool ok = mbar_wait_bounded(&mbar[g], parity, a.spin_limit, abort_flag);
+        return __all_sync(0xffffffffu, ok) != 0;
+    };
+    // this warp's sends: nsent steps of the groups below gsent, one less from there on
+    int nsent = 0, gsent = G;
+    bool dead = false, ready = false;
+    float src_next = source(0, 0);
+    for (int kb = 0; kb < N; kb += kAdjTab) {
+        // (the barrier also keeps the last table until every warp has read it)
+        if (__syncthreads_or(dead)) break;
+        if (!vrole) {
+            for (int idx = tid; idx < kAdjTab * W; idx += kThreads) {
+                const int i = idx / W, c = idx - i * W, n = a.n_hi - 1 - kb - i;
+                dfT[idx] = n >= a.n_lo && c < ncol
+                               ? wavelet_dT_eval<float>(a.wavelet, (long long)a.n0 + n, a.dt, Tcol[c]) : 0.f;
             }
         }
-        cluster.sync();
+        __syncthreads();
+        const int ke = min(N, kb + kAdjTab);
+        for (int k = kb; k < ke && !dead; ++k) {
+            // operand: lamS after k steps, phase k - 1 (V role), the new lamV, phase k (S role)
+            const int ph = vrole ? k - 1 : k;
+            for (int g = 0; g < G; ++g) {
+                const float* Xg = X + g * kGroup;
+                float* yp = own + g * kThreads + tid;
+                float* cp = comp + g * kThreads + tid;
+                const float y0 = *yp, src = src_next;
+                float carry = *cp;
+                src_next = g + 1 < G ? source(k, g + 1) : source(k + 1, 0);
+                if (ph >= 0) {
+                    if (!ready && !wait(g, (unsigned)(ph & 1))) {
+                        dead = true;
+                        nsent = k + 1, gsent = g;
+                        break;
+                    }
+                    if (tid == 0 && ph + 1 < N) mbar_arrive_expect_tx(&mbar[g], kGroupBytes);
+                }
+                SplitAcc<KI> acc;
+                acc.products(op, Xg, j);
+                {
+                    // has the next group's operand arrived? (asked ahead, as forwards)
+                    const bool wrap = g + 1 == G;
+                    const int ph2 = wrap ? ph + 1 : ph;
+                    ready = __all_sync(0xffffffffu, ph2 >= 0 && ph2 < N && mbar_test_wait(&mbar[wrap ? 0 : g + 1], ph2 & 1));
+                }
+                const float tot = acc.reduce(j);
+                // half A: lamV += dt Asv^T lamS + 2 C^T r;  half B: lamS += dt Avs^T lamV
+                const float inc = vrole ? __fmaf_rn(tot, dt, 2.f * src) : tot * dt;
+                const float y = kahan_add(y0, inc, carry);
+                *yp = y;
+                *cp = carry;
+                if (!vrole) {
+                    // period gradient of the step over this slab's rows of the same new
+                    // lamV: dt (g_slab . a_V[:, c]) df/dT(t_n; T_c), fixed order
+                    const int c4 = (warp - CB * g) & (kSplitWarps - 1);  // column c of the group with c = warp (mod 8)
+                    if (c4 < CB && CB * g + c4 < ncol) {
+                        const int c = CB * g + c4;
+                        float sg = gown[lane] * Xg[Lay::at(c4, row0 + lane)];
+                        sg = __fmaf_rn(gown[lane + 32], Xg[Lay::at(c4, row0 + lane + 32)], sg);
+#pragma unroll
+                        for (int o = 16; o > 0; o >>= 1) sg += __shfl_xor_sync(0xffffffffu, sg, o);
+                        if (lane == 0) gTacc[c] = __fmaf_rn(dt * sg, dfT[(k - kb) * W + c], gTacc[c]);
+                    }
+                    __syncwarp();
+                }
+                link.send(g, y);
+            }
+        }
+        if (!dead) nsent = ke;
     }
+    // the V role has received the last lamS, too
+    if (vrole && !dead && nsent == N && N > 0)
+        for (int g = 0; g < G && !dead; ++g) dead = !wait(g, (unsigned)((N - 1) & 1));
+    if (dead && lane == 0) *abort_flag = 1;
+    split_drain<KI>(cluster, mbar, sent_out, sent_in, Gmax, G, N, vrole, sl, peer0, nsent, gsent, true, abort_flag,
+                    a.status);
 
     // ---- write back the owned rows, carries and the period-gradient partials
-    float* out = vrole ? a.lamV : a.lamS;
-    float* cout_ = vrole ? a.compV : a.compS;
     int bad = 0;
-    for (int b = 0; b < 2; ++b) {
-        for (int idx = tid; idx < ncol(b) * kSplitRows; idx += kThreads) {
-            const int c = idx / kSplitRows, rl = idx % kSplitRows, row = row0 + rl;
-            if (row < Kown) {
-                const float x = own[(size_t)b * Wa * kOwnStride + c * kOwnStride + rl];
-                out[(size_t)(gc0(b) + c) * Kown + row] = x;
-                cout_[(size_t)(gc0(b) + c) * Kown + row] = comp[(size_t)b * Wa * kOwnStride + c * kOwnStride + rl];
-                bad |= !is_finite(x);
-            }
+    for (int e = tid; e < G * kThreads; e += kThreads) {
+        const int c = e_col(e), row = e_row(e);
+        if (c < ncol && row < Kown) {
+            own_g[(size_t)(gc0 + c) * Kown + row] = own[e];
+            comp_g[(size_t)(gc0 + c) * Kown + row] = comp[e];
+            bad |= !is_finite(own[e]);
         }
-        for (int c = tid; c < ncol(b); c += kThreads) a.gTpart[(size_t)crank * M + gc0(b) + c] = gTacc[b * Wa + c];
     }
+    for (int c = tid; c < ncol; c += kThreads) a.gTpart[(size_t)crank * M + gc0 + c] = gTacc[c];
     bad = __syncthreads_or(bad);
     if (bad && tid == 0 && a.status) atomicCAS(a.status, 0, 6 /* ROM_E_NONFINITE */);
 }

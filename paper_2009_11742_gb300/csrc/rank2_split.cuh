@@ -60,7 +60,6 @@
 namespace romk {
 
 constexpr int kSplitRows = 64;   // rows of one operator per CTA
-constexpr int kOwnStride = 72;   // padded column stride of the own-row buffers (reverse kernel)
 constexpr int kSplitCB = 4;      // columns per register group
 constexpr int kSplitBlock = 2;   // a block's columns are a multiple of this: two blocks hold whole groups
 constexpr int kSplitWarps = kThreads / 32;
@@ -131,92 +130,6 @@ __device__ __forceinline__ void load_op_quad(float (&op)[4][4 * KI], const float
             load4_ro(A + (size_t)(row + rr) * Kp + 64 * i + 4 * j, x);
 #pragma unroll
             for (int t = 0; t < 4; ++t) op[rr][4 * i + t] = x[t];
-        }
-    }
-}
-
-// One phase of one role of the reverse-time kernel on block b: own rows += dt (op . X_b [+ g f^T] [+ Xref]),
-// pushing every finished 8 x 4 warp tile to the H peer CTAs of the other role.
-// With XR, Xref points at block b's first column of the role's reduced
-// reference state (Krows x columns); each lane fetches its epilogue's value
-// before the products.  XR is a template flag so that runs without the term
-// compile to exactly the code they had without it.  ADJ (the reverse-time
-// adjoint's half A): own rows += dt (op . X_b) + 2 C_own^T r, with asrc
-// block b's C_own^T r for this step ([Wa][kOwnStride], precomputed).
-template <int KI, bool FORCED, bool XR, bool ADJ = false>
-__device__ __forceinline__ void split_phase(cg::cluster_group& cluster, const float (&op)[4][4 * KI],
-                                            const float* __restrict__ X, float* __restrict__ own,
-                                            float* __restrict__ comp, const float* __restrict__ gown,
-                                            const float* __restrict__ fcol, float* remote_X_b,
-                                            const float dt, const int Wa, const int Kp,
-                                            const int row0, const int H, const int peer0,
-                                            const int q, const int j, const int warp,
-                                            const int lane, const float* __restrict__ Xref,
-                                            const int Krows, const int ncol,
-                                            const float* __restrict__ asrc = nullptr) {
-    constexpr int CB = kSplitCB;
-    for (int c0 = 0; c0 < Wa; c0 += CB) {
-        float xr = 0.f;
-        if constexpr (XR) {
-            // Xref is null for a role whose part of the term is not given
-            const int si = rs16_slot<4 * CB>(j);
-            const int rl = 4 * q + si / CB, c = c0 + si % CB;
-            if (Xref && c < ncol && row0 + rl < Krows) xr = Xref[(size_t)c * Krows + row0 + rl];
-        }
-        float acc[4][CB];
-#pragma unroll
-        for (int r = 0; r < 4; ++r)
-#pragma unroll
-            for (int cc = 0; cc < CB; ++cc) acc[r][cc] = 0.f;
-#pragma unroll
-        for (int i = 0; i < KI; ++i) {
-            float x[CB][4];
-#pragma unroll
-            for (int cc = 0; cc < CB; ++cc) load4(X + (size_t)(c0 + cc) * Kp + 64 * i + 4 * j, x[cc]);
-#pragma unroll
-            for (int t = 0; t < 4; ++t)
-#pragma unroll
-                for (int cc = 0; cc < CB; ++cc)
-#pragma unroll
-                    for (int r = 0; r < 4; ++r)
-                        acc[r][cc] = __fmaf_rn(op[r][4 * i + t], x[cc][t], acc[r][cc]);
-        }
-        float v[4 * CB];
-#pragma unroll
-        for (int r = 0; r < 4; ++r)
-#pragma unroll
-            for (int cc = 0; cc < CB; ++cc) v[r * CB + cc] = acc[r][cc];
-        int vi;
-        bool active;
-        const float tot = reduce_scatter16<float, 4 * CB>(v, j, vi, active);
-        {
-            const int rl = 4 * q + vi / CB;
-            const int c = c0 + vi % CB;
-            float inc = tot;
-            if constexpr (ADJ) {
-                const float src = asrc[c * kOwnStride + rl];
-                inc = __fmaf_rn(tot, dt, 2.f * src);
-            } else {
-                if (FORCED) inc = __fmaf_rn(gown[rl], fcol[c], inc);
-                if constexpr (XR) inc = inc + xr;
-                inc = inc * dt;
-            }
-            float* yp = own + c * kOwnStride + rl;
-            *yp = kahan_add(*yp, inc, comp[c * kOwnStride + rl]);
-        }
-        __syncwarp();
-        // this warp's tile: rows 8 warp .. 8 warp + 7, columns c0 .. c0 + 3, as
-        // eight 16-byte pieces; lane L carries piece L % 8 to peers L/8, L/8 + 4
-        {
-            const int piece = lane & 7, cc = piece >> 1, half = piece & 1;
-            const int c = c0 + cc;
-            const int rloc = 8 * warp + 4 * half;
-            const float4 val = *reinterpret_cast<const float4*>(own + c * kOwnStride + rloc);
-            float4* dst_local = reinterpret_cast<float4*>(remote_X_b + (size_t)c * Kp + row0 + rloc);
-            for (int d = lane >> 3; d < H; d += 4) {
-                float4* dst = cluster.map_shared_rank(dst_local, peer0 + d);
-                *dst = val;
-            }
         }
     }
 }
@@ -310,6 +223,128 @@ __device__ __forceinline__ void trace_tile(const float* C, const float* X, int K
                     if ((lane & 1) == 0 && jj < nj && c < nc) out[(size_t)c * R + jj] = acc[0];
 }
 
+// The products of the thread's 4 rows with a group's 4 columns, reduced over the
+// 16 chunk lanes: lane chunk j is left with row j / 4, column j mod 4.
+template <int KI>
+struct SplitAcc {
+    float a[4][kSplitCB];
+    __device__ __forceinline__ void products(const float (&op)[4][4 * KI], const float* Xg, int j) {
+        constexpr int CB = kSplitCB;
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+            for (int cc = 0; cc < CB; ++cc) a[r][cc] = 0.f;
+#pragma unroll
+        for (int i = 0; i < KI; ++i) {
+            float x[CB][4];
+#pragma unroll
+            for (int cc = 0; cc < CB; ++cc) AsyncLayout<float, CB>::load(Xg + 64 * CB * i, cc, j, x[cc]);
+#pragma unroll
+            for (int t = 0; t < 4; ++t)
+#pragma unroll
+                for (int cc = 0; cc < CB; ++cc)
+#pragma unroll
+                    for (int r = 0; r < 4; ++r) a[r][cc] = __fmaf_rn(op[r][4 * i + t], x[cc][t], a[r][cc]);
+        }
+    }
+    __device__ __forceinline__ float reduce(int j) {
+        float v[4 * kSplitCB];
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+            for (int cc = 0; cc < kSplitCB; ++cc) v[r * kSplitCB + cc] = a[r][cc];
+        int vi;
+        bool active;
+        return reduce_scatter16<float, 4 * kSplitCB>(v, j, vi, active);
+    }
+};
+
+// A warp's way to the other role: 8 lanes a peer carry its 8 x 4 piece of a
+// group, lane p of them unit p (the rows of quad p / 4, column (p mod 4) ^ swz).
+template <int KI>
+struct SplitLink {
+    static constexpr int H = KI, NP = (H + 3) / 4;  // peers, peers a lane sends to
+    static constexpr unsigned kGroupBytes = 64u * KI * kSplitCB * sizeof(float);
+    static constexpr unsigned kWarpBytes = 8 * kSplitCB * sizeof(float);
+    unsigned mX, mB, dpeer[NP];  // own addresses of the piece and the mbarriers, distance of the peers' windows
+    int src_lane, peer, npeer;
+    __device__ __forceinline__ SplitLink(unsigned base, unsigned xoff, unsigned boff, int row0, int warp, int lane,
+                                         int peer0, int npeer_)
+        : peer(lane >> 3), npeer(npeer_) {
+        using Lay = AsyncLayout<float, kSplitCB>;
+        const int p8 = lane & 7, kqs = (row0 >> 2) + 2 * warp + (p8 >> 2);
+        src_lane = 16 * (p8 >> 2) + ((p8 & 3) ^ Lay::swz(kqs));
+        mX = base + xoff + (unsigned)(kqs * Lay::U + (p8 & 3)) * 16u;
+        mB = base + boff;
+#pragma unroll
+        for (int m = 0; m < NP; ++m) {
+            const int d = peer + 4 * m;
+            dpeer[m] = cluster_addr(base, peer0 + (d < H ? d : 0)) - base;
+        }
+    }
+    __device__ __forceinline__ void send(int g, float y) const {
+        float u[4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) u[r] = __shfl_sync(0xffffffffu, y, src_lane + 4 * r);
+#pragma unroll
+        for (int m = 0; m < NP; ++m)
+            if (peer + 4 * m < npeer)
+                asm volatile(
+                    "st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];"
+                    ::"r"(mX + (unsigned)g * kGroupBytes + dpeer[m]), "f"(u[0]), "f"(u[1]), "f"(u[2]), "f"(u[3]),
+                      "r"(mB + 8u * (unsigned)g + dpeer[m])
+                    : "memory");
+    }
+};
+
+// The end of a split-role run.  Every CTA (a timeout or not, so the barriers
+// stay cluster-uniform) tells each consumer how many bytes it sent per group;
+// past the barrier no CTA issues another store.  A consumer then retires, on
+// the phase armed last, the bytes that will not come, so that the phase
+// completes when every byte sent has landed, and waits for it (bounded).
+// After a complete run nothing is outstanding.  nsent, gsent: the calling
+// warp has sent nsent steps of the groups below gsent, one less from there on.
+template <int KI>
+__device__ __forceinline__ void split_drain(cg::cluster_group& cluster, unsigned long long* mbar, unsigned* sent_out,
+                                            unsigned* sent_in, int Gmax, int G, int N, bool vrole, int s, int peer0,
+                                            int nsent, int gsent, bool sends, volatile int* abort_flag,
+                                            int* status) {
+    constexpr int H = KI;
+    using Link = SplitLink<KI>;
+    const int tid = threadIdx.x;
+    if ((tid & 31) == 0 && sends)
+        for (int g = 0; g < G; ++g)
+            atomicAdd(&sent_out[g], Link::kWarpBytes * (unsigned)(nsent - (g >= gsent ? 1 : 0)));
+    __syncthreads();
+    for (int idx = tid; idx < H * G; idx += kThreads) {
+        const int d = idx / G, g = idx - d * G;
+        asm volatile("st.shared::cluster.u32 [%0], %1;"
+                     ::"r"(cluster_addr(smem_addr(sent_in + s * Gmax + g), peer0 + d)), "r"(sent_out[g])
+                     : "memory");
+    }
+    cluster.sync();
+    if (tid == 0) {
+        bool late = false;
+        for (int g = 0; g < (N > 0 ? G : 0); ++g) {
+            unsigned got = 0u;
+            for (int d = 0; d < H; ++d) got += sent_in[d * Gmax + g];
+            // phases this thread armed: one at the start, one after each wait but the last
+            const int done = nsent - (g >= gsent ? 1 : 0), arms = min(N, max(1, vrole ? done : done + 1));
+            const unsigned expect = (unsigned)arms * Link::kGroupBytes;
+            if (expect != got) mbar_complete_tx(&mbar[g], expect - got);
+            const long long t0 = clock64();
+            while (!mbar_try_wait(&mbar[g], (unsigned)(arms - 1) & 1u)) {
+                if (clock64() - t0 > 4000000000LL) {
+                    late = true;
+                    break;
+                }
+            }
+        }
+        if ((late || *abort_flag) && status) atomicCAS(status, 0, 5 /* ROM_E_TIMEOUT */);
+    }
+    __syncthreads();
+}
+
 // MODE: 0 plain; 1 adds the reduced reference state (a.Xv / a.Xs); 2 is the
 // rank-3 grouped launch (operator table a.group).  A template parameter, so
 // that each instance compiles to exactly the code its runs need.
@@ -318,9 +353,7 @@ __global__ void __launch_bounds__(kThreads, 1) rank2_split_kernel(const Rank2Arg
     using Lay = AsyncLayout<float, kSplitCB>;
     constexpr int CB = kSplitCB, Kp = 64 * KI, H = KI, cs = 2 * KI;
     constexpr int kGroup = Kp * CB;                                  // elements of a group's operand
-    constexpr unsigned kGroupBytes = (unsigned)(kGroup * sizeof(float));
-    constexpr unsigned kWarpBytes = 8 * CB * sizeof(float);          // a warp's part of it
-    constexpr int NP = (H + 3) / 4;                                  // peers a lane sends to
+    constexpr unsigned kGroupBytes = SplitLink<KI>::kGroupBytes;
     cg::cluster_group cluster = cg::this_cluster();
     const int crank = (int)cluster.block_rank();
     // rank-3 grouped launch: operator `job` of the table, cluster `clu` of it
@@ -399,19 +432,8 @@ __global__ void __launch_bounds__(kThreads, 1) rank2_split_kernel(const Rank2Arg
     // this lane's element of a group: row 4 q + j / 4 of the slab, column j mod 4
     const float gr = vrole ? static_cast<const float*>(MODE == 2 ? gop->g_p : a.g_p)[row0 + 4 * q + (j >> 2)] : 0.f;
     const int own_row = row0 + 4 * q + (j >> 2);
-    // sends: 8 lanes a peer carry the warp's piece, lane p its unit p: the rows
-    // of quad p / 4, column (p mod 4) ^ swz
-    const int p8 = lane & 7, kqs = (row0 >> 2) + 2 * warp + (p8 >> 2);
-    const int src_lane = 16 * (p8 >> 2) + ((p8 & 3) ^ Lay::swz(kqs));
-    const unsigned base = smem_addr(smem);
-    const unsigned mX = base + (unsigned)L.X + (unsigned)(kqs * Lay::U + (p8 & 3)) * 16u, mB = smem_addr(mbar);
-    unsigned dpeer[NP];
-#pragma unroll
-    for (int m = 0; m < NP; ++m) {
-        const int d = (lane >> 3) + 4 * m;
-        dpeer[m] = cluster_addr(base, peer0 + (d < H ? d : 0)) - base;
-    }
-    const int npeer = a.debug_skip_push && crank == 0 ? 0 : H;  // fault injection: this CTA sends nothing
+    const bool sends = !(a.debug_skip_push && crank == 0);  // fault injection: this CTA sends nothing
+    const SplitLink<KI> link(smem_addr(smem), (unsigned)L.X, (unsigned)L.mbar, row0, warp, lane, peer0, sends ? H : 0);
     const float* Xrole = static_cast<const float*>(vrole ? a.Xv : a.Xs);
     const float* ftg = static_cast<const float*>(a.ftab);
     // every CTA's buffers and mbarriers are there before a peer writes to them
@@ -468,24 +490,8 @@ __global__ void __launch_bounds__(kThreads, 1) rank2_split_kernel(const Rank2Arg
                     }
                     if (tid == 0 && ph + 1 < N) mbar_arrive_expect_tx(&mbar[g], kGroupBytes);
                 }
-                float acc[4][CB];
-#pragma unroll
-                for (int r = 0; r < 4; ++r)
-#pragma unroll
-                    for (int cc = 0; cc < CB; ++cc) acc[r][cc] = 0.f;
-#pragma unroll
-                for (int i = 0; i < KI; ++i) {
-                    float x[CB][4];
-#pragma unroll
-                    for (int cc = 0; cc < CB; ++cc) Lay::load(Xg + 64 * CB * i, cc, j, x[cc]);
-#pragma unroll
-                    for (int t = 0; t < 4; ++t)
-#pragma unroll
-                        for (int cc = 0; cc < CB; ++cc)
-#pragma unroll
-                            for (int r = 0; r < 4; ++r)
-                                acc[r][cc] = __fmaf_rn(op[r][4 * i + t], x[cc][t], acc[r][cc]);
-                }
+                SplitAcc<KI> acc;
+                acc.products(op, Xg, j);
                 // has the next group's operand arrived?  Asked here, the answer
                 // is there when the reduction and the update are done.
                 {
@@ -493,14 +499,7 @@ __global__ void __launch_bounds__(kThreads, 1) rank2_split_kernel(const Rank2Arg
                     const int ph2 = wrap ? ph + 1 : ph;
                     ready = __all_sync(0xffffffffu, ph2 >= 0 && ph2 < N && mbar_test_wait(&mbar[wrap ? 0 : g + 1], ph2 & 1));
                 }
-                float v[4 * CB];
-#pragma unroll
-                for (int r = 0; r < 4; ++r)
-#pragma unroll
-                    for (int cc = 0; cc < CB; ++cc) v[r * CB + cc] = acc[r][cc];
-                int vi;
-                bool active;
-                float inc = reduce_scatter16<float, 4 * CB>(v, j, vi, active);  // value vi = j
+                float inc = acc.reduce(j);
                 if (vrole) inc = __fmaf_rn(gr, f, inc);
                 if constexpr (MODE == 1) inc = inc + xr;
                 inc = inc * dt;
@@ -514,17 +513,7 @@ __global__ void __launch_bounds__(kThreads, 1) rank2_split_kernel(const Rank2Arg
                                    traces + ((size_t)rec * a.Mtot + gc0 + CB * g) * a.R + s * a.rpc, a.R);
                     __syncwarp();
                 }
-                float u[4];
-#pragma unroll
-                for (int r = 0; r < 4; ++r) u[r] = __shfl_sync(0xffffffffu, y, src_lane + 4 * r);
-#pragma unroll
-                for (int m = 0; m < NP; ++m)
-                    if ((lane >> 3) + 4 * m < npeer)
-                        asm volatile(
-                            "st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];"
-                            ::"r"(mX + (unsigned)g * kGroupBytes + dpeer[m]), "f"(u[0]), "f"(u[1]), "f"(u[2]),
-                            "f"(u[3]), "r"(mB + 8u * (unsigned)g + dpeer[m])
-                            : "memory");
+                link.send(g, y);
             }
             if (record) {
                 to_rec = a.r;
@@ -537,43 +526,8 @@ __global__ void __launch_bounds__(kThreads, 1) rank2_split_kernel(const Rank2Arg
     if (vrole && !dead && nsent == N && N > 0)
         for (int g = 0; g < G && !dead; ++g) dead = !wait(g, (unsigned)((N - 1) & 1));
     if (dead && lane == 0) *abort_flag = 1;
-    // ---- drain.  Every CTA (a timeout or not, so the barriers stay
-    // cluster-uniform) tells each consumer how many bytes it sent per group;
-    // past the barrier no CTA issues another store.  A consumer then retires, on
-    // the phase armed last, the bytes that will not come, so that the phase
-    // completes when every byte sent has landed, and waits for it (bounded).
-    // After a complete run nothing is outstanding.
-    if (lane == 0 && npeer > 0)
-        for (int g = 0; g < G; ++g) atomicAdd(&sent_out[g], kWarpBytes * (unsigned)(nsent - (g >= gsent ? 1 : 0)));
-    __syncthreads();
-    for (int idx = tid; idx < H * G; idx += kThreads) {
-        const int d = idx / G, g = idx - d * G;
-        asm volatile("st.shared::cluster.u32 [%0], %1;"
-                     ::"r"(cluster_addr(smem_addr(sent_in + s * Gmax + g), peer0 + d)), "r"(sent_out[g])
-                     : "memory");
-    }
-    cluster.sync();
-    if (tid == 0) {
-        bool late = false;
-        for (int g = 0; g < (N > 0 ? G : 0); ++g) {
-            unsigned got = 0u;
-            for (int d = 0; d < H; ++d) got += sent_in[d * Gmax + g];
-            // phases this thread armed: one at the start, one after each wait but the last
-            const int done = nsent - (g >= gsent ? 1 : 0), arms = min(N, max(1, vrole ? done : done + 1));
-            const unsigned expect = (unsigned)arms * kGroupBytes;
-            if (expect != got) mbar_complete_tx(&mbar[g], expect - got);
-            const unsigned parity = (unsigned)(arms - 1) & 1u;
-            const long long t0 = clock64();
-            while (!mbar_try_wait(&mbar[g], parity)) {
-                if (clock64() - t0 > 4000000000LL) {
-                    late = true;
-                    break;
-                }
-            }
-        }
-        if ((late || *abort_flag) && a.status) atomicCAS(a.status, 0, 5 /* ROM_E_TIMEOUT */);
-    }
-    __syncthreads();
+    split_drain<KI>(cluster, mbar, sent_out, sent_in, Gmax, G, N, vrole, s, peer0, nsent, gsent, sends, abort_flag,
+                    a.status);
 
     // ---- write back the owned rows and carries
     int bad = 0;

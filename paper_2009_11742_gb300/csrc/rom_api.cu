@@ -2020,6 +2020,7 @@ rom_status adjoint_run(rom_s* h, const void* V0, const void* S0, const void* Tp,
         aa.status = h->status;
         aa.dt = h->dt;
         aa.wavelet = h->wavelet;
+        aa.spin_limit = h->wait_limit;
         aa.n0 = 0;
         aa.n_lo = n_start;
         aa.n_hi = n_start + len;

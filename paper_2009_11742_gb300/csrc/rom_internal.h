@@ -223,6 +223,7 @@ struct AdjArgsT {
     int Kv, Ks, Kp, R, M, Wv, Wa;
     int nrt;              // 32-row tiles the layout holds per CTA (FP32 above Kp = 512)
     int wavelet;          // source signal of the periods (see Rank2Args)
+    long long spin_limit; // see Rank2Args (the split-role kernel)
 };
 using AdjArgs = AdjArgsT<float>;
 struct AdjPlan {
