@@ -34,6 +34,7 @@
 #include <map>
 #include <mutex>
 #include <new>
+#include <utility>
 #include <tuple>
 #include <vector>
 
@@ -95,6 +96,7 @@ struct FomPass {
     const FomCtl* ctl;
     long long off, n0;
     int Nr, Nt, M, nrecv, r, wavelet;
+    int Mt;             // realizations of the run (M: of the buffers, padded)
     int src_i, src_j;   // the source's grid point
     int seg_rows;       // radial rows per block
     int nmarch;         // blocks that march; those beyond record receivers
@@ -225,13 +227,13 @@ __device__ __forceinline__ void fom_march_record(const FomPass<T>& a, long long 
     const bool rec0 = n > 0 && n % a.r == 0;
     const bool rec1 = NS == 2 && (n + 1) % a.r == 0;
     if (!rec0 && !rec1) return;
-    const int Nt1 = a.Nt - 1, Nt2 = a.Nt - 2, M = a.M;
+    const int Nt1 = a.Nt - 1, Nt2 = a.Nt - 2, M = a.M, Mt = a.Mt;
     const T dt = (T)a.dt;
-    const long long tot = (long long)a.nrecv * M;
+    const long long tot = (long long)a.nrecv * Mt;
     const long long nthr = (long long)(gridDim.x - a.nmarch) * kFomThreads;
     const int tid = (int)(threadIdx.y * blockDim.x + threadIdx.x);
     for (long long idx = (long long)(blockIdx.x - a.nmarch) * kFomThreads + tid; idx < tot; idx += nthr) {
-        const int kk = (int)(idx / M), m = (int)(idx - (long long)kk * M);
+        const int kk = (int)(idx / Mt), m = (int)(idx - (long long)kk * Mt);
         const long long u = a.recv[kk];
         const T v = a.Vo[u * M + m];
         if (rec0) a.traces[(n / a.r - 1) * tot + idx] = v;
@@ -408,7 +410,7 @@ __global__ void __launch_bounds__(kFomThreads, fom_occupancy<NS>()) fom_march_ke
             if (src_col && i == a.src_i && m0 < M) {
 #pragma unroll
                 for (int q = 0; q < VW; ++q)
-                    vn[q] = fom_src(vn[q], (T)(a.dt / a.rho), a.wavelet, n0 + n, a.dt, a.Tper[m0 + q]);
+                    vn[q] = fom_src(vn[q], (T)(a.dt / a.rho), a.wavelet, n0 + n, a.dt, a.Tper[min(m0 + q, a.Mt - 1)]);
             }
             fom_store<T, VW>(rb + self, vn);
             // the face below row i (of the first row: not used, or face 0, whose factors are 0)
@@ -422,7 +424,7 @@ __global__ void __launch_bounds__(kFomThreads, fom_occupancy<NS>()) fom_march_ke
                 if (src_col && i - 1 == a.src_i && m0 < M) {
 #pragma unroll
                     for (int q = 0; q < VW; ++q)
-                        w[q] = fom_src(w[q], (T)(a.dt / a.rho), a.wavelet, n0 + n + 1, a.dt, a.Tper[m0 + q]);
+                        w[q] = fom_src(w[q], (T)(a.dt / a.rho), a.wavelet, n0 + n + 1, a.dt, a.Tper[min(m0 + q, a.Mt - 1)]);
                 }
                 fom_store<T, VW>(rb + rstep + self, w);
             }
@@ -541,12 +543,26 @@ __global__ void fom_advance_kernel(FomCtl* ctl, int steps) { ctl->step = ctl->st
 template <typename T>
 __global__ void __launch_bounds__(kFomThreads) fom_last_record_kernel(const T* __restrict__ V,
                                                                       const int* __restrict__ recv, int nrecv,
-                                                                      int M, T* __restrict__ out) {
-    const long long tot = (long long)nrecv * M;
+                                                                      int M, int Mt, T* __restrict__ out) {
+    const long long tot = (long long)nrecv * Mt;
     for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < tot;
          idx += (long long)gridDim.x * blockDim.x) {
-        const int kk = (int)(idx / M), m = (int)(idx - (long long)kk * M);
+        const int kk = (int)(idx / Mt), m = (int)(idx - (long long)kk * Mt);
         out[idx] = V[(long long)recv[kk] * M + m];
+    }
+}
+
+// Rows of M values to rows of Mp >= M (zeros beyond) or back, n rows.
+template <bool IN>
+__global__ void __launch_bounds__(kFomThreads) fom_pad_kernel(const float* __restrict__ src, long long n, int M,
+                                                              int Mp, float* __restrict__ dst) {
+    const int w = IN ? Mp : M;
+    const long long tot = n * w;
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < tot;
+         i += (long long)gridDim.x * blockDim.x) {
+        const long long k = i / w;
+        const int m = (int)(i - k * w);
+        dst[i] = m < M ? src[k * (IN ? M : Mp) + m] : 0.f;
     }
 }
 
@@ -590,9 +606,9 @@ struct FomShape {
     int bx, by;
 };
 template <typename T>
-FomShape fom_shape(int M, std::initializer_list<const void*> bufs) {
+FomShape fom_shape(int M, std::initializer_list<const void*> bufs, bool allow_wide = true) {
     constexpr int VWIDE = 16 / (int)sizeof(T);
-    FomShape s{M % VWIDE == 0, 1, 0};
+    FomShape s{allow_wide && M % VWIDE == 0, 1, 0};
     for (const void* p : bufs) s.wide = s.wide && ((uintptr_t)p % 16 == 0);
     const int vw = s.wide ? VWIDE : 1;
     while (s.bx * vw < M && s.bx < 32) s.bx *= 2;
@@ -639,7 +655,7 @@ cudaError_t launch_march(FomPass<T> a, const FomShape& s, int nsm, cudaStream_t 
     const int nstrip = (a.Nt - 1 + TJ - 1) / TJ;
     a.seg_rows = fom_seg_rows<NS>(a.Nr, nstrip, nsm);
     a.nmarch = nstrip * ((a.Nr + a.seg_rows - 1) / a.seg_rows);
-    const unsigned grid = (unsigned)a.nmarch + (a.traces ? fom_blocks((long long)a.nrecv * a.M) : 0u);
+    const unsigned grid = (unsigned)a.nmarch + (a.traces ? fom_blocks((long long)a.nrecv * a.Mt) : 0u);
     const dim3 blk(s.bx, s.by, 1);
     const size_t smem = ((size_t)(2 * NS + 4 * fom_stages<NS>()) * kFomThreads * (s.wide ? VWIDE : 1) +
                          (size_t)8 * (a.seg_rows + NS + 3)) * sizeof(T);
@@ -741,7 +757,25 @@ struct FomRun {
     long n0;
     int src, wavelet, nrecv, r;
     bool fused;
+    int Mp;             // realizations per row of the fused form's buffers: M, or padded
+    void *Vp, *S1p, *S2p;  // padded: the first buffer set (V2, S12, S22 are the second)
 };
+
+// Should a thread of the fused FP32 form take 4 realizations with 16-byte
+// accesses (n unknowns)?  One realization a thread shortens the chain of a row
+// while the grid does not fill the GPU; with more, it is bound by its scalar
+// accesses and, above 16 realizations, by the strips that 32 lanes along m
+// leave.  us a step, one / four (padded to a multiple of 4): 512 x 2048
+// M = 2 9.0 / 11.6, 3 16.1 / 11.7, 9 66 / 33, 17 154 / 59, 33 304 / 119;
+// 256 x 1024 M = 3 5.8 / 6.8, 5 9.2 / 8.0; 128 x 512 M = 9 6.3 / 6.5,
+// 13 6.3 / 6.3, 17 13.0 / 7.9; 64 x 256 M = 15 3.6 / 4.7, 26 5.1 / 5.6,
+// 33 8.9 / 6.6; 40 x 100 M = 5 2.5 / 4.4, 33 5.0 / 4.7.
+bool fom_wide(long long n, int M) {
+    return M > 32 || (M >= 3 && n * M >= (M > 16 ? 1500000 : 2500000));
+}
+// A run of that kind whose M is not a multiple of 4 marches on copies padded to
+// one, except for a few steps, which the copies would cost as much as.
+bool fom_padded(long long n, int M, int nsteps) { return M % 4 != 0 && nsteps >= 16 && fom_wide(n, M); }
 
 // The graph of a run's buffers and arguments, captured on its first use.
 template <typename F>
@@ -768,9 +802,12 @@ cudaError_t run_fom(rom_fom_s* f, const FomRun& q, cudaStream_t st) {
     const size_t nv = (size_t)f->Nr * (f->Nt - 1), n1 = (size_t)(f->Nr - 1) * (f->Nt - 1),
                  n2 = (size_t)f->Nr * (f->Nt - 2);
     const int nsm = fom_sm_count();
-    const FomShape s = fom_shape<T>(q.M, {q.V, q.S1, q.S2, q.V2, q.S12, q.S22});
-    const std::vector<long long> key = {(long long)(uintptr_t)q.V, (long long)(uintptr_t)q.S1,
-                                        (long long)(uintptr_t)q.S2, q.M, q.src, (long long)(uintptr_t)q.T,
+    const bool pad = q.Mp != q.M;
+    void *V = pad ? q.Vp : q.V, *S1 = pad ? q.S1p : q.S1, *S2 = pad ? q.S2p : q.S2;
+    const FomShape s = fom_shape<T>(q.Mp, {V, S1, S2, q.V2, q.S12, q.S22},
+                                    !q.fused || sizeof(T) == 8 || fom_wide((long long)(nv + n1 + n2), q.M));
+    const std::vector<long long> key = {(long long)(uintptr_t)V, (long long)(uintptr_t)S1,
+                                        (long long)(uintptr_t)S2, q.M, q.Mp, q.src, (long long)(uintptr_t)q.T,
                                         q.wavelet, (long long)(uintptr_t)q.recv, q.nrecv, q.traces ? q.r : 0,
                                         (long long)(uintptr_t)q.traces, (long long)sizeof(T), q.fused,
                                         (long long)(uintptr_t)q.V2};
@@ -790,17 +827,34 @@ cudaError_t run_fom(rom_fom_s* f, const FomRun& q, cudaStream_t st) {
     }
     FomPass<T> a{};
     a.tb = tables_of<T>(f);
-    a.Vo = static_cast<T*>(q.V), a.S1o = static_cast<T*>(q.S1), a.S2o = static_cast<T*>(q.S2);
+    a.Vo = static_cast<T*>(V), a.S1o = static_cast<T*>(S1), a.S2o = static_cast<T*>(S2);
     a.Vn = static_cast<T*>(q.V2), a.S1n = static_cast<T*>(q.S12), a.S2n = static_cast<T*>(q.S22);
     a.Tper = static_cast<const T*>(q.T);
     a.recv = q.recv;
     a.traces = static_cast<T*>(q.traces);
     a.n0 = q.n0;
-    a.Nr = f->Nr, a.Nt = f->Nt, a.M = q.M;
+    a.Nr = f->Nr, a.Nt = f->Nt, a.M = q.Mp, a.Mt = q.M;
     a.nrecv = q.nrecv, a.r = q.r, a.wavelet = q.wavelet;
     a.src_i = q.src >= 0 ? q.src / (f->Nt - 1) : -1;
     a.src_j = q.src >= 0 ? q.src % (f->Nt - 1) + 1 : -1;
     a.dt = f->dt, a.rho = f->rho;
+    auto copies = [&](bool in, void* v, void* s1, void* s2) {
+        const std::pair<void*, size_t> user[3] = {{q.V, nv}, {q.S1, n1}, {q.S2, n2}};
+        void* own[3] = {v, s1, s2};
+        for (int i = 0; i < 3; ++i) {
+            const long long n = (long long)user[i].second;
+            const long long b = (n * q.Mp + kFomThreads - 1) / kFomThreads;
+            const unsigned grid = (unsigned)(b < 8LL * nsm ? b : 8LL * nsm);
+            float *u = static_cast<float*>(user[i].first), *p = static_cast<float*>(own[i]);
+            if (in) fom_pad_kernel<true><<<grid, kFomThreads, 0, st>>>(u, n, q.M, q.Mp, p);
+            else fom_pad_kernel<false><<<grid, kFomThreads, 0, st>>>(p, n, q.M, q.Mp, u);
+        }
+        return cudaGetLastError();
+    };
+    if (pad) {
+        e = copies(true, V, S1, S2);
+        if (e != cudaSuccess) return e;
+    }
     // whole groups of kFomGraphSteps steps by graph, the rest launched
     const int reps = q.nsteps / kFomGraphSteps;
     if (reps > 0) {
@@ -815,7 +869,10 @@ cudaError_t run_fom(rom_fom_s* f, const FomRun& q, cudaStream_t st) {
     bool odd = false;
     a.off = (long long)reps * kFomGraphSteps;
     if (e == cudaSuccess) e = march_steps<T>(a, s, nsm, q.nsteps - reps * kFomGraphSteps, st, &odd);
-    if (e == cudaSuccess && odd) {
+    const T* Vend = static_cast<const T*>(odd ? q.V2 : V);
+    if (e == cudaSuccess && pad) {
+        e = copies(false, odd ? q.V2 : V, odd ? q.S12 : S1, odd ? q.S22 : S2);
+    } else if (e == cudaSuccess && odd) {
         e = cudaMemcpyAsync(q.V, q.V2, nv * q.M * sizeof(T), cudaMemcpyDeviceToDevice, st);
         if (e == cudaSuccess) e = cudaMemcpyAsync(q.S1, q.S12, n1 * q.M * sizeof(T), cudaMemcpyDeviceToDevice, st);
         if (e == cudaSuccess) e = cudaMemcpyAsync(q.S2, q.S22, n2 * q.M * sizeof(T), cudaMemcpyDeviceToDevice, st);
@@ -823,7 +880,7 @@ cudaError_t run_fom(rom_fom_s* f, const FomRun& q, cudaStream_t st) {
     if (e == cudaSuccess && a.traces && q.nsteps % q.r == 0) {
         // a pass records the velocity it finds: the last step's record is left
         fom_last_record_kernel<T><<<fom_blocks((long long)q.nrecv * q.M), kFomThreads, 0, st>>>(
-            static_cast<const T*>(q.V), q.recv, q.nrecv, q.M,
+            Vend, q.recv, q.nrecv, q.Mp, q.M,
             a.traces + (size_t)(q.nsteps / q.r - 1) * q.nrecv * q.M);
         e = cudaGetLastError();
     }
@@ -957,7 +1014,18 @@ rom_status rom_fom_run(rom_fom_t f, void* V, void* S1, void* S2, int M, int nste
     // the fused pass writes every other step into a second buffer set
     const bool fused = f->passes == 1;
     const size_t es = prec == ROM_FP64 ? 8 : 4;
-    const size_t need = (size_t)(nv + ns) * (size_t)M * es + 64;
+    bool pad = fused && prec == ROM_FP32 && fom_padded(nv + ns, M, nsteps);
+    auto al = [](size_t b) { return (b + 255) & ~(size_t)255; };
+    int Mp = 0;
+    size_t bV = 0, b1 = 0, set = 0, need = 0;
+    auto layout = [&]() {
+        Mp = pad ? (M + 3) / 4 * 4 : M;
+        bV = al((size_t)nv * Mp * es);
+        b1 = al((size_t)(f->Nr - 1) * (f->Nt - 1) * Mp * es);
+        set = bV + b1 + al((size_t)f->Nr * (f->Nt - 2) * Mp * es);
+        need = pad ? 2 * set : set;
+    };
+    layout();
     if (fused && f->ws_bytes < need) {
         cudaStreamSynchronize(st);
         cudaDeviceSynchronize();
@@ -967,6 +1035,12 @@ rom_status rom_fom_run(rom_fom_t f, void* V, void* S1, void* S2, int M, int nste
         f->ws = nullptr;
         f->ws_bytes = 0;
         cudaError_t em = cudaMalloc(&f->ws, need);
+        if (em == cudaErrorMemoryAllocation && pad) {  // no room for the copies: march in place
+            cudaGetLastError();
+            pad = false;
+            layout();
+            em = cudaMalloc(&f->ws, need);
+        }
         if (em != cudaSuccess) {
             set_last_error(cudaGetErrorString(em));
             return em == cudaErrorMemoryAllocation ? ROM_E_NOMEM : ROM_E_CUDA;
@@ -974,31 +1048,12 @@ rom_status rom_fom_run(rom_fom_t f, void* V, void* S1, void* S2, int M, int nste
         f->ws_bytes = need;
     }
     char* w = static_cast<char*>(f->ws);
-    auto al = [](size_t b) { return (b + 255) & ~(size_t)255; };
-    void* V2 = fused ? w : nullptr;
-    void* S12 = fused ? w + al((size_t)nv * M * es) : nullptr;
-    void* S22 = fused ? w + al((size_t)nv * M * es) + al((size_t)(f->Nr - 1) * (f->Nt - 1) * M * es) : nullptr;
-    if (fused && (size_t)((char*)S22 - w) + (size_t)f->Nr * (f->Nt - 2) * M * es > f->ws_bytes) {
-        // the aligned layout needs a little more than `need`: grow once more
-        cudaDeviceSynchronize();
-        for (auto& kv : f->graphs) cudaGraphExecDestroy(kv.second);
-        f->graphs.clear();
-        cudaFree(f->ws);
-        f->ws_bytes = 0;
-        const size_t need2 = need + 1024;
-        cudaError_t em = cudaMalloc(&f->ws, need2);
-        if (em != cudaSuccess) {
-            f->ws = nullptr;
-            set_last_error(cudaGetErrorString(em));
-            return em == cudaErrorMemoryAllocation ? ROM_E_NOMEM : ROM_E_CUDA;
-        }
-        f->ws_bytes = need2;
-        w = static_cast<char*>(f->ws);
-        V2 = w;
-        S12 = w + al((size_t)nv * M * es);
-        S22 = w + al((size_t)nv * M * es) + al((size_t)(f->Nr - 1) * (f->Nt - 1) * M * es);
+    FomRun q{V, S1, S2, nullptr, nullptr, nullptr, T, recv, traces, M, nsteps, n0, src, wavelet, nrecv,
+             traces ? r : 1, fused, Mp, nullptr, nullptr, nullptr};
+    if (fused) {
+        q.V2 = w, q.S12 = w + bV, q.S22 = w + bV + b1;
+        if (pad) q.Vp = w + set, q.S1p = w + set + bV, q.S2p = w + set + bV + b1;
     }
-    FomRun q{V, S1, S2, V2, S12, S22, T, recv, traces, M, nsteps, n0, src, wavelet, nrecv, traces ? r : 1, fused};
     const cudaError_t e = prec == ROM_FP64 ? run_fom<double>(f, q, st) : run_fom<float>(f, q, st);
     if (e != cudaSuccess) {
         set_last_error(cudaGetErrorString(e));

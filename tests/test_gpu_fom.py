@@ -196,6 +196,23 @@ def test_fom_fused_bitwise_two_passes(rom, Nr, Nt, M, nsteps):
             assert np.array_equal(x, y)
 
 
+# padded marches (M = 17, 33 and, large enough, 3 and 7) with an even and an odd
+# number of passes, and with and without whole groups of 64 steps
+@pytest.mark.parametrize("Nr,Nt,M,nsteps", [(20, 30, 33, 16), (9, 40, 37, 83), (90, 340, 17, 65), (300, 950, 3, 18),
+                                            (200, 600, 7, 17)])
+def test_fom_padded_bitwise_two_passes(rom, Nr, Nt, M, nsteps):
+    f = rom.Fom(Nr, Nt, dt=0.01)
+    X0 = case(Nr, Nt, M, seed=Nr + nsteps)
+    T = np.linspace(60.0, 80.0, M)
+    for src, r in ((0, 1), (f.nv // 2, 2), (f.nv - 1, 4)):
+        outs = []
+        for passes in (1, 2):
+            f.set_passes(passes)
+            outs.append(gpu_run(rom, f, X0, nsteps, "fp32", src=src, T=T, n0=7000, r=r, recv=[0, src, f.nv - 1]))
+        for x, y in zip(*outs):
+            assert np.array_equal(x, y)
+
+
 def test_fom_rejects_bad_arguments(rom):
     f = rom.Fom(8, 12)
     V, S1, S2 = f.new_state(2)
