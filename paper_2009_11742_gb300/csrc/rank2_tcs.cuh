@@ -94,7 +94,7 @@ __host__ __device__ inline size_t tcs_smem_bytes(int W, int stages) {
     size_t o = 1024;                                    // alignment slack
     o += (size_t)stages * tcs_stage_bytes(W);
     o += 8 * (2 * stages + 2);                          // full[], empty[], dready, drain
-    o += 32;                                            // tmem slot, flags, chunk counter
+    o += 64;                                            // tmem slot, flags, chunk counter, every CTA's abort flag
     o += (size_t)W * 4 * 4;                             // fcol, Tcol, xsc, xinv
     o += (size_t)kTcRows * 4 * 3;                       // g rows, row scales of Avs and Asv
     o += (size_t)4 * W * 4;                             // column maxima per TMEM quadrant
@@ -267,11 +267,11 @@ __global__ void __launch_bounds__(kTcsThreads, 1) rank2_tcs_kernel(const TcArgs 
     uint32_t* tslot = reinterpret_cast<uint32_t*>(drain + 1);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tslot + 1);
     volatile int* abort_all = reinterpret_cast<volatile int*>(tslot + 2);
-    // abort flag as published for the cluster-wide decision: written between
-    // the two barriers of a half-step, where no wait can change abort_flag
-    volatile int* abort_pub = reinterpret_cast<volatile int*>(tslot + 3);
     long long* consumed = reinterpret_cast<long long*>(tslot + 4);
-    float* fcol = reinterpret_cast<float*>(tslot + 8);
+    // every CTA's abort flag, stored here by its owner with the column maxima:
+    // a half-step's waits are over by then, and the first barrier publishes it
+    int* abort_in = reinterpret_cast<int*>(tslot + 8);  // [kTcsMaxCS]
+    float* fcol = reinterpret_cast<float*>(tslot + 8 + kTcsMaxCS);
     float* Tcol = fcol + W;
     float* xsc = Tcol + W;                          // 2^(eX_j - 7) of the current B operand
     float* xinv = xsc + W;                          // 2^(7 - eX_j)
@@ -287,7 +287,7 @@ __global__ void __launch_bounds__(kTcsThreads, 1) rank2_tcs_kernel(const TcArgs 
     if (tid == 0) {
         *abort_flag = 0;
         *abort_all = 0;
-        *abort_pub = 0;
+        for (int q = 0; q < kTcsMaxCS; ++q) abort_in[q] = 0;
         for (int s = 0; s < STAGES; ++s) { mbarrier_init(&full[s], 1); mbarrier_init(&empty[s], 1); }
         mbarrier_init(dready, 1);
         mbarrier_init(drain, 1);
@@ -588,8 +588,17 @@ __global__ void __launch_bounds__(kTcsThreads, 1) rank2_tcs_kernel(const TcArgs 
                     for (int q = 0; q < CS; ++q)
                         *cluster.map_shared_rank(gmax + crank * W + ridx, q) = __uint_as_float(bm);
                 }
+                if (ridx == kTcsThreads - 1) {
+                    const int ab = *abort_flag;
+                    for (int q = 0; q < CS; ++q) *cluster.map_shared_rank(abort_in + crank, q) = ab;
+                }
             }
             cluster.sync();
+            if (tid == kTcsThreads - 1) {  // the same decision in every CTA
+                int any = 0;
+                for (int q = 0; q < CS; ++q) any |= abort_in[q];
+                *abort_all = any;
+            }
             // ---- column exponents of the new state (the B operand of the next half-step)
             for (int j = tid; j < W; j += kTcsThreads) {
                 float mx = 0.f;
@@ -643,20 +652,9 @@ __global__ void __launch_bounds__(kTcsThreads, 1) rank2_tcs_kernel(const TcArgs 
                     fcol[c] = f;
                 }
             }
-            if (tid == 0) *abort_pub = *abort_flag;
             tc_fence_before();
             cluster.sync();
             tc_fence_after();
-            // cluster-uniform abort decision from the published flags
-            if (tid == 0) {
-                int any = 0;
-                for (int q = 0; q < CS; ++q) {
-                    const int* pf = cluster.map_shared_rank(const_cast<int*>(abort_pub), q);
-                    any |= *reinterpret_cast<volatile const int*>(pf);
-                }
-                *abort_all = any;
-            }
-            __syncthreads();
             if (*abort_all) break;
             // ---- receiver traces of V^{n+1} (after the velocity half is published)
             if (tr_step && !chip_step) {
