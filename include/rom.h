@@ -169,7 +169,7 @@ rom_status rom_get_plan(rom_t h, int prec, int M, int* variant, int* cluster_siz
  *                   when the two-block kernel already uses every cluster
  *                   that fits, it narrows the column blocks and hands the
  *                   freed columns to the companion if that is predicted to
- *                   be at least 5 % faster;
+ *                   be at least 3 % faster;
  *   cluster_size -1 never;
  *   cluster_size 2 or 4: always, with `columns` (>= 1) columns on the
  *                   companion (all of them when columns >= M).
