@@ -297,10 +297,12 @@ __device__ __forceinline__ void fom_cp_async(T* dst, const T* src, int src_bytes
 // the halo's extra work would be a loss.
 template <typename T, int VW, int NS>
 __global__ void __launch_bounds__(kFomThreads, fom_occupancy<NS>()) fom_march_kernel(const FomPass<T> a) {
-    const long long n = a.off + (a.ctl ? a.ctl->step : 0);
-    const long long n0 = a.ctl ? a.ctl->n0 : a.n0;
+    // the next pass's blocks may take their places as this pass's leave them;
+    // like these, they read nothing that a pass writes before the wait below
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if ((int)blockIdx.x >= a.nmarch) {
-        fom_march_record<T, NS>(a, n, n0);
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        fom_march_record<T, NS>(a, a.off + (a.ctl ? a.ctl->step : 0), a.ctl ? a.ctl->n0 : a.n0);
         return;
     }
     constexpr int LH = NS - 1;                    // halo columns on the left
@@ -346,6 +348,10 @@ __global__ void __launch_bounds__(kFomThreads, fom_occupancy<NS>()) fom_march_ke
         e[4] = in ? a.tb.q_u[i] : T(0);
         e[5] = in ? a.tb.q_d[i] : T(0);
     }
+    // the last pass has ended and its writes are visible
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const long long n = a.off + (a.ctl ? a.ctl->step : 0);
+    const long long n0 = a.ctl ? a.ctl->n0 : a.n0;
     const int chunk = (int)blockDim.x * VW;
     const size_t rv = (size_t)Nt1 * M, r2 = (size_t)Nt2 * M;  // elements per row
     for (int mb = 0; mb < M; mb += chunk) {       // same trip count in every thread
@@ -661,9 +667,26 @@ cudaError_t launch_march(FomPass<T> a, const FomShape& s, int nsm, cudaStream_t 
                          (size_t)8 * (a.seg_rows + NS + 3)) * sizeof(T);
     const void* fn = s.wide ? (const void*)fom_march_kernel<T, VWIDE, NS> : (const void*)fom_march_kernel<T, 1, NS>;
     if (smem > 48 * 1024) cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (s.wide) fom_march_kernel<T, VWIDE, NS><<<grid, blk, smem, st>>>(a);
-    else fom_march_kernel<T, 1, NS><<<grid, blk, smem, st>>>(a);
-    return cudaGetLastError();
+    // An FP32 pass may start before the last one has ended: its launch, and what
+    // it does before it needs the state, are then hidden (us a step, M = 1:
+    // 512 x 2048 6.0 -> 5.7, 40 x 100 2.45 -> 2.12; M = 2, 128 x 512 3.1 -> 2.5).
+    // Blocks that come early take whichever SM has room, which costs more than
+    // that where the SMs' load matters and the grid leaves some idle (FP64
+    // 40 x 100, M = 16 8.6 -> 14; FP32 with four realizations a thread there,
+    // M = 33 4.7 -> 5.0).
+    const bool early = sizeof(T) == 4 && (!s.wide || a.nmarch >= nsm * fom_occupancy<NS>());
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = blk;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = early ? 1 : 0;
+    void* args[] = {(void*)&a};
+    return cudaLaunchKernelExC(&cfg, fn, args);
 }
 
 // Passes over `count` steps from step a.off on, two steps a pass in FP32.
