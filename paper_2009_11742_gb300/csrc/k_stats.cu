@@ -6,7 +6,7 @@
 // statistics of the Hyndman-Fan type 7 quantiles off it.
 //
 // Bound: the ALU pipe, by the network's min / max (45 steps of 16 elements a
-// lane at M = 512).  1000 records x 64 receivers x 512 realizations: 200 us
+// lane at M = 512).  1000 records x 64 receivers x 512 realizations: 180 us
 // against 774 us for one block per column with a shared-memory bitonic network
 // behind 45 block barriers, whose reads took 4 bytes of every sector; the
 // traces alone are 20 us of HBM traffic.  FP64 is kept out of the columns'
@@ -142,9 +142,16 @@ __device__ __forceinline__ void stat_exchange(int (&x)[EPL], int* xb, int wcol, 
     }
 }
 
+// Resident blocks an SM: as many as the tiles leave shared memory for hide the
+// chains of the network's steps (1000 x 64 x M = 512 217 us without a bound on
+// the registers, 198 with 6 blocks, 209 with 7; 500 x 64 x 1000 265, 208 with 4,
+// 218 with 5).
+template <int EPL, int W>
+__host__ __device__ constexpr int stat_blocks() { return EPL <= 16 ? 6 : (W == 1 ? 4 : 2); }
+
 // EPL values a lane, W warps a column (W > 1: EPL = 32).
 template <int EPL, int W>
-__global__ void __launch_bounds__(kStatThreads) trace_stats_kernel(const StatArgs a) {
+__global__ void __launch_bounds__(kStatThreads, stat_blocks<EPL, W>()) trace_stats_kernel(const StatArgs a) {
     static_assert(W == 1 || EPL == 32, "wide columns hold 1024 values a warp");
     constexpr int B = EPL * 32 * W <= 512 ? 21 : 18;
     extern __shared__ __align__(16) unsigned char smem[];
