@@ -115,7 +115,7 @@ struct rom_s {
     // caller's stream and join it back
     int comp_cs = 0, comp_cols = 0;
     cudaStream_t aux = nullptr;
-    cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
+    cudaEvent_t ev_fork = nullptr, ev_placed = nullptr, ev_join = nullptr;
 };
 
 namespace {
@@ -144,6 +144,7 @@ void free_handle(rom_s* h) {
         cudaFree(h->xref[t][1]);
     }
     if (h->ev_fork) cudaEventDestroy(h->ev_fork);
+    if (h->ev_placed) cudaEventDestroy(h->ev_placed);
     if (h->ev_join) cudaEventDestroy(h->ev_join);
     if (h->aux) cudaStreamDestroy(h->aux);
     delete h;
@@ -634,16 +635,19 @@ rom_status launch_simt_with_plan(rom_s* h, const RunBufs& b, int M, int nsteps, 
 // forked after the work already queued on the caller's stream and joined
 // back before anything queued after this call.  The split kernel's large
 // clusters must be placed before the companion's small ones, or one of them
-// waits for a whole run: the companion is released by an event that the split
-// kernel's last block to start records (when all of its clusters fit at once;
-// K = 512, M = 256, 1000 steps queued back to back: 9.47 ms each, 10.0 to
-// 10.6 ms with the companion only issued second).  In a stream capture the
-// two are parallel nodes.
+// waits for a whole run: outside a stream capture, and when all of the split
+// kernel's clusters fit at once, the companion also waits for an event that
+// their last block to start records (K = 512, M = 256, 1000 steps queued back
+// to back: 9.47 ms each, 10.0 to 10.6 ms with the companion only issued
+// second).  That event decides placement alone: CUDA documents it as best
+// effort, so what the companion reads and writes is ordered by the fork.  In a
+// capture the two are parallel nodes.
 rom_status launch_with_companion(rom_s* h, const Rank2Args& a, const Rank2Plan& plan, cudaStream_t st) {
     cudaError_t e = cudaSuccess;
     if (!h->aux) {
         e = cudaStreamCreateWithFlags(&h->aux, cudaStreamNonBlocking);
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming);
+        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_placed, cudaEventDisableTiming);
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_join, cudaEventDisableTiming);
         if (e != cudaSuccess) return cuda_fail(e, "companion stream");
     }
@@ -655,11 +659,12 @@ rom_status launch_with_companion(rom_s* h, const Rank2Args& a, const Rank2Plan& 
     ac.M = mc;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     e = cudaStreamIsCapturing(st, &cap);
-    const bool started = e == cudaSuccess && cap == cudaStreamCaptureStatusNone && am.M > 0 &&
-                         plan.nclusters <= plan.max_active_clusters;
-    if (e == cudaSuccess && !started) e = cudaEventRecord(h->ev_fork, st);
-    if (e == cudaSuccess && am.M > 0) e = launch_rank2_split_f32(am, plan, st, started ? h->ev_fork : nullptr);
+    const bool placed = e == cudaSuccess && cap == cudaStreamCaptureStatusNone && am.M > 0 &&
+                        plan.nclusters <= plan.max_active_clusters;
+    if (e == cudaSuccess) e = cudaEventRecord(h->ev_fork, st);
+    if (e == cudaSuccess && am.M > 0) e = launch_rank2_split_f32(am, plan, st, placed ? h->ev_placed : nullptr);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(h->aux, h->ev_fork, 0);
+    if (e == cudaSuccess && placed) e = cudaStreamWaitEvent(h->aux, h->ev_placed, 0);
     if (e == cudaSuccess) e = launch_rank2_stream_f32(ac, plan.comp_cs, plan.comp_W, plan.comp_n, h->aux);
     if (e == cudaSuccess) e = cudaEventRecord(h->ev_join, h->aux);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(st, h->ev_join, 0);

@@ -167,6 +167,39 @@ def test_companion_headline_workload_sampled(rom):
     assert colmax_rel(tr[:, :, cols], tro) <= 1e-4
 
 
+@pytest.mark.parametrize("csz", [2, 4])
+def test_companion_after_slow_writers_on_the_stream(rom, csz):
+    """What earlier work on the caller's stream writes (V, S, periods, traces)
+    late is what the companion reads, and what it writes is there for later
+    work: bit for bit a run between synchronizations."""
+    Kv, M, N, r = 512, 32, 60, 5
+    p = inputs.make_problem(Kv, Kv, M, 8, seed=23)
+    h = rom.Rom.from_problem(p)
+    h.set_companion(csz, 8)
+    assert h.plan(M)["variant"] == 4
+    V0 = inputs.random_state(Kv, M, seed=1, scale=0.1)
+    S0 = inputs.random_state(Kv, M, seed=2, scale=0.1)
+    Va, Sa, tra = run(rom, h, p, V0, S0, N, r=r)
+    dV, dS = rom.Rom.new_state(Kv, M, "fp32", fill=V0), rom.Rom.new_state(Kv, M, "fp32", fill=S0)
+    dT = torch.as_tensor(p.T, dtype=torch.float32, device="cuda")
+    V, S, T = torch.full_like(dV, 7.0), torch.full_like(dS, 7.0), torch.full_like(dT, 1.0)
+    tr = torch.full((N // r, M, p.R), 3.0, device="cuda")
+    st = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    outs = []
+    with torch.cuda.stream(st):
+        for _ in range(3):
+            torch.cuda._sleep(20_000_000)  # about 10 ms
+            V.copy_(dV), S.copy_(dS), T.copy_(dT), tr.zero_()
+            h.run_rank2(V, S, T, N, r=r, traces=tr, prec="fp32")
+            outs.append((V.clone(), S.clone(), tr.clone()))
+    torch.cuda.synchronize()
+    assert h.sync_status() == 0
+    for Vb, Sb, trb in outs:
+        assert np.array_equal(Va, Vb.cpu().numpy()) and np.array_equal(Sa, Sb.cpu().numpy())
+        assert np.array_equal(tra, trb.transpose(1, 2).cpu().numpy())
+
+
 def test_set_companion_rejects_bad_arguments(rom):
     p = inputs.make_problem(64, 64, 4, 0, seed=1)
     h = rom.Rom.from_problem(p)
