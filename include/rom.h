@@ -264,8 +264,8 @@ rom_status rom_set_wait_limit(rom_t h, long long cycles);
 /*
  * rom_debug_inject_stall -- failure injection for tests of the timeout path:
  * when on, one CTA of every cluster of a kernel with asynchronous exchange
- * (two-block, one-block in its asynchronous form) never publishes
- * its rows, so its peers' waits run out (set a small wait limit first).  The
+ * (two-block, its companion, one-block in its asynchronous form) never
+ * publishes its rows, so its peers' waits run out (set a small wait limit first).  The
  * kernel then ends with ROM_E_TIMEOUT instead of hanging.  Off by default.
  */
 rom_status rom_debug_inject_stall(rom_t h, int on);

@@ -153,6 +153,7 @@ __global__ void __launch_bounds__(kStrThreads, 1) rank2_stream_kernel(const Rank
     const int p8 = lane & 7, kqs = (r0 >> 2) + 2 * warp + (p8 >> 2);
     const int src_lane = 16 * (p8 >> 2) + ((p8 & 3) ^ Lay::swz(kqs));
     const int peer = lane >> 3;
+    const int npeer = a.debug_skip_push && crank == 0 ? 0 : CSZ;  // fault injection: this CTA sends nothing
     const unsigned base = smem_addr(smem);
     const unsigned dpeer = cluster_addr(base, peer < CSZ ? peer : 0) - base;
     const unsigned piece = (unsigned)(kqs * Lay::U + (p8 & 3)) * 16u;
@@ -316,7 +317,7 @@ __global__ void __launch_bounds__(kStrThreads, 1) rank2_stream_kernel(const Rank
                     float u[4];
 #pragma unroll
                     for (int r = 0; r < 4; ++r) u[r] = __shfl_sync(0xffffffffu, y, src_lane + 4 * r);
-                    if (peer < CSZ)
+                    if (peer < npeer)
                         asm volatile(
                             "st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];"
                             ::"r"(base + (unsigned)(h ? L.Sf : L.Vf) + piece + (unsigned)(p * (kStrRows / 4) * Lay::U * 16) +
@@ -330,11 +331,11 @@ __global__ void __launch_bounds__(kStrThreads, 1) rank2_stream_kernel(const Rank
         if (!dead && warp < NW) halves = 2 * ne;
     }
     // the last S has arrived, too
-    if (!dead && N > 0 && warp < NW && !*abort_flag)
+    if (!dead && N > 0 && warp < NW)
         dead = !__all_sync(0xffffffffu, mbar_wait_bounded(&mbar[1], (unsigned)((N - 1) & 1), a.spin_limit, abort_flag));
     if (dead && lane == 0) *abort_flag = 1;
     // ---- drain, as in the split kernel
-    if (lane == 0) {
+    if (lane == 0 && npeer > 0) {
         int np = 0;  // this warp's passes per half-step
         for (int p = 0; p < NP; ++p) np += quad_in(p) ? 1 : 0;
         atomicAdd(&sent_out[0], kPassBytes * (unsigned)(np * ((halves + 1) / 2)));

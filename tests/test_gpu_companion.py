@@ -200,6 +200,32 @@ def test_companion_after_slow_writers_on_the_stream(rom, csz):
         assert np.array_equal(tra, trb.transpose(1, 2).cpu().numpy())
 
 
+# one, partial and several passes a CTA, a run shorter than the forcing table and
+# one that ends inside the second; every column on the companion, so that it alone stalls
+@pytest.mark.parametrize("csz", [2, 4])
+@pytest.mark.parametrize("Kv,M,N", [(192, 5, 20), (256, 6, 45), (448, 9, 45), (512, 4, 1)])
+def test_companion_wait_limit(rom, csz, Kv, M, N):
+    """A CTA of the companion that sends nothing: the waits run out, the run
+    ends with a status, and the next run on the handle is right."""
+    p = inputs.make_problem(Kv, Kv, M, 4, seed=20)
+    h = rom.Rom.from_problem(p)
+    h.set_companion(csz, M)
+    plan = h.plan(M)
+    assert plan["variant"] == 4 and plan["companion"]["columns"] == M
+    V0 = inputs.random_state(Kv, M, seed=1, scale=0.1)
+    T = torch.as_tensor(p.T, dtype=torch.float32, device="cuda")
+    assert rom.rom_set_wait_limit(h.h, 2_000_000) == rom.ROM_OK  # about 1 ms
+    assert rom.rom_debug_inject_stall(h.h, 1) == rom.ROM_OK
+    V, S = rom.Rom.new_state(Kv, M, "fp32", fill=V0), rom.Rom.new_state(Kv, M, "fp32", fill=V0)
+    h.run_rank2(V, S, T, N, prec="fp32")
+    assert h.sync_status() == rom.ROM_E_TIMEOUT
+    assert rom.rom_debug_inject_stall(h.h, 0) == rom.ROM_OK
+    assert rom.rom_set_wait_limit(h.h, 4_000_000_000) == rom.ROM_OK
+    V, S, _ = run(rom, h, p, V0, V0, N)
+    Vo, So, _ = oracle.forward(p.Avs, p.Asv, p.g, None, p.dt, V0, V0, N, T=p.T)
+    assert colmax_rel(V, Vo) <= 1e-4 and colmax_rel(S, So) <= 1e-4
+
+
 def test_set_companion_rejects_bad_arguments(rom):
     p = inputs.make_problem(64, 64, 4, 0, seed=1)
     h = rom.Rom.from_problem(p)
