@@ -252,8 +252,8 @@ rom_status rom_set_tc_columns(rom_t h, int cols);
 /*
  * rom_set_wait_limit -- bound, in SM clock cycles, on every device-side wait
  * of the kernels with asynchronous exchange (a consumer waiting for a
- * producer's rows: two-block, its companion, and one-block in its asynchronous
- * form) and of the
+ * producer's rows: two-block, its companion, one-block in its asynchronous
+ * form, and rom_adjoint's FP32 reverse kernel up to Kp = 512) and of the
  * tensor-core kernels (stage and accumulator handshakes).  A wait that
  * runs out makes the kernel stop, leave cleanly, and record ROM_E_TIMEOUT in
  * the handle's status word (rom_sync_status).  Default
@@ -264,9 +264,9 @@ rom_status rom_set_wait_limit(rom_t h, long long cycles);
 /*
  * rom_debug_inject_stall -- failure injection for tests of the timeout path:
  * when on, one CTA of every cluster of a kernel with asynchronous exchange
- * (two-block, its companion, one-block in its asynchronous form) never
- * publishes its rows, so its peers' waits run out (set a small wait limit first).  The
- * kernel then ends with ROM_E_TIMEOUT instead of hanging.  Off by default.
+ * (two-block, its companion, one-block in its asynchronous form, the FP32
+ * reverse kernel up to Kp = 512) never publishes its rows, so its peers'
+ * waits run out (set a small wait limit first).  The kernel then ends with ROM_E_TIMEOUT instead of hanging.  Off by default.
  */
 rom_status rom_debug_inject_stall(rom_t h, int on);
 

@@ -445,7 +445,8 @@ __global__ void __launch_bounds__(kThreads, 1) rank2_adjoint_split_kernel(const 
     }
     float op[4][4 * KI];
     load_op_quad<KI>(op, vrole ? a.opA_rm : a.opB_rm, Kp, row0 + 4 * q, j);
-    const SplitLink<KI> link(smem_addr(smem), (unsigned)L.X, (unsigned)L.mbar, row0, warp, lane, peer0, H);
+    const bool sends = !(a.debug_skip_push && crank == 0);  // fault injection: this CTA sends nothing
+    const SplitLink<KI> link(smem_addr(smem), (unsigned)L.X, (unsigned)L.mbar, row0, warp, lane, peer0, sends ? H : 0);
     // this lane's element of C^T r at step n (every row of src is Kp wide)
     const int own_row = row0 + 4 * q + (j >> 2);
     auto source = [&](int k, int g) {
@@ -531,7 +532,7 @@ __global__ void __launch_bounds__(kThreads, 1) rank2_adjoint_split_kernel(const 
     if (vrole && !dead && nsent == N && N > 0)
         for (int g = 0; g < G && !dead; ++g) dead = !wait(g, (unsigned)((N - 1) & 1));
     if (dead && lane == 0) *abort_flag = 1;
-    split_drain<KI>(cluster, mbar, sent_out, sent_in, Gmax, G, N, vrole, sl, peer0, nsent, gsent, true, abort_flag,
+    split_drain<KI>(cluster, mbar, sent_out, sent_in, Gmax, G, N, vrole, sl, peer0, nsent, gsent, sends, abort_flag,
                     a.status);
 
     // ---- write back the owned rows, carries and the period-gradient partials

@@ -2026,6 +2026,7 @@ rom_status adjoint_run(rom_s* h, const void* V0, const void* S0, const void* Tp,
         aa.dt = h->dt;
         aa.wavelet = h->wavelet;
         aa.spin_limit = h->wait_limit;
+        aa.debug_skip_push = h->inject_stall;
         aa.n0 = 0;
         aa.n_lo = n_start;
         aa.n_hi = n_start + len;

@@ -224,6 +224,7 @@ struct AdjArgsT {
     int nrt;              // 32-row tiles the layout holds per CTA (FP32 above Kp = 512)
     int wavelet;          // source signal of the periods (see Rank2Args)
     long long spin_limit; // see Rank2Args (the split-role kernel)
+    int debug_skip_push;  // likewise
 };
 using AdjArgs = AdjArgsT<float>;
 struct AdjPlan {

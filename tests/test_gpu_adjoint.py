@@ -407,3 +407,26 @@ def test_adjoint_allocation_failure_is_reported(rom):
     loss, gV2, gS2, gT2 = gpu_adjoint(rom, h, p, V0, S0, ystar, 10, 0)
     Lo, gVo, _, _ = oracle.adjoint(p.Avs, p.Asv, p.g, p.C, p.dt, V0, S0, p.T, 10, ystar)
     assert abs(loss - Lo) <= 1e-4 * abs(Lo) and rel(gV2, gVo) <= 1e-4
+
+
+# Kp <= 128: the forward sweep runs the one-CTA kernel, which waits for nobody, so the
+# reverse kernel alone stalls (one and several column groups, ranges shorter and longer
+# than its table of 32 steps); K = 256: the forward kernels' waits run out as well
+@pytest.mark.parametrize("Kv,M,N,ckpt", [(64, 3, 20, 0), (100, 400, 45, 0), (128, 300, 40, 16), (256, 12, 30, 0)])
+def test_adjoint_wait_limit(rom, Kv, M, N, ckpt):
+    """A CTA that sends nothing: the waits run out, the call ends with a status,
+    and the next call on the handle is right."""
+    p, V0, S0, ystar = case(Kv, Kv, M, 3, N, seed=77)
+    h = rom.Rom.from_problem(p)
+    ys = torch.as_tensor(np.ascontiguousarray(np.transpose(ystar, (0, 2, 1))), device="cuda")
+    assert rom.rom_set_wait_limit(h.h, 2_000_000) == rom.ROM_OK  # about 1 ms
+    assert rom.rom_debug_inject_stall(h.h, 1) == rom.ROM_OK
+    rom.adjoint(h, rom.Rom.new_state(Kv, M, "fp32", fill=V0), rom.Rom.new_state(Kv, M, "fp32", fill=S0),
+                torch.as_tensor(p.T, device="cuda"), ys, N, ckpt_every=ckpt)
+    assert h.sync_status() == rom.ROM_E_TIMEOUT
+    assert rom.rom_debug_inject_stall(h.h, 0) == rom.ROM_OK
+    assert rom.rom_set_wait_limit(h.h, 4_000_000_000) == rom.ROM_OK
+    loss, gV, gS, gT = gpu_adjoint(rom, h, p, V0, S0, ystar, N, ckpt)
+    lo, gVo, gSo, gTo = oracle.adjoint(p.Avs, p.Asv, p.g, p.C, p.dt, V0, S0, p.T, N, ystar)
+    assert abs(loss - lo) <= 1e-4 * lo
+    assert rel(gV, gVo) <= 1e-4 and rel(gS, gSo) <= 1e-4 and rel(gT, gTo) <= 1e-4
