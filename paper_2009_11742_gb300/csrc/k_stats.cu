@@ -167,17 +167,23 @@ __global__ void __launch_bounds__(kStatThreads, stat_blocks<EPL, W>()) trace_sta
     const int k0 = (int)(blockIdx.x / ntj) * a.nr, j0 = (int)(blockIdx.x % ntj) * a.nj;
     const int nr = min(a.nr, a.nrec - k0), nj = min(a.nj, a.R - j0);
     const int nc = nr * nj;                        // column c = rr nj + jj
-    // ---- the tile: consecutive threads on consecutive receivers
+    // ---- the tile: consecutive threads on consecutive receivers, all records
+    // in one loop (the rows of a record follow those of the last)
     {
         int lg = 0;
         while ((1 << lg) < nj) ++lg;
         const int jj = tid & ((1 << lg) - 1), step = kStatThreads >> lg;
-        for (int rr = 0; rr < nr; ++rr) {
-            const float* src = a.traces + (size_t)(k0 + rr) * M * a.R + j0 + jj;
-            if (jj < nj) {
+        const float* src = a.traces + (size_t)k0 * M * a.R + j0 + jj;
+        const int nrow = jj < nj ? nr * M : 0;
+        int m = tid >> lg, c = jj;                 // row of the record, column of the tile
 #pragma unroll 4
-                for (int m = tid >> lg; m < M; m += step) tile[m * TS + rr * nj + jj] = src[(size_t)m * a.R];
+        for (int p = tid >> lg; p < nrow; p += step) {
+            if (m >= M) {
+                c += m / M * nj;
+                m %= M;
             }
+            tile[m * TS + c] = src[(size_t)p * a.R];
+            m += step;
         }
     }
     __syncthreads();
@@ -290,6 +296,39 @@ __global__ void __launch_bounds__(kStatThreads, stat_blocks<EPL, W>()) trace_sta
     }
 }
 
+// Columns per tile.  16 keep 6 blocks on an SM at M = 512.  With too few
+// columns for the GPU's resident blocks a tile has fewer: first down to one turn
+// of the block's warps, then to as few as give every tile an SM of its own (a
+// turn takes as long for one column as for a warp each, but two one-column
+// blocks on an SM may share a scheduler: 300 columns of M = 1000 in 200 blocks
+// 18.8 us, in 100 below 15).  us a call with one receiver, tiles of 8 to 32
+// columns whatever their number / these / one block a column: M = 256, 100
+// records 20.7 / 12.6 / 14.3, M = 512, 100 records 18.5 / 12.6 / 14.5, M = 4000,
+// 10 records 53.5 / 16.8 / 37.2 (about 12.5 is the host's part).
+static void stat_tiles(StatArgs& a, int W, long long* nblk) {
+    int dev = 0, nsm = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    const int res = a.M <= 512 ? stat_blocks<16, 1>() : (W == 1 ? stat_blocks<32, 1>() : stat_blocks<32, 2>());
+    // receivers of one record, evenly, or with few of them several records
+    auto cut = [&](int G) {
+        a.G = G;
+        a.nj = (a.R + G - 1) / G;
+        a.nj = (a.R + a.nj - 1) / a.nj;
+        a.nr = G / a.nj;
+        *nblk = ((long long)(a.nrec + a.nr - 1) / a.nr) * ((a.R + a.nj - 1) / a.nj);
+    };
+    int G = a.M <= 256 ? 32 : (a.M <= 512 ? 16 : 8);
+    while (G > kStatWarps / W && (long long)a.nrec * a.R < (long long)G * nsm * res) G /= 2;
+    cut(G);
+    while (G > 1) {
+        cut(G / 2);
+        if (*nblk > nsm) break;
+        G /= 2;
+    }
+    cut(G);
+}
+
 static bool device_pointer(const void* p) {
     cudaPointerAttributes at{};
     if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
@@ -329,12 +368,9 @@ extern "C" rom_status rom_trace_stats(const float* traces, int nrec, int R, int 
         a.lo[i] = lo;
         a.t[i] = h - (double)lo;
     }
-    // 16 columns a tile keep 6 blocks on an SM at M = 512; with few receivers
-    // a tile takes several records
-    a.G = M <= 256 ? 32 : (M <= 512 ? 16 : 8);
-    a.nj = R < a.G ? R : a.G;
-    a.nr = a.G / a.nj;
-    const long long nblk = ((long long)(nrec + a.nr - 1) / a.nr) * ((R + a.nj - 1) / a.nj);
+    const int W = M <= 1024 ? 1 : (M <= 2048 ? 2 : 4);
+    long long nblk = 0;
+    stat_tiles(a, W, &nblk);
     if ((long long)nrec * R > 0x7fffffffLL) return ROM_E_INVAL;
     const void* fn = M <= 32     ? (const void*)trace_stats_kernel<1, 1>
                      : M <= 64   ? (const void*)trace_stats_kernel<2, 1>
@@ -344,7 +380,7 @@ extern "C" rom_status rom_trace_stats(const float* traces, int nrec, int R, int 
                      : M <= 1024 ? (const void*)trace_stats_kernel<32, 1>
                      : M <= 2048 ? (const void*)trace_stats_kernel<32, 2>
                                  : (const void*)trace_stats_kernel<32, 4>;
-    const size_t smem = stat_smem_layout(M, a.G, nprobs, M <= 1024 ? 1 : (M <= 2048 ? 2 : 4)).total;
+    const size_t smem = stat_smem_layout(M, a.G, nprobs, W).total;
     cudaError_t e = cudaSuccess;
     if (smem > 48 * 1024) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e == cudaSuccess) {

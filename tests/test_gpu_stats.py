@@ -57,6 +57,16 @@ def test_stats_sort_widths(rom, M, R):
     check(rom, x.astype(np.float32))
 
 
+# enough columns for tiles of 32, 16, 8 and 4 of them (fewer: above), several turns
+# of the block's warps a tile, one and several records a tile, uneven last tiles
+@pytest.mark.parametrize("nrec,M,R", [(600, 40, 50), (1001, 40, 30), (300, 40, 50), (5001, 20, 3), (31, 40, 50),
+                                      (20, 200, 33), (300, 300, 50), (41, 700, 30), (50, 1500, 49), (41, 1500, 30),
+                                      (50, 3000, 49), (41, 3000, 31), (1300, 600, 1), (200, 3, 7)])
+def test_stats_tile_shapes(rom, nrec, M, R):
+    rng = np.random.default_rng(nrec)
+    check(rom, rng.standard_normal((nrec, M, R), dtype=np.float32))
+
+
 def test_stats_extreme_scales(rom):
     """All-zero, denormal and largest-magnitude columns, and columns with an
     infinity (kept in order; their mean is not finite)."""
