@@ -580,7 +580,10 @@ rom_status rom_fom_destroy(rom_fom_t f);
  * run that needs it, sized by M), two steps per pass in FP32 (4 bytes per
  * unknown, realization and step), one in FP64 (16 bytes); 2: a velocity pass
  * then a stress pass in place (12 bytes in FP32).  The values agree bit for
- * bit in FP32.  ROM_E_INVAL for another value. */
+ * bit in FP32.  Wide FP32 runs of 16 or more steps whose M is not a multiple
+ * of 4 march on copies with padded rows, for which the library owns a third
+ * set of the second's size; without memory for it they march in place, with
+ * the same values.  ROM_E_INVAL for another value. */
 rom_status rom_fom_set_passes(rom_fom_t f, int passes);
 
 /* Unknowns per realization: velocity Nr (Ntheta - 1), sigma_rp
@@ -600,7 +603,9 @@ rom_status rom_fom_dims(rom_fom_t f, int* nv, int* n1, int* n2);
  * Every 64 steps are one launch of a CUDA graph, captured on the first call
  * for a given set of buffers and arguments and replayed; the fused form
  * launches the remaining steps one pass at a time.  Asynchronous on
- * `stream` (the first fused run allocates the second buffer set).  A handle is not re-entrant across concurrent streams.  Errors:
+ * `stream`, but for a fused run that needs larger buffer sets than any before
+ * it: it waits for the device and allocates them (and the first padded run the
+ * third).  A handle is not re-entrant across concurrent streams.  Errors:
  * ROM_E_INVAL (host buffers, bad indices), ROM_E_UNSUPPORTED (prec other than
  * ROM_FP32 / ROM_FP64), ROM_E_CUDA.
  */

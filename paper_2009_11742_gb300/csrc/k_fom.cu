@@ -592,8 +592,10 @@ struct rom_fom_s {
     std::mutex mu;
     std::map<std::vector<long long>, cudaGraphExec_t> graphs;
     int passes = 1;          // 1: fused single pass (default), 2: velocity and stress passes
-    void* ws = nullptr;      // second state buffer set of the fused pass
+    void* ws = nullptr;      // second state buffer set of the fused form
     size_t ws_bytes = 0;
+    void* pad = nullptr;     // first buffer set of padded runs: ws_bytes, or not there
+    bool no_pad = false;     // there was no memory for it beside this ws
 };
 
 namespace {
@@ -797,8 +799,53 @@ bool fom_wide(long long n, int M) {
     return M > 32 || (M >= 3 && n * M >= (M > 16 ? 1500000 : 2500000));
 }
 // A run of that kind whose M is not a multiple of 4 marches on copies padded to
-// one, except for a few steps, which the copies would cost as much as.
+// one, except for a few steps, which the copies would cost as much as, and where
+// there is no memory for the copies.
 bool fom_padded(long long n, int M, int nsteps) { return M % 4 != 0 && nsteps >= 16 && fom_wide(n, M); }
+
+// The buffers of the fused form for sets of `need` bytes.  They grow to `want`
+// (rows of a multiple of 16 bytes, so that a padded run asks for no more than a
+// run of its M) where there is room.
+cudaError_t fom_grow(rom_fom_s* f, size_t need, size_t want, cudaStream_t st) {
+    if (f->ws_bytes >= need) return cudaSuccess;
+    cudaStreamSynchronize(st);
+    cudaDeviceSynchronize();
+    for (auto& kv : f->graphs) cudaGraphExecDestroy(kv.second);
+    f->graphs.clear();
+    cudaFree(f->ws);
+    cudaFree(f->pad);
+    f->ws = f->pad = nullptr;
+    f->ws_bytes = 0;
+    f->no_pad = false;
+    cudaError_t e = cudaMalloc(&f->ws, want);
+    if (e == cudaErrorMemoryAllocation && want > need) {
+        cudaGetLastError();
+        want = need;
+        e = cudaMalloc(&f->ws, want);
+    }
+    if (e == cudaSuccess) f->ws_bytes = want;
+    return e;
+}
+
+// Are there copies for a padded run with sets of `bytes`?  They have the size of
+// the second set, whatever this run needs: so they are allocated once for it,
+// and no later run frees what a caller's graph may hold.  Not allocated in a
+// stream capture; a failure is remembered.
+bool fom_pad_buffers(rom_fom_s* f, size_t bytes, cudaStream_t st) {
+    if (f->ws_bytes < bytes || f->no_pad) return false;
+    if (f->pad) return true;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        return false;
+    }
+    const cudaError_t e = cudaMalloc(&f->pad, f->ws_bytes);
+    if (e == cudaSuccess) return true;
+    cudaGetLastError();
+    f->pad = nullptr;
+    f->no_pad = e == cudaErrorMemoryAllocation;
+    return false;
+}
 
 // The graph of a run's buffers and arguments, captured on its first use.
 template <typename F>
@@ -989,6 +1036,7 @@ rom_status rom_fom_destroy(rom_fom_t f) {
     cudaFree(f->tables[1]);
     cudaFree(f->ctl);
     cudaFree(f->ws);
+    cudaFree(f->pad);
     if (f->cap) cudaStreamDestroy(f->cap);
     delete f;
     return ROM_OK;
@@ -1037,45 +1085,30 @@ rom_status rom_fom_run(rom_fom_t f, void* V, void* S1, void* S2, int M, int nste
     // the fused pass writes every other step into a second buffer set
     const bool fused = f->passes == 1;
     const size_t es = prec == ROM_FP64 ? 8 : 4;
-    bool pad = fused && prec == ROM_FP32 && fom_padded(nv + ns, M, nsteps);
     auto al = [](size_t b) { return (b + 255) & ~(size_t)255; };
-    int Mp = 0;
-    size_t bV = 0, b1 = 0, set = 0, need = 0;
-    auto layout = [&]() {
-        Mp = pad ? (M + 3) / 4 * 4 : M;
-        bV = al((size_t)nv * Mp * es);
-        b1 = al((size_t)(f->Nr - 1) * (f->Nt - 1) * Mp * es);
-        set = bV + b1 + al((size_t)f->Nr * (f->Nt - 2) * Mp * es);
-        need = pad ? 2 * set : set;
+    const long long n1 = (long long)(f->Nr - 1) * (f->Nt - 1), n2 = (long long)f->Nr * (f->Nt - 2);
+    auto set_bytes = [&](long long m) {
+        return al((size_t)(nv * m) * es) + al((size_t)(n1 * m) * es) + al((size_t)(n2 * m) * es);
     };
-    layout();
-    if (fused && f->ws_bytes < need) {
-        cudaStreamSynchronize(st);
-        cudaDeviceSynchronize();
-        for (auto& kv : f->graphs) cudaGraphExecDestroy(kv.second);
-        f->graphs.clear();
-        cudaFree(f->ws);
-        f->ws = nullptr;
-        f->ws_bytes = 0;
-        cudaError_t em = cudaMalloc(&f->ws, need);
-        if (em == cudaErrorMemoryAllocation && pad) {  // no room for the copies: march in place
-            cudaGetLastError();
-            pad = false;
-            layout();
-            em = cudaMalloc(&f->ws, need);
-        }
+    const long long per = 16 / (long long)es, Mw = (M + per - 1) / per * per;
+    bool pad = false;
+    if (fused) {
+        const cudaError_t em = fom_grow(f, set_bytes(M), set_bytes(Mw), st);
         if (em != cudaSuccess) {
             set_last_error(cudaGetErrorString(em));
             return em == cudaErrorMemoryAllocation ? ROM_E_NOMEM : ROM_E_CUDA;
         }
-        f->ws_bytes = need;
+        pad = prec == ROM_FP32 && fom_padded(nv + ns, M, nsteps) && fom_pad_buffers(f, set_bytes(Mw), st);
     }
-    char* w = static_cast<char*>(f->ws);
+    const int Mp = pad ? (int)Mw : M;
     FomRun q{V, S1, S2, nullptr, nullptr, nullptr, T, recv, traces, M, nsteps, n0, src, wavelet, nrecv,
              traces ? r : 1, fused, Mp, nullptr, nullptr, nullptr};
     if (fused) {
+        const size_t bV = al((size_t)(nv * Mp) * es), b1 = al((size_t)(n1 * Mp) * es);
+        char* w = static_cast<char*>(f->ws);
         q.V2 = w, q.S12 = w + bV, q.S22 = w + bV + b1;
-        if (pad) q.Vp = w + set, q.S1p = w + set + bV, q.S2p = w + set + bV + b1;
+        w = static_cast<char*>(f->pad);
+        if (pad) q.Vp = w, q.S1p = w + bV, q.S2p = w + bV + b1;
     }
     const cudaError_t e = prec == ROM_FP64 ? run_fom<double>(f, q, st) : run_fom<float>(f, q, st);
     if (e != cudaSuccess) {

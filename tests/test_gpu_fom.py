@@ -1,6 +1,8 @@
 """GPU parity of the rank-2 full-order model (rom_fom_*; Sec. 3, Eq.
 (fom_asym), App. A material) against the FP64 oracle (oracle/fom_oracle.c),
 run one realization at a time."""
+import time
+
 import numpy as np
 import pytest
 
@@ -211,6 +213,68 @@ def test_fom_padded_bitwise_two_passes(rom, Nr, Nt, M, nsteps):
             outs.append(gpu_run(rom, f, X0, nsteps, "fp32", src=src, T=T, n0=7000, r=r, recv=[0, src, f.nv - 1]))
         for x, y in zip(*outs):
             assert np.array_equal(x, y)
+
+
+def on_device(X0):
+    return [torch.as_tensor(np.ascontiguousarray(x), dtype=torch.float32, device="cuda") for x in X0]
+
+
+# widths that march in place and ones that would be padded
+@pytest.mark.parametrize("Nr,Nt,M,nsteps", [(20, 30, 32, 30), (40, 100, 1, 33), (90, 340, 17, 50), (9, 40, 37, 16)])
+def test_fom_in_a_stream_capture(rom, Nr, Nt, M, nsteps):
+    """A run of less than 64 steps whose buffer set is there from an earlier run
+    of at least its width can be captured, and a later run of no larger width
+    leaves what the graph holds alone: replays equal a plain run bit for bit."""
+    T = torch.linspace(60.0, 80.0, M, device="cuda")
+    X0 = case(Nr, Nt, M, seed=3)
+    ref = gpu_run(rom, rom.Fom(Nr, Nt, dt=0.01), X0, nsteps, "fp32", src=2, T=T.cpu().numpy(), n0=7000, r=2,
+                  recv=[0, 2, 5])
+    f = rom.Fom(Nr, Nt, dt=0.01)
+    gpu_run(rom, f, case(Nr, Nt, 48, seed=4), 3, "fp32")  # the buffer set
+    V, S1, S2 = on_device(X0)
+    recv = torch.as_tensor(np.array([0, 2, 5], np.int32), device="cuda")
+    tr = torch.zeros((nsteps // 2, 3, M), device="cuda")
+    st, g = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=st):
+        f.run(V, S1, S2, nsteps, src=2, T=T, n0=7000, recv=recv, r=2, traces=tr)
+    for width in (48, 33, 3):
+        gpu_run(rom, f, case(Nr, Nt, width, seed=4), 70, "fp32")
+        for x, x0 in zip((V, S1, S2), on_device(X0)):
+            x.copy_(x0)
+        torch.cuda.synchronize()
+        g.replay()
+        torch.cuda.synchronize()
+        for a, b in zip(ref, (V, S1, S2, tr)):
+            assert np.array_equal(a, b.cpu().numpy())
+
+
+def test_fom_without_memory_for_the_padded_copies(rom):
+    """No room for a padded run's copies: it marches in place, with the same
+    bits, and the next call asks for nothing again and does not wait."""
+    Nr, Nt, M, nsteps = 512, 2048, 17, 66
+    f = rom.Fom(Nr, Nt, dt=0.01)
+    X0 = case(Nr, Nt, M, seed=3)
+    ref = gpu_run(rom, f, X0, nsteps, "fp32")
+    f = rom.Fom(Nr, Nt, dt=0.01)
+    V, S1, S2 = on_device(X0)
+    torch.cuda.empty_cache()
+    set_bytes = 4 * 20 * (f.nv + f.n1 + f.n2)
+    filler = torch.empty(torch.cuda.mem_get_info()[0] - set_bytes * 3 // 2, dtype=torch.uint8, device="cuda")
+    try:
+        f.run(V, S1, S2, nsteps)
+        torch.cuda.synchronize()
+        for a, b in zip(ref, (V, S1, S2)):
+            assert np.array_equal(a, b.cpu().numpy())
+        free = torch.cuda.mem_get_info()[0]
+        torch.cuda._sleep(200_000_000)  # about 100 ms
+        t0 = time.perf_counter()
+        f.run(V, S1, S2, nsteps)
+        assert time.perf_counter() - t0 < 0.05
+        torch.cuda.synchronize()
+        assert torch.cuda.mem_get_info()[0] == free
+    finally:
+        del filler
+        torch.cuda.empty_cache()
 
 
 def test_fom_rejects_bad_arguments(rom):
