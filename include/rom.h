@@ -397,7 +397,7 @@ rom_status rom_run_rank3(const rom_t* handles, int nops, void* V, void* S, const
  * tries the size thresholds 0 (every job BF16S), 256, 512 and none (every
  * job FP32), and with tensor-core jobs both the batch widths and the ones
  * the planner picks for a job alone; with ROM_FP32 it also times the
- * work-list form; it keeps the fastest combination.  *best_us (may be
+ * work-list forms, the one of an untuned call first; it keeps the fastest combination.  *best_us (may be
  * NULL) receives the chosen schedule's probe time per step.  Synchronous on
  * `stream`.  Errors as for rom_run_batched, plus ROM_E_NOMEM.
  */

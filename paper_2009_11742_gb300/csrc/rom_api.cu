@@ -1691,10 +1691,18 @@ rom_status rom_autotune_batched(const rom_job* jobs, int njobs, int prec, int pr
     double best = -1.0, best_scale = 1.0;
     int best_kthr = kAutoKthr, best_tcw = 1, best_wl = 0;
     rom_status rs = ROM_OK;
-    // FP32: work-list forms (clusters of 2 or 4 CTAs, width caps 8 / 16 /
-    // 32 / 64) besides one launch per job (0)
-    const int wls[9] = {kWlDefault, 2008, 2032, 2064, 4008, 4016, 4032, 4064, 0};
-    const int nwl = prec == ROM_FP32 ? 9 : 1;
+    // FP32: the form an untuned call takes, then work-list forms (clusters of 2
+    // or 4 CTAs, width caps 8 / 16 / 32 / 64) besides one launch per job (0)
+    std::vector<int> wls = {0};
+    if (prec == ROM_FP32) {
+        int dev = 0, nsm = 0;
+        if (e == cudaSuccess) e = cudaGetDevice(&dev);
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+        if (e == cudaSuccess) wls = {batched_default_form(jobs, njobs, dev, nsm)};
+        for (int wl : {2016, 2008, 2032, 2064, 4008, 4016, 4032, 4064, 0})
+            if (wl != wls[0]) wls.push_back(wl);
+    }
+    const int nwl = (int)wls.size();
     for (int iw = 0; iw < nwl && e == cudaSuccess && rs == ROM_OK; ++iw)
     for (int t = 0; t < nk && e == cudaSuccess && rs == ROM_OK; ++t) {
         const int wl = prec == ROM_FP32 ? wls[iw] : 0;
