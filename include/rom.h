@@ -125,8 +125,8 @@ rom_status rom_sync_status(rom_t h, rom_status* device_status);
 /* Model dimensions of a handle (any output may be NULL). */
 rom_status rom_get_dims(rom_t h, int* Kv, int* Ks, int* R, double* dt);
 
-/* Kernel selection for the rank-2 FP32 path (the FP64 path always uses the
- * one-block kernel):
+/* Kernel selection for the rank-2 FP32 path (FP64 and rank-1 runs have the
+ * one-block kernel alone and return ROM_E_UNSUPPORTED for the last two):
  *  ROM_KERNEL_AUTO      planner's choice (default: up to Kp = 128 one CTA per
  *                       column block, without clusters; above, one-block with
  *                       asynchronous exchange for up to 4 columns per

@@ -400,8 +400,8 @@ rom_status get_plan(rom_s* h, int prec, int M, bool rank1, Rank2Plan* plan) {
     // stay in registers, and FP32 blocks of few columns unless the caller
     // pinned a kernel or a companion (the same bits as the two-block kernel).
     const bool one_block_only = prec == ROM_FP64 || rank1;
-    const bool async_open = prec == ROM_FP64 || h->kernel_choice == ROM_KERNEL_AUTO ||
-                            (rank1 && h->kernel_choice == ROM_KERNEL_ONE_BLOCK);
+    const bool async_open = h->kernel_choice == ROM_KERNEL_AUTO ||
+                            (one_block_only && h->kernel_choice == ROM_KERNEL_ONE_BLOCK);
     if (!ok && async_open && (one_block_only || h->comp_cs <= 0)) {
         Rank2Plan pa{};
         ok = plan_rank2_async(h->Kp, M, h->R, prec == ROM_FP64, &pa) &&

@@ -82,3 +82,24 @@ def test_async_wait_limit(rom, Kv, M, prec):
     Z = np.zeros((Kv, M))
     Vo, _, _ = oracle.forward(p.Avs, p.Asv, p.g, None, p.dt, Z, Z, 100, T=p.T)
     assert status == rom.ROM_OK and np.linalg.norm(V - Vo) <= 1e-4 * np.linalg.norm(Vo)
+
+
+@pytest.mark.parametrize("K", [64, 256, 400])
+def test_fp64_and_rank1_refuse_a_two_block_pin(rom, K):
+    """FP64 and rank-1 runs have no two-block kernel, whatever their size."""
+    p = inputs.make_problem(K, K, 3, 0, seed=1)
+    h = rom.Rom.from_problem(p)
+    T = torch.as_tensor(p.T, dtype=torch.float64, device="cuda")
+    for kernel in (rom.ROM_KERNEL_AUTO, rom.ROM_KERNEL_ONE_BLOCK, rom.ROM_KERNEL_TWO_BLOCK, rom.ROM_KERNEL_DATAFLOW):
+        h.set_kernel(kernel)
+        pinned = kernel in (rom.ROM_KERNEL_TWO_BLOCK, rom.ROM_KERNEL_DATAFLOW)
+        V, S = rom.Rom.new_state(K, 3, "fp64"), rom.Rom.new_state(K, 3, "fp64")
+        v, s = torch.zeros(K, device="cuda"), torch.zeros(K, device="cuda")
+        for call in (lambda: h.run_rank2(V, S, T, 4, prec="fp64"), lambda: h.run_rank1(v, s, 30.0, 4)):
+            if pinned:
+                with pytest.raises(rom.RomError) as err:
+                    call()
+                assert err.value.status == rom.ROM_E_UNSUPPORTED
+            else:
+                call()
+        assert h.sync_status() == rom.ROM_OK
