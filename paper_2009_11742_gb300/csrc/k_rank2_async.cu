@@ -59,7 +59,6 @@ static bool plan_async(int Kp, int M, int R, Rank2Plan* p) {
     p->nrt = 1;
     p->resident = true;
     p->variant = 1;
-    p->async = true;
     const int rpc = (R + p->cs - 1) / p->cs;
     p->c_global = (size_t)rpc * Kp * sizeof(T) > 64 * 1024;
     const int nC = p->c_global ? 0 : rpc;
@@ -82,7 +81,8 @@ static bool plan_async(int Kp, int M, int R, Rank2Plan* p) {
     p->Wv = p->Wa = w;
     p->nclusters = (M + w - 1) / w;
     p->smem = bytes(w, p->cb);
-    return p->smem <= smax;
+    p->async = p->smem <= smax;
+    return p->async;
 }
 
 template <typename T>

@@ -865,7 +865,10 @@ rom_status rom_autotune(rom_t h, int prec, int M, int probe_steps, double* best_
         Rank2Plan p0;
         int nact = 0;
         if (h->Kp <= 128 && h->comp_cs <= 0 && plan_rank2_cta_f32(h->Kp, M, h->R, &p0)) simt.push_back(p0);
-        if (h->Kp > 128 && h->comp_cs <= 0 && plan_rank2_async(h->Kp, M, h->R, false, &p0)) simt.push_back(p0);
+        if (h->Kp > 128 && h->comp_cs <= 0 && plan_rank2_async(h->Kp, M, h->R, false, &p0) &&
+            async_beats_two_block(p0.Wa))
+            simt.push_back(p0);
+        p0.async = false;
         if (plan_rank2_split_f32(h->Kp, M, h->R, &p0)) nact = p0.max_active_clusters;
         else if (plan_rank2_simt_f32(h->Kp, M, h->R, false, &p0)) nact = p0.max_active_clusters;
         const int budgets[3] = {nact, nact / 2, nact / 4};
