@@ -62,6 +62,31 @@ def test_async_f64(rom, Kv, Ks, M):
             assert np.linalg.norm(a.cpu().numpy() - b) <= 1e-13 * np.linalg.norm(b)
 
 
+# wider blocks: several column groups of 1, 2 and 4 columns, ragged last clusters, and
+# (M = 1100) more clusters than fit at once
+@pytest.mark.parametrize("Kv,Ks,M,group", [(128, 128, 150, 1), (128, 120, 200, 2), (128, 128, 512, 4),
+                                           (256, 256, 269, 2), (200, 256, 300, 4), (256, 250, 1100, 4),
+                                           (60, 64, 500, 4), (64, 64, 380, 1)])
+def test_async_f64_several_groups(rom, Kv, Ks, M, group):
+    N, r, R = 9, 2, 7
+    p = inputs.make_problem(Kv, Ks, M, R, seed=M)
+    h = rom.Rom.from_problem(p)
+    W = h.plan(M, "fp64")["cols_per_block"]
+    # the planner's blocks are a multiple of 4, 2 or 1 columns for groups of as many
+    assert W > group and {0: 4, 2: 2}.get(W % 4, 1) == group
+    V0, S0 = inputs.random_state(Kv, M, seed=1, scale=0.1), inputs.random_state(Ks, M, seed=2, scale=0.1)
+    V, S = rom.Rom.new_state(Kv, M, "fp64", fill=V0), rom.Rom.new_state(Ks, M, "fp64", fill=S0)
+    tr = torch.zeros((N // r, M, R), dtype=torch.float64, device="cuda")
+    h.run_rank2(V, S, torch.as_tensor(p.T, dtype=torch.float64, device="cuda"), N, r=r, traces=tr, prec="fp64")
+    assert h.sync_status() == rom.ROM_OK
+    Vo, So, tro = oracle.forward(p.Avs, p.Asv, p.g, p.C, p.dt, V0, S0, N, T=p.T, r=r)
+    for a, b in ((V, Vo), (S, So), (tr.transpose(1, 2), tro)):
+        a = a.cpu().numpy()
+        # column by column; as above, with 9 steps
+        num, den = np.linalg.norm(a - b, axis=-2), np.linalg.norm(b, axis=-2)
+        assert np.all(num <= 1e-13 * den)
+
+
 @pytest.mark.parametrize("Kv,M,prec", [(512, 20, "fp32"), (128, 16, "fp64")])
 def test_async_wait_limit(rom, Kv, M, prec):
     """Waits that run out end the kernel with a status; the context stays usable."""
