@@ -193,13 +193,14 @@ rom_status rom_get_companion(rom_t h, int M, int* cluster_size, int* nclusters, 
  * rom_run_rank2_ex calls with the same precision and M use it while the
  * kernel choice (rom_set_kernel) and the tensor-core width
  * (rom_set_tc_columns) are automatic.  Candidates:
- *   ROM_FP32  the one-CTA kernel (up to Kp = 128); the two-block and the one-block kernels, each with the cluster
- *             count capped at the co-resident maximum, half and a quarter of
- *             it (wider column blocks on fewer clusters); and, when the
- *             two-block kernel fills every cluster that fits, the same with
- *             4, 8 or 12 fewer columns per block and the freed columns on the
- *             streaming companion (rom_set_companion) in clusters of 2 or 4;
- *   ROM_FP64  the one-block kernel;
+ *   ROM_FP32  the untuned plan; the two-block and the one-block kernels, each
+ *             with the cluster count capped at the co-resident maximum, half
+ *             and a quarter of it (wider column blocks on fewer clusters);
+ *             and, when the two-block kernel fills every cluster that fits,
+ *             the same with 4, 8 or 12 fewer columns per block and the freed
+ *             columns on the streaming companion (rom_set_companion) in
+ *             clusters of 2 or 4;
+ *   ROM_FP64  the untuned plan;
  *   tensor-core precisions: every column-block width the precision provides.
  * Every candidate computes the same leapfrog; the FP32 kernels differ only in
  * the order of FP32 roundings (results agree to FP32 rounding).

@@ -371,6 +371,53 @@ struct RunBufs {
     void *V, *S, *T, *ftab, *compV, *compS, *traces;
 };
 
+// The planner's plan for a kernel choice (under the handle's lock).
+bool choose_plan(const rom_s* h, int prec, int M, bool rank1, int choice, Rank2Plan* plan) {
+    bool ok = false;
+    // FP32 with more than one realization: the two-block split-role kernel,
+    // unless the caller pinned the one-block kernel.
+    const bool two_block = prec != ROM_FP64 && !rank1 && choice != ROM_KERNEL_ONE_BLOCK;
+    // Small models run one CTA per column block unless the caller pinned a
+    // cluster kernel or a companion: no cluster barrier in the step, the same
+    // bits (see rank2_cta.cuh for both sides' times).
+    if (prec != ROM_FP64 && h->Kp <= 128 && choice == ROM_KERNEL_AUTO && h->comp_cs <= 0)
+        ok = plan_rank2_cta_f32(h->Kp, M, h->R, plan);
+    // The asynchronous one-block kernel: FP64 and rank-1 runs whose operators
+    // stay in registers, and FP32 blocks of few columns unless the caller
+    // pinned a kernel or a companion (the same bits as the two-block kernel).
+    const bool one_block_only = prec == ROM_FP64 || rank1;
+    const bool async_open = choice == ROM_KERNEL_AUTO ||
+                            (one_block_only && choice == ROM_KERNEL_ONE_BLOCK);
+    if (!ok && async_open && (one_block_only || h->comp_cs <= 0)) {
+        Rank2Plan pa{};
+        ok = plan_rank2_async(h->Kp, M, h->R, prec == ROM_FP64, &pa) &&
+             (one_block_only || async_beats_two_block(pa.Wa));
+        if (ok) *plan = pa;
+    }
+    if (!ok && two_block && choice == ROM_KERNEL_DATAFLOW) {
+        ok = plan_rank2_split_f32(h->Kp, M, h->R, plan);
+        plan->variant = 3;
+    } else if (!ok && two_block) {
+        ok = plan_rank2_split_f32(h->Kp, M, h->R, plan);
+        // the streaming companion on the SMs the split kernel's clusters
+        // leave idle (automatic kernel choice only)
+        if (ok && choice == ROM_KERNEL_AUTO) {
+            Rank2Plan cp;
+            if (h->comp_cs == 0 && plan_rank2_companion(h->Kp, M, h->R, &cp)) *plan = cp;
+            else if ((h->comp_cs == 2 || h->comp_cs == 4) &&
+                     plan_rank2_companion_pinned(h->Kp, M, h->R, h->comp_cs,
+                                                 h->comp_cols < M ? h->comp_cols : M, &cp))
+                *plan = cp;
+        }
+    }
+    if (!ok && choice != ROM_KERNEL_TWO_BLOCK && choice != ROM_KERNEL_DATAFLOW) {
+        ok = prec == ROM_FP64 ? plan_rank2_simt_f64(h->Kp, M, h->R, rank1, plan)
+                              : plan_rank2_simt_f32(h->Kp, M, h->R, rank1, plan);
+        if (ok) plan->variant = 1;
+    }
+    return ok;
+}
+
 rom_status get_plan(rom_s* h, int prec, int M, bool rank1, Rank2Plan* plan) {
     std::lock_guard<std::mutex> lk(h->mu);
     if (!rank1 && h->kernel_choice == ROM_KERNEL_AUTO) {
@@ -387,49 +434,7 @@ rom_status get_plan(rom_s* h, int prec, int M, bool rank1, Rank2Plan* plan) {
         *plan = it->second;
         return ROM_OK;
     }
-    bool ok = false;
-    // FP32 with more than one realization: the two-block split-role kernel,
-    // unless the caller pinned the one-block kernel.
-    const bool two_block = prec != ROM_FP64 && !rank1 && h->kernel_choice != ROM_KERNEL_ONE_BLOCK;
-    // Small models run one CTA per column block unless the caller pinned a
-    // cluster kernel or a companion: no cluster barrier in the step, the same
-    // bits (see rank2_cta.cuh for both sides' times).
-    if (prec != ROM_FP64 && h->Kp <= 128 && h->kernel_choice == ROM_KERNEL_AUTO && h->comp_cs <= 0)
-        ok = plan_rank2_cta_f32(h->Kp, M, h->R, plan);
-    // The asynchronous one-block kernel: FP64 and rank-1 runs whose operators
-    // stay in registers, and FP32 blocks of few columns unless the caller
-    // pinned a kernel or a companion (the same bits as the two-block kernel).
-    const bool one_block_only = prec == ROM_FP64 || rank1;
-    const bool async_open = h->kernel_choice == ROM_KERNEL_AUTO ||
-                            (one_block_only && h->kernel_choice == ROM_KERNEL_ONE_BLOCK);
-    if (!ok && async_open && (one_block_only || h->comp_cs <= 0)) {
-        Rank2Plan pa{};
-        ok = plan_rank2_async(h->Kp, M, h->R, prec == ROM_FP64, &pa) &&
-             (one_block_only || async_beats_two_block(pa.Wa));
-        if (ok) *plan = pa;
-    }
-    if (!ok && two_block && h->kernel_choice == ROM_KERNEL_DATAFLOW) {
-        ok = plan_rank2_split_f32(h->Kp, M, h->R, plan);
-        plan->variant = 3;
-    } else if (!ok && two_block) {
-        ok = plan_rank2_split_f32(h->Kp, M, h->R, plan);
-        // the streaming companion on the SMs the split kernel's clusters
-        // leave idle (automatic kernel choice only)
-        if (ok && h->kernel_choice == ROM_KERNEL_AUTO) {
-            Rank2Plan cp;
-            if (h->comp_cs == 0 && plan_rank2_companion(h->Kp, M, h->R, &cp)) *plan = cp;
-            else if ((h->comp_cs == 2 || h->comp_cs == 4) &&
-                     plan_rank2_companion_pinned(h->Kp, M, h->R, h->comp_cs,
-                                                 h->comp_cols < M ? h->comp_cols : M, &cp))
-                *plan = cp;
-        }
-    }
-    if (!ok && h->kernel_choice != ROM_KERNEL_TWO_BLOCK && h->kernel_choice != ROM_KERNEL_DATAFLOW) {
-        ok = prec == ROM_FP64 ? plan_rank2_simt_f64(h->Kp, M, h->R, rank1, plan)
-                              : plan_rank2_simt_f32(h->Kp, M, h->R, rank1, plan);
-        if (ok) plan->variant = 1;
-    }
-    if (!ok) {
+    if (!choose_plan(h, prec, M, rank1, h->kernel_choice, plan)) {
         snprintf(g_last_error, sizeof(g_last_error),
                  "no SIMT rank-2 plan for Kp=%d M=%d (prec %d)", h->Kp, M, prec);
         return ROM_E_UNSUPPORTED;
@@ -857,18 +862,15 @@ rom_status rom_autotune(rom_t h, int prec, int M, int probe_steps, double* best_
             TcPlan p;
             if (plan_rank2_tc(prec, h->Kp_tc, M, h->R, ws[i], &p)) tcp.push_back(p);
         }
-    } else if (f64) {
-        Rank2Plan p;
-        if (plan_rank2_async(h->Kp, M, h->R, true, &p)) simt.push_back(p);
-        else if (plan_rank2_simt_f64(h->Kp, M, h->R, false, &p)) { p.variant = 1; simt.push_back(p); }
     } else {
-        Rank2Plan p0;
+        // the untuned plan
+        std::lock_guard<std::mutex> lk(h->mu);
+        Rank2Plan p{};
+        if (choose_plan(h, prec, M, false, ROM_KERNEL_AUTO, &p)) simt.push_back(p);
+    }
+    if (!tc && !f64) {
+        Rank2Plan p0{};
         int nact = 0;
-        if (h->Kp <= 128 && h->comp_cs <= 0 && plan_rank2_cta_f32(h->Kp, M, h->R, &p0)) simt.push_back(p0);
-        if (h->Kp > 128 && h->comp_cs <= 0 && plan_rank2_async(h->Kp, M, h->R, false, &p0) &&
-            async_beats_two_block(p0.Wa))
-            simt.push_back(p0);
-        p0.async = false;
         if (plan_rank2_split_f32(h->Kp, M, h->R, &p0)) nact = p0.max_active_clusters;
         else if (plan_rank2_simt_f32(h->Kp, M, h->R, false, &p0)) nact = p0.max_active_clusters;
         const int budgets[3] = {nact, nact / 2, nact / 4};
@@ -878,9 +880,6 @@ rom_status rom_autotune(rom_t h, int prec, int M, int probe_steps, double* best_
             if (plan_rank2_split_f32(h->Kp, M, h->R, &p, b)) { p.variant = 2; simt.push_back(p); }
             if (plan_rank2_simt_f32(h->Kp, M, h->R, false, &p, b)) { p.variant = 1; simt.push_back(p); }
         }
-        // above Kp = 512 the planner's own choice (clusters of Kp/64, 4 or 2
-        // CTAs; the budgeted plans above keep Kp/64)
-        if (h->Kp > 512 && nact > 0 && p0.variant == 1) simt.push_back(p0);
         // the saturated split kernel with 4, 8 or 12 fewer columns per block,
         // the freed columns on the streaming companion (clusters of 2 or 4)
         Rank2Plan ps;

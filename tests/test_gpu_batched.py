@@ -250,6 +250,28 @@ def test_autotune_single_handle(rom):
     assert np.linalg.norm(V3.cpu().numpy() - a) <= 1e-4 * np.linalg.norm(a)
 
 
+def test_autotune_tries_the_untuned_plan(rom):
+    """K = 512, M = 300: the planner's companion (20 columns; 10.1 us a step) is
+    none of the splits the tuner lists, the best of which takes 11.1."""
+    p = inputs.make_problem(512, 512, 300, 0, seed=4)
+    h = rom.Rom.from_problem(p)
+    V, S, T = rom.Rom.new_state(512, 300, "fp32"), rom.Rom.new_state(512, 300, "fp32"), torch.as_tensor(p.T, device="cuda")
+
+    def us_per_step(N=300):
+        best = 1e30
+        for _ in range(4):
+            a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            a.record()
+            h.run_rank2(V, S, T, N, prec="fp32")
+            b.record()
+            torch.cuda.synchronize()
+            best = min(best, 1e3 * a.elapsed_time(b) / N)
+        return best
+    untuned = us_per_step()
+    assert h.autotune(300, "fp32", probe_steps=300) <= 1.03 * untuned
+    assert us_per_step() <= 1.03 * untuned
+
+
 def test_autotune_single_handle_above_512(rom):
     """K = 768: the planner picks clusters of 4 or 2 for the streamed
     operators; the tuner, which also times that plan, keeps one of the
