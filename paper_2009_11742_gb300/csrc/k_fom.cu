@@ -668,7 +668,10 @@ cudaError_t launch_march(FomPass<T> a, const FomShape& s, int nsm, cudaStream_t 
     const size_t smem = ((size_t)(2 * NS + 4 * fom_stages<NS>()) * kFomThreads * (s.wide ? VWIDE : 1) +
                          (size_t)8 * (a.seg_rows + NS + 3)) * sizeof(T);
     const void* fn = s.wide ? (const void*)fom_march_kernel<T, VWIDE, NS> : (const void*)fom_march_kernel<T, 1, NS>;
-    if (smem > 48 * 1024) cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (smem > 48 * 1024) {
+        const cudaError_t e = allow_smem(fn, smem);
+        if (e != cudaSuccess) return e;
+    }
     // An FP32 pass may start before the last one has ended: its launch, and what
     // it does before it needs the state, are then hidden (us a step, M = 1:
     // 512 x 2048 6.0 -> 5.7, 40 x 100 2.45 -> 2.12; M = 2, 128 x 512 3.1 -> 2.5).

@@ -134,7 +134,7 @@ static cudaError_t launch_ens_nt(const Rank1EnsArgs& a, cudaStream_t st) {
     const int KS = ens_ksplit(NT, a.Kp);
     const size_t smem = sizeof(T) * (size_t)(2 * a.Kp + KS * a.Kp);
     auto fn = (a.Xv || a.Xs) ? rank1_ensemble_kernel<T, NT, true> : rank1_ensemble_kernel<T, NT, false>;
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem((const void*)fn, smem);
     if (e != cudaSuccess) return e;
     fn<<<a.M, NT, smem, st>>>(a);
     return cudaGetLastError();

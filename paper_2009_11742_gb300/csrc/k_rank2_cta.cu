@@ -52,7 +52,7 @@ cudaError_t launch_rank2_cta_f32(const Rank2Args& a_in, const Rank2Plan& p, cuda
     a.Wa = p.Wa;
     a.c_global = p.c_global ? 1 : 0;
     void* fn = cta_kernel(p.KI, p.cb, a.Xv != nullptr || a.Xs != nullptr);
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem);
+    cudaError_t e = allow_smem(fn, p.smem);
     if (e != cudaSuccess) return e;
     void* args[] = {(void*)&a};
     return cudaLaunchKernel(fn, dim3((unsigned)p.nclusters), dim3(kThreads), args, p.smem, st);

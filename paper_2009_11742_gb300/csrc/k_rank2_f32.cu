@@ -18,11 +18,12 @@ size_t worklist_smem(int W, int Kp, int rpc, int nrt) {
     return rank2_smem_layout<float>(W, Kp, rpc, nrt).total;
 }
 
-// 1 KB is left for the kernel's static shared memory.
+// Left for the kernel's static shared memory.
+constexpr size_t kWlStatic = 1024;
 int worklist_max_clusters(int cs, size_t smem) {
-    if (cs < 1 || cs > 16 || smem + 1024 > (size_t)device_smem_optin()) return 0;
+    if (cs < 1 || cs > 16 || smem + kWlStatic > (size_t)device_smem_optin()) return 0;
     void* fn = worklist_fn();
-    if (prepare_kernel<float>(fn, smem) != cudaSuccess) return 0;
+    if (prepare_kernel<float>(fn, smem, kWlStatic) != cudaSuccess) return 0;
     ClusterLaunch probe(cs, 1, kThreads, smem);
     return probe.max_active(fn);
 }
@@ -30,7 +31,7 @@ int worklist_max_clusters(int cs, size_t smem) {
 cudaError_t launch_rank2_worklist_f32(const Rank2Args& a, int cs, int ncl, size_t smem, cudaStream_t st) {
     if (!a.group || !a.items || !a.item_counter || cs < 1 || cs > 16 || ncl < 1) return cudaErrorInvalidValue;
     void* fn = worklist_fn();
-    cudaError_t e = prepare_kernel<float>(fn, smem);
+    cudaError_t e = prepare_kernel<float>(fn, smem, kWlStatic);
     if (e != cudaSuccess) return e;
     ClusterLaunch L(cs, ncl, kThreads, smem, st);
     void* args[] = {(void*)&a};

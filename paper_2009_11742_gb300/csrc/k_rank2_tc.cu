@@ -199,8 +199,7 @@ static bool plan_rank2_tcs(int Kp, int M, int R, int Wforce, TcPlan* p) {
             if (tcs_smem_bytes(W, s) <= (size_t)smax) { stages = s; break; }
         if (!fn || stages == 0) continue;
         const size_t smem = tcs_smem_bytes(W, stages);
-        if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
-            cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+        if (prepare_kernel<float>(fn, smem) != cudaSuccess) {
             cudaGetLastError();
             continue;
         }
@@ -236,8 +235,7 @@ bool plan_rank2_tc(int prec, int Kp, int M, int R, int Wforce, TcPlan* p) {
     if (!fn64) return false;
     const size_t smem64 = tc_smem_for(prec, 64, 2, p->rpc, Kp);
     if (smem64 > (size_t)smax) return false;
-    if (cudaFuncSetAttribute(fn64, cudaFuncAttributeMaxDynamicSharedMemorySize, smax) != cudaSuccess ||
-        cudaFuncSetAttribute(fn64, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+    if (prepare_kernel<float>(fn64, smem64) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
@@ -280,9 +278,7 @@ cudaError_t launch_rank2_tc(const TcArgs& a_in, const TcPlan& p, cudaStream_t st
         if (smem > smax) return cudaErrorInvalidValue;
         a.stages = s;
     }
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    cudaError_t e = prepare_kernel<float>(fn, smem);
     if (e != cudaSuccess) return e;
     ClusterLaunch L(p.cs, p.nclusters, p.prec == ROM_BF16S ? kTcsThreads : kTcThreads, smem, st);
     void* args[] = {(void*)&a};

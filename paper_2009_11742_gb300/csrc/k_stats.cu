@@ -16,6 +16,7 @@
 #include <math.h>
 
 #include "../../include/rom.h"
+#include "rom_internal.h"
 
 namespace romk {
 
@@ -382,7 +383,7 @@ extern "C" rom_status rom_trace_stats(const float* traces, int nrec, int R, int 
                                  : (const void*)trace_stats_kernel<32, 4>;
     const size_t smem = stat_smem_layout(M, a.G, nprobs, W).total;
     cudaError_t e = cudaSuccess;
-    if (smem > 48 * 1024) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (smem > 48 * 1024) e = allow_smem(fn, smem);
     if (e == cudaSuccess) {
         void* args[] = {(void*)&a};
         e = cudaLaunchKernel(fn, dim3((unsigned)nblk), dim3(kStatThreads), args, smem, static_cast<cudaStream_t>(stream));

@@ -105,16 +105,9 @@ static void* rank2_kernel(int KI, int cb, bool* resident) {
     return nullptr;
 }
 
-static int device_smem_optin() {
-    int dev = 0, v = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&v, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    return v;
-}
-
 template <typename T>
-static cudaError_t prepare_kernel(void* fn, size_t smem) {
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+static cudaError_t prepare_kernel(void* fn, size_t smem, size_t fixed = 0) {
+    cudaError_t e = allow_smem(fn, smem, fixed);
     if (e != cudaSuccess) return e;
     return cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
 }

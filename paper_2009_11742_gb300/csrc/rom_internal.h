@@ -14,6 +14,22 @@ void set_last_error(const char* msg);
 // a status: ROM_E_NOMEM for an allocation failure, ROM_E_CUDA otherwise.
 rom_status cuda_fail(cudaError_t e, const char* where);
 
+// Shared memory a block of the current device can have (opt-in).
+inline int device_smem_optin() {
+    int dev = 0, v = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&v, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    return v;
+}
+// Lets kernel fn have `smem` bytes of dynamic shared memory beside `fixed` static
+// ones.  The limit belongs to the kernel, not to a launch, and a thread may set it
+// between another's setting and launch: so every caller sets the same, all there is.
+inline cudaError_t allow_smem(const void* fn, size_t smem, size_t fixed = 0) {
+    const size_t most = (size_t)device_smem_optin();
+    if (smem + fixed > most) return cudaErrorInvalidValue;
+    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(most - fixed));
+}
+
 // Arguments of one rank-2 launch (all device pointers).  Element type T of
 // the state-like buffers is double for ROM_FP64 and float otherwise.
 // One operator of a grouped (rank-3) launch: its handle's device copies.
