@@ -60,27 +60,26 @@ static bool plan_async(int Kp, int M, int R, Rank2Plan* p) {
     p->resident = true;
     p->variant = 1;
     const int rpc = (R + p->cs - 1) / p->cs;
-    p->c_global = (size_t)rpc * Kp * sizeof(T) > 64 * 1024;
-    const int nC = p->c_global ? 0 : rpc;
-    int dev = 0, nsm = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     const size_t smax = (size_t)device_smem_optin();
-    auto bytes = [&](int w, int cb) { return async_smem_layout<T>(w, w / cb, Kp, nC).total; };
-    // one CTA per SM: the clusters that fit are those of the widest block
+    auto bytes = [&](int w, int cb, int nC) { return async_smem_layout<T>(w, w / cb, Kp, nC).total; };
+    // one CTA per SM
     void* probe_fn = async_kernel<T>(p->KI, 4);
-    const size_t probe_smem = bytes(4, 4) > smax / 2 + 1024 ? bytes(4, 4) : smax / 2 + 1024;
-    if (probe_smem > smax || prepare_kernel<T>(probe_fn, probe_smem) != cudaSuccess) return false;
+    const size_t probe_smem = smax / 2 + 1024;
+    if (prepare_kernel<T>(probe_fn, probe_smem) != cudaSuccess) return false;
     ClusterLaunch probe(p->cs, 1, kThreads, probe_smem);
     p->max_active_clusters = probe.max_active(probe_fn);
     if (p->max_active_clusters <= 0) return false;
     int w = (M + p->max_active_clusters - 1) / p->max_active_clusters;
     p->cb = async_group(w, sizeof(T) == 8);
     w = (w + p->cb - 1) / p->cb * p->cb;
-    while (w > p->cb && bytes(w, p->cb) > smax) w -= p->cb;
+    // receiver rows are staged while they take at most 64 KB, or fit beside the
+    // columns
+    p->c_global = (size_t)rpc * Kp * sizeof(T) > 64 * 1024 && bytes(w, p->cb, rpc) > smax;
+    const int nC = p->c_global ? 0 : rpc;
+    while (w > p->cb && bytes(w, p->cb, nC) > smax) w -= p->cb;
     p->Wv = p->Wa = w;
     p->nclusters = (M + w - 1) / w;
-    p->smem = bytes(w, p->cb);
+    p->smem = bytes(w, p->cb, nC);
     p->async = p->smem <= smax;
     return p->async;
 }

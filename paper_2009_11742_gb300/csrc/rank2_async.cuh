@@ -162,20 +162,21 @@ __device__ __forceinline__ double async_wavelet(const Rank2Args& a, int n, const
 }
 
 // Receiver traces of the first nc columns of group X for this CTA's nj rows of
-// C: one dot product per warp at a time, or in FP32 with more of them than
-// warps a tile of 4 receivers x CB columns (the same values: lanes sum the same
-// stripes and meet in the same order).
+// C: one dot product per warp at a time, or with many of them (in FP32 with 4
+// columns: more than warps) a tile of 4 receivers x CB columns (the same values:
+// lanes sum the same stripes and meet in the same order).  1000 receivers on
+// every step, us a step one by one / in tiles: FP64 K = 256 M = 100 174 / 110,
+// rank-1 FP32 K = 512 8.5 / 2.2 (rows staged beyond 64 KB, too).
 template <typename T, int CB>
 __device__ __forceinline__ void async_traces(const T* C, const T* X, int Kp, int nj, int nc, int warp, int lane,
                                              T* out, int R) {
     using Lay = AsyncLayout<T, CB>;
-    if constexpr (sizeof(T) == 4 && CB == 4) {
-        if (nj * nc > kThreads / 32) {
-            for (int j0 = 4 * warp; j0 < nj; j0 += 4 * (kThreads / 32)) trace_tile(C, X, Kp, j0, nj, nc, lane, out, R);
-            return;
-        }
+    constexpr int kWarps = kThreads / 32;
+    if (sizeof(T) == 4 && CB == 4 ? nj * nc > kWarps : nj >= 4 * kWarps) {
+        for (int j0 = 4 * warp; j0 < nj; j0 += 4 * kWarps) trace_group<T, CB>(C, X, Kp, j0, nj, nc, lane, out, R);
+        return;
     }
-    for (int pr = warp; pr < nj * nc; pr += kThreads / 32) {
+    for (int pr = warp; pr < nj * nc; pr += kWarps) {
         const int jj = pr / nc, c = pr - jj * nc;
         T acc = T(0);
         for (int k = 4 * lane; k < Kp; k += 128) {

@@ -134,93 +134,66 @@ __device__ __forceinline__ void load_op_quad(float (&op)[4][4 * KI], const float
     }
 }
 
-// One stage of a 32-lane reduce-scatter of 16 values: lanes with bit `o`
-// set keep the upper H entries, the others the lower H, each adding its
-// partner's copy of the entries it keeps.
-template <int H>
-__device__ __forceinline__ void rs32_stage(float (&v)[16], int lane, int o) {
-    const bool up = (lane & o) != 0;
+// Sums of NV values (a power of two, at most 16) over the 32 lanes: entry
+// lane / (32 / NV) is returned.  Lanes with bit `o` set keep the upper half of
+// what is left, the others the lower, each adding its partner's copy; the last
+// stages add what the remaining lanes hold of one entry.  The order is that of a
+// butterfly over each value, so the bits are, too.
+template <typename T, int NV>
+__device__ __forceinline__ T reduce_scatter32(T (&v)[NV], int lane) {
+    int o = 16;
 #pragma unroll
-    for (int i = 0; i < H; ++i) {
-        const float send = up ? v[i] : v[i + H];
-        const float keep = up ? v[i + H] : v[i];
-        v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
-    }
-}
-
-// Receiver traces y = C V^{n+1} of one block (Sec. 4.5.2): out[c R + jj] for
-// this CTA's nj receiver rows Cown (row-major, Kp wide) and the nc columns of
-// the new V in Xb (columns xstride apart, Kp rows), dealt out to nwarps warps.  A warp takes a tile of 4
-// receivers x 4 columns over the whole K: each lane sums 4-wide stripes of k
-// into 16 independent accumulators, then a 32-lane reduce-scatter (fixed
-// order) leaves entry lane / 2 of the tile in lanes 2e and 2e + 1.
-__device__ __forceinline__ void split_traces(const float* __restrict__ Cown, const float* __restrict__ Xb,
-                                             int Kp, int nj, int nc, int warp, int lane,
-                                             float* __restrict__ out, int R, int xstride,
-                                             int nwarps) {
-    const int tcn = (nc + 3) >> 2;
-    const int ntile = ((nj + 3) >> 2) * tcn;
-    for (int t = warp; t < ntile; t += nwarps) {
-        const int tj = t / tcn;
-        const int j0 = 4 * tj, c0 = 4 * (t - tj * tcn);
-        float acc[16];
+    for (int H = NV / 2; H > 0; H >>= 1, o >>= 1) {
+        const bool up = (lane & o) != 0;
 #pragma unroll
-        for (int i = 0; i < 16; ++i) acc[i] = 0.f;
-#pragma unroll 1
-        for (int k = 4 * lane; k < Kp; k += 128) {
-            float cv[4][4], xv[4][4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                load4(Cown + (size_t)min(j0 + u, nj - 1) * Kp + k, cv[u]);
-                load4(Xb + (size_t)min(c0 + u, nc - 1) * xstride + k, xv[u]);
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-#pragma unroll
-                for (int w = 0; w < 4; ++w)
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) acc[4 * u + w] = __fmaf_rn(cv[u][q], xv[w][q], acc[4 * u + w]);
+        for (int i = 0; i < H; ++i) {
+            const T send = up ? v[i] : v[i + H];
+            const T keep = up ? v[i + H] : v[i];
+            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
         }
-        rs32_stage<8>(acc, lane, 16);
-        rs32_stage<4>(acc, lane, 8);
-        rs32_stage<2>(acc, lane, 4);
-        rs32_stage<1>(acc, lane, 2);
-        acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], 1);
-        const int e = lane >> 1, jj = j0 + (e >> 2), c = c0 + (e & 3);
-        if ((lane & 1) == 0 && jj < nj && c < nc) out[(size_t)c * R + jj] = acc[0];
     }
+#pragma unroll
+    for (int q = 16 / NV; q > 0; q >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], q);
+    return v[0];
 }
 
-// Traces of receivers j0 .. j0 + 3 (of the nj rows of C) for the first nc of a
-// group's 4 columns: split_traces' tile on the exchange layout, by one warp.
-__device__ __forceinline__ void trace_tile(const float* C, const float* X, int Kp, int j0, int nj, int nc, int lane,
-                                           float* out, int R) {
-                    float acc[16];
+// Receiver traces y = C V^{n+1} (Sec. 4.5.2) of receivers j0 .. j0 + RT - 1 (of
+// the nj rows of C, Kp wide) for the first nc of CT columns, by one warp:
+// out[c R + jj].  Each lane sums 4-wide stripes of k into RT CT independent
+// accumulators; load(c, kq, x) gives rows 4 kq .. 4 kq + 3 of column c.
+template <int RT, int CT, typename T, typename Load>
+__device__ __forceinline__ void trace_tile(const T* C, int Kp, int j0, int nj, int nc, int lane, T* out, int R,
+                                           const Load& load) {
+    T acc[RT * CT];
 #pragma unroll
-                    for (int i = 0; i < 16; ++i) acc[i] = 0.f;
+    for (int i = 0; i < RT * CT; ++i) acc[i] = T(0);
 #pragma unroll 1
-                    for (int k = 4 * lane; k < Kp; k += 128) {
-                        float cv[4][4], xv[4][4];
+    for (int k = 4 * lane; k < Kp; k += 128) {
+        T cv[RT][4], xv[CT][4];
 #pragma unroll
-                        for (int u = 0; u < 4; ++u) {
-                            load4(C + (size_t)min(j0 + u, nj - 1) * Kp + k, cv[u]);
-                            AsyncLayout<float, 4>::load(X, u, k >> 2, xv[u]);
-                        }
+        for (int u = 0; u < RT; ++u) load4(C + (size_t)min(j0 + u, nj - 1) * Kp + k, cv[u]);
 #pragma unroll
-                        for (int u = 0; u < 4; ++u)
+        for (int w = 0; w < CT; ++w) load(w, k >> 2, xv[w]);
 #pragma unroll
-                            for (int w = 0; w < 4; ++w)
+        for (int u = 0; u < RT; ++u)
 #pragma unroll
-                                for (int q = 0; q < 4; ++q)
-                                    acc[4 * u + w] = __fmaf_rn(cv[u][q], xv[w][q], acc[4 * u + w]);
-                    }
-                    rs32_stage<8>(acc, lane, 16);
-                    rs32_stage<4>(acc, lane, 8);
-                    rs32_stage<2>(acc, lane, 4);
-                    rs32_stage<1>(acc, lane, 2);
-                    acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], 1);
-                    const int e = lane >> 1, jj = j0 + (e >> 2), c = e & 3;
-                    if ((lane & 1) == 0 && jj < nj && c < nc) out[(size_t)c * R + jj] = acc[0];
+            for (int w = 0; w < CT; ++w)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) acc[CT * u + w] = fmadd(cv[u][q], xv[w][q], acc[CT * u + w]);
+    }
+    const T y = reduce_scatter32<T, RT * CT>(acc, lane);
+    constexpr int LPE = 32 / (RT * CT);  // lanes an entry
+    const int e = lane / LPE, jj = j0 + e / CT, c = e % CT;
+    if (lane % LPE == 0 && jj < nj && c < nc) out[(size_t)c * R + jj] = y;
+}
+
+// The same for 4 receivers and the first nc of a group's CB columns X on the
+// exchange layout.
+template <typename T, int CB>
+__device__ __forceinline__ void trace_group(const T* C, const T* X, int Kp, int j0, int nj, int nc, int lane, T* out,
+                                            int R) {
+    trace_tile<4, CB, T>(C, Kp, j0, nj, nc, lane, out, R,
+                         [&](int c, int kq, T (&x)[4]) { AsyncLayout<T, CB>::load(X, c, kq, x); });
 }
 
 // The products of the thread's 4 rows with a group's 4 columns, reduced over the
@@ -509,8 +482,8 @@ __global__ void __launch_bounds__(kThreads, 1) rank2_split_kernel(const Rank2Arg
                 if (record) {  // before this warp's S lets V be overwritten
                     const int nt = (nj + 3) >> 2;
                     for (int t = (warp + kSplitWarps - g * nt % kSplitWarps) % kSplitWarps; t < nt; t += kSplitWarps)
-                        trace_tile(Cown, Xg, Kp, 4 * t, nj, min(CB, ncol - CB * g), lane,
-                                   traces + ((size_t)rec * a.Mtot + gc0 + CB * g) * a.R + s * a.rpc, a.R);
+                        trace_group<float, CB>(Cown, Xg, Kp, 4 * t, nj, min(CB, ncol - CB * g), lane,
+                                               traces + ((size_t)rec * a.Mtot + gc0 + CB * g) * a.R + s * a.rpc, a.R);
                     __syncwarp();
                 }
                 link.send(g, y);

@@ -239,8 +239,8 @@ __global__ void __launch_bounds__(kStrThreads, 1) rank2_stream_kernel(const Rank
                     for (int sl = crank; sl < H; sl += CSZ) {
                         const int nj = min(rpc, a.R - sl * rpc);
                         for (int j0 = 4 * warp; j0 < nj; j0 += 4 * NW)
-                            trace_tile(Cp + (size_t)sl * rpc * Kp, Vf, Kp, j0, nj, ncol, lane,
-                                       traces + ((size_t)rec * a.Mtot + col0) * a.R + sl * rpc, a.R);
+                            trace_group<float, CB>(Cp + (size_t)sl * rpc * Kp, Vf, Kp, j0, nj, ncol, lane,
+                                                   traces + ((size_t)rec * a.Mtot + col0) * a.R + sl * rpc, a.R);
                     }
                     to_rec = a.r;
                     ++rec;

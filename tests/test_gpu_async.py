@@ -14,11 +14,12 @@ pytestmark = pytest.mark.gpu
 
 # columns per cluster 1, 2, 3 and 4, ragged
 # rows and last clusters, one step, steps around the forcing table's
-# 32, few and many receivers
+# 32, few and many receivers (300 and more: tiles of 4 receivers, staged beyond 64 KB)
 @pytest.mark.parametrize("Kv,Ks,M,R,N,r", [
     (129, 192, 1, 2, 33, 4), (192, 150, 40, 3, 64, 1), (256, 256, 9, 100, 31, 2), (200, 256, 31, 7, 70, 9),
     (512, 512, 7, 64, 40, 5), (512, 500, 14, 1, 1, 1), (512, 512, 27, 40, 65, 8), (512, 512, 28, 9, 40, 3),
-    (384, 380, 25, 33, 36, 6)])
+    (384, 380, 25, 33, 36, 6),
+    (256, 256, 1, 300, 12, 1), (250, 256, 30, 301, 9, 2), (512, 512, 3, 800, 6, 3)])
 @pytest.mark.parametrize("form", ["ricker", "gauss1", "ftab", "xref"])
 def test_async_bitwise_two_block(rom, Kv, Ks, M, R, N, r, form):
     p = inputs.make_problem(Kv, Ks, M, R, seed=Kv + M)
@@ -62,13 +63,15 @@ def test_async_f64(rom, Kv, Ks, M):
             assert np.linalg.norm(a.cpu().numpy() - b) <= 1e-13 * np.linalg.norm(b)
 
 
-# wider blocks: several column groups of 1, 2 and 4 columns, ragged last clusters, and
-# (M = 1100) more clusters than fit at once
-@pytest.mark.parametrize("Kv,Ks,M,group", [(128, 128, 150, 1), (128, 120, 200, 2), (128, 128, 512, 4),
-                                           (256, 256, 269, 2), (200, 256, 300, 4), (256, 250, 1100, 4),
-                                           (60, 64, 500, 4), (64, 64, 380, 1)])
-def test_async_f64_several_groups(rom, Kv, Ks, M, group):
-    N, r, R = 9, 2, 7
+# wider blocks: several column groups of 1, 2 and 4 columns, ragged last clusters,
+# (M = 1100) more clusters than fit at once, and many receivers (tiles of 4, staged up to
+# and beyond 64 KB, or, R = 1000, read from global memory)
+@pytest.mark.parametrize("Kv,Ks,M,R,group", [
+    (128, 128, 150, 7, 1), (128, 120, 200, 7, 2), (128, 128, 512, 7, 4), (256, 256, 269, 7, 2), (200, 256, 300, 7, 4),
+    (256, 250, 1100, 7, 4), (60, 64, 500, 7, 4), (64, 64, 380, 7, 1), (128, 128, 150, 301, 1), (256, 256, 269, 300, 2),
+    (60, 64, 500, 203, 4), (256, 250, 269, 1000, 2)])
+def test_async_f64_several_groups(rom, Kv, Ks, M, R, group):
+    N, r = 9, 2
     p = inputs.make_problem(Kv, Ks, M, R, seed=M)
     h = rom.Rom.from_problem(p)
     W = h.plan(M, "fp64")["cols_per_block"]

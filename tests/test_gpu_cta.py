@@ -38,11 +38,13 @@ def one_run(rom, h, p, kernel, N, r, ftab=None, n0=3):
 
 # (Kv, Ks, M, R, N, r): both Kp, every column group, one block and several,
 # more blocks than SMs, steps on both sides of the forcing table's length,
-# receiver rows staged and (R = 200 at Kp = 128) read from global memory
+# receiver rows staged and (R = 200 at Kp = 128) read from global memory, and many
+# receivers of one column (8 x 1 tiles: R = 77 and more)
 @pytest.mark.parametrize("Kv,Ks,M,R,N,r", [
     (1, 1, 1, 0, 1, 0), (64, 64, 1, 1, 33, 1), (63, 2, 2, 5, 31, 2), (17, 40, 3, 64, 32, 3), (64, 50, 305, 3, 40, 7),
     (30, 64, 1300, 2, 20, 20), (65, 65, 1, 9, 65, 5), (128, 128, 2, 3, 64, 64), (100, 90, 5, 3, 50, 5),
-    (90, 128, 153, 4, 30, 9), (128, 127, 460, 200, 12, 4), (66, 128, 1100, 1, 9, 3)])
+    (90, 128, 153, 4, 30, 9), (128, 127, 460, 200, 12, 4), (66, 128, 1100, 1, 9, 3),
+    (64, 64, 1, 200, 12, 4), (128, 120, 1, 77, 12, 1), (100, 128, 150, 130, 6, 2)])
 @pytest.mark.parametrize("form", ["ricker", "gauss1", "ftab", "xref"])
 def test_cta_bitwise_split(rom, Kv, Ks, M, R, N, r, form):
     p = inputs.make_problem(Kv, Ks, M, R, seed=Kv + M)
