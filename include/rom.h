@@ -461,7 +461,11 @@ size_t rom_adjoint_workspace_size(rom_t h, int M, int nsteps, int ckpt_every, in
  *            every value finite.
  *   probs    host array of nprobs probabilities in [0, 1] (nprobs <= 16).
  *   mean_out device double, nrec x R (may be NULL): mean over the M
- *            realizations, summed in FP64 by a fixed pairwise tree.
+ *            realizations.  The sum is exact over integers that hold each
+ *            value to 2^-56 of the column's largest or better (2^-65 up to
+ *            M = 512) and rounded once; columns with an infinity or NaN, or
+ *            whose largest magnitude is below about 2^-105, are added up in
+ *            FP64 in order.
  *   q_out    device double, nprobs x nrec x R (may be NULL): for each p the
  *            quantile by linear interpolation between order statistics
  *            (Hyndman-Fan type 7): h = (M - 1) p, i = floor(h), t = h - i,

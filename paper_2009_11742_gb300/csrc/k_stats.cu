@@ -168,23 +168,29 @@ __global__ void __launch_bounds__(kStatThreads, stat_blocks<EPL, W>()) trace_sta
     const int k0 = (int)(blockIdx.x / ntj) * a.nr, j0 = (int)(blockIdx.x % ntj) * a.nj;
     const int nr = min(a.nr, a.nrec - k0), nj = min(a.nj, a.R - j0);
     const int nc = nr * nj;                        // column c = rr nj + jj
-    // ---- the tile: consecutive threads on consecutive receivers, all records
-    // in one loop (the rows of a record follow those of the last)
+    // ---- the tile: consecutive threads on consecutive receivers; several records
+    // in one loop (the rows of a record follow those of the last).  A tile of one
+    // record has a loop without the record's bookkeeping, in which the loads
+    // stay ahead of the stores (1000 x 64 x 512: 180 us, 215 with one loop for both).
     {
         int lg = 0;
         while ((1 << lg) < nj) ++lg;
         const int jj = tid & ((1 << lg) - 1), step = kStatThreads >> lg;
         const float* src = a.traces + (size_t)k0 * M * a.R + j0 + jj;
-        const int nrow = jj < nj ? nr * M : 0;
-        int m = tid >> lg, c = jj;                 // row of the record, column of the tile
+        if (jj < nj && nr == 1) {
 #pragma unroll 4
-        for (int p = tid >> lg; p < nrow; p += step) {
-            if (m >= M) {
-                c += m / M * nj;
-                m %= M;
+            for (int m = tid >> lg; m < M; m += step) tile[m * TS + jj] = src[(size_t)m * a.R];
+        } else if (jj < nj) {
+            int m = tid >> lg, c = jj;             // row of the record, column of the tile
+#pragma unroll 4
+            for (int p = m; p < nr * M; p += step) {
+                if (m >= M) {
+                    c += m / M * nj;
+                    m %= M;
+                }
+                tile[m * TS + c] = src[(size_t)p * a.R];
+                m += step;
             }
-            tile[m * TS + c] = src[(size_t)p * a.R];
-            m += step;
         }
     }
     __syncthreads();
