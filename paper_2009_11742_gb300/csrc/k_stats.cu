@@ -150,6 +150,22 @@ __device__ __forceinline__ void stat_exchange(int (&x)[EPL], int* xb, int wcol, 
 template <int EPL, int W>
 __host__ __device__ constexpr int stat_blocks() { return EPL <= 16 ? 6 : (W == 1 ? 4 : 2); }
 
+// Rows p, p + step, .. of nr short records (M rows each, R values apart in src),
+// receiver jj of nj, to the tile.
+__device__ __noinline__ void stat_load_rows(float* tile, const float* src, int R, int M, int nr, int nj, int jj,
+                                            int p, int step, int TS) {
+    int m = p, c = jj;                             // row of the record, column of the tile
+#pragma unroll 4
+    for (; p < nr * M; p += step) {
+        if (m >= M) {
+            c += m / M * nj;
+            m %= M;
+        }
+        tile[m * TS + c] = src[(size_t)p * R];
+        m += step;
+    }
+}
+
 // EPL values a lane, W warps a column (W > 1: EPL = 32).
 template <int EPL, int W>
 __global__ void __launch_bounds__(kStatThreads, stat_blocks<EPL, W>()) trace_stats_kernel(const StatArgs a) {
@@ -168,28 +184,23 @@ __global__ void __launch_bounds__(kStatThreads, stat_blocks<EPL, W>()) trace_sta
     const int k0 = (int)(blockIdx.x / ntj) * a.nr, j0 = (int)(blockIdx.x % ntj) * a.nj;
     const int nr = min(a.nr, a.nrec - k0), nj = min(a.nj, a.R - j0);
     const int nc = nr * nj;                        // column c = rr nj + jj
-    // ---- the tile: consecutive threads on consecutive receivers; several records
-    // in one loop (the rows of a record follow those of the last).  A tile of one
-    // record has a loop without the record's bookkeeping, in which the loads
-    // stay ahead of the stores (1000 x 64 x 512: 180 us, 215 with one loop for both).
+    // ---- the tile: consecutive threads on consecutive receivers.  Record by
+    // record while one gives every thread 4 loads in flight; of short records, all
+    // rows in one loop (the rows of a record follow those of the last), whose
+    // bookkeeping costs long ones (1000 x 64 x 512: 180 us, 215 with this loop).
     {
         int lg = 0;
         while ((1 << lg) < nj) ++lg;
         const int jj = tid & ((1 << lg) - 1), step = kStatThreads >> lg;
-        const float* src = a.traces + (size_t)k0 * M * a.R + j0 + jj;
-        if (jj < nj && nr == 1) {
+        if (nr > 1 && M < 4 * step) {
+            if (jj < nj) stat_load_rows(tile, a.traces + (size_t)k0 * M * a.R + j0 + jj, a.R, M, nr, nj, jj, tid >> lg, step, TS);
+        } else {
+            for (int rr = 0; rr < nr; ++rr) {
+                const float* src = a.traces + (size_t)(k0 + rr) * M * a.R + j0 + jj;
+                if (jj < nj) {
 #pragma unroll 4
-            for (int m = tid >> lg; m < M; m += step) tile[m * TS + jj] = src[(size_t)m * a.R];
-        } else if (jj < nj) {
-            int m = tid >> lg, c = jj;             // row of the record, column of the tile
-#pragma unroll 4
-            for (int p = m; p < nr * M; p += step) {
-                if (m >= M) {
-                    c += m / M * nj;
-                    m %= M;
+                    for (int m = tid >> lg; m < M; m += step) tile[m * TS + rr * nj + jj] = src[(size_t)m * a.R];
                 }
-                tile[m * TS + c] = src[(size_t)p * a.R];
-                m += step;
             }
         }
     }
@@ -303,36 +314,32 @@ __global__ void __launch_bounds__(kStatThreads, stat_blocks<EPL, W>()) trace_sta
     }
 }
 
-// Columns per tile.  16 keep 6 blocks on an SM at M = 512.  With too few
-// columns for the GPU's resident blocks a tile has fewer: first down to one turn
-// of the block's warps, then to as few as give every tile an SM of its own (a
-// turn takes as long for one column as for a warp each, but two one-column
-// blocks on an SM may share a scheduler: 300 columns of M = 1000 in 200 blocks
-// 18.8 us, in 100 below 15).  us a call with one receiver, tiles of 8 to 32
-// columns whatever their number / these / one block a column: M = 256, 100
-// records 20.7 / 12.6 / 14.3, M = 512, 100 records 18.5 / 12.6 / 14.5, M = 4000,
-// 10 records 53.5 / 16.8 / 37.2 (about 12.5 is the host's part).
+// Columns per tile.  16 keep 6 blocks on an SM at M = 512.  With less than two
+// tiles an SM, a tile has fewer: first down to one turn of the block's warps,
+// then to as few as give every tile an SM of its own (a turn takes as long for
+// one column as for a warp each, but two one-column blocks on an SM may share a
+// scheduler: 300 columns of M = 1000 in 200 blocks 18.8 us, in 100 below 15).  us
+// a call with one receiver, tiles of 8 to 32 columns whatever their number /
+// these / one block a column: M = 256, 100 records 20.7 / 12.6 / 14.3, M = 512,
+// 100 records 18.5 / 12.6 / 14.5, M = 4000, 10 records 53.5 / 16.8 / 37.2 (about
+// 12.5 is the host's part).  Smaller tiles beyond that cost turns and reads:
+// 1000 records of 20 receivers, M = 200, tiles of 20 39, of 10 51.
 static void stat_tiles(StatArgs& a, int W, long long* nblk) {
     int dev = 0, nsm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    const int res = a.M <= 512 ? stat_blocks<16, 1>() : (W == 1 ? stat_blocks<32, 1>() : stat_blocks<32, 2>());
-    // receivers of one record, evenly, or with few of them several records
+    // the tiles for at most G columns: receivers of one record, or with few of
+    // them several records
     auto cut = [&](int G) {
         a.G = G;
-        a.nj = (a.R + G - 1) / G;
-        a.nj = (a.R + a.nj - 1) / a.nj;
+        a.nj = a.R < G ? a.R : G;
         a.nr = G / a.nj;
-        *nblk = ((long long)(a.nrec + a.nr - 1) / a.nr) * ((a.R + a.nj - 1) / a.nj);
+        return *nblk = ((long long)(a.nrec + a.nr - 1) / a.nr) * ((a.R + a.nj - 1) / a.nj);
     };
     int G = a.M <= 256 ? 32 : (a.M <= 512 ? 16 : 8);
-    while (G > kStatWarps / W && (long long)a.nrec * a.R < (long long)G * nsm * res) G /= 2;
-    cut(G);
-    while (G > 1) {
-        cut(G / 2);
-        if (*nblk > nsm) break;
-        G /= 2;
-    }
+    while (cut(G) < 2 * nsm && G > kStatWarps / W) G /= 2;
+    if (G <= kStatWarps / W)
+        while (G > 1 && cut(G / 2) <= nsm) G /= 2;
     cut(G);
 }
 
