@@ -150,30 +150,31 @@ __device__ __forceinline__ void cta_half(const float (&op)[RT][4 * KI], const fl
     }
 }
 
-// Receiver traces of the block's ncol columns (ST apart), in tiles of 4 receivers
-// x 4 columns, or of one column, where there are many receivers, 8 x 1 (Kp = 128,
-// one column, 1000 receivers, read from global memory, on every step: 16.4 us a
-// step in tiles of 4 x 4, 6.9 in these).
-template <int ST>
+// Receiver traces of the block's ncol columns (ST apart) in tiles of 4 receivers
+// x 4 columns, of a one-column block in tiles of 8 receivers (Kp = 128, us a step
+// with 4 x 4 / 8 x 1: 1000 receivers, read from global memory, on every step
+// 16.4 / 6.9, 64 receivers 1.35 / 0.81).
+template <int ST, int CB>
 __device__ __forceinline__ void cta_traces(const float* C, const float* V, int Kp, int R, int ncol, int warp, int lane,
                                            float* out) {
     constexpr int kWarps = kThreads / 32;
-    if (ncol == 1 && R >= 8 * kWarps) {
+    if constexpr (CB == 1) {
         for (int j0 = 8 * warp; j0 < R; j0 += 8 * kWarps)
             trace_tile<8, 1, float>(C, Kp, j0, R, 1, lane, out, R,
-                                     [&](int, int kq, float (&x)[4]) { load4(V + 4 * kq, x); });
-        return;
-    }
-    const int tcn = (ncol + 3) >> 2, ntile = ((R + 3) >> 2) * tcn;
-    for (int t = warp; t < ntile; t += kWarps) {
-        const int tj = t / tcn, c0 = 4 * (t - tj * tcn), nc = ncol - c0;
-        trace_tile<4, 4, float>(C, Kp, 4 * tj, R, nc, lane, out + (size_t)c0 * R, R,
-                                [&](int c, int kq, float (&x)[4]) { load4(V + (c0 + min(c, nc - 1)) * ST + 4 * kq, x); });
+                                    [&](int, int kq, float (&x)[4]) { load4(V + 4 * kq, x); });
+    } else {
+        const int tcn = (ncol + 3) >> 2, ntile = ((R + 3) >> 2) * tcn;
+        for (int t = warp; t < ntile; t += kWarps) {
+            const int tj = t / tcn, c0 = 4 * (t - tj * tcn), nc = ncol - c0;
+            trace_tile<4, 4, float>(
+                C, Kp, 4 * tj, R, nc, lane, out + (size_t)c0 * R, R,
+                [&](int c, int kq, float (&x)[4]) { load4(V + (c0 + min(c, nc - 1)) * ST + 4 * kq, x); });
+        }
     }
 }
 
 template <int KI, int CB, bool XR>
-__global__ void __launch_bounds__(kThreads, KI == 1 ? 2 : 1) rank2_cta_kernel(const Rank2Args a) {
+__global__ void __launch_bounds__(kThreads, 1) rank2_cta_kernel(const Rank2Args a) {
     constexpr int NT = kThreads, Kp = 64 * KI, ST = Kp + kCtaPad;
     constexpr int RT = 4 * KI;                      // rows per thread
     constexpr int NV = CtaTile<RT, CB>::NV, NG = CtaTile<RT, CB>::NG;
@@ -249,7 +250,7 @@ __global__ void __launch_bounds__(kThreads, KI == 1 ? 2 : 1) rank2_cta_kernel(co
         __syncthreads();
         cta_half<KI, RT, CB, false, XR>(opB, V, S, cS, yS, kS, g, nullptr, dt, Wa, row, j, Xs, a.Ks, ncol);
         if (traces && --to_rec == 0) {
-            cta_traces<ST>(Crows, V, Kp, a.R, ncol, warp, lane, traces + ((size_t)rec * a.Mtot + gc0) * a.R);
+            cta_traces<ST, CB>(Crows, V, Kp, a.R, ncol, warp, lane, traces + ((size_t)rec * a.Mtot + gc0) * a.R);
             to_rec = a.r;
             ++rec;
         }
