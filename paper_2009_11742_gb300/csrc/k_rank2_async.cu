@@ -2,36 +2,21 @@
 // (FP32, Kp <= 512; FP64, Kp <= 256).
 #include <cuda_runtime.h>
 
-#include "rank2_async.cuh"
+#include "rank2_async_launch.cuh"
 #include "rank2_launch.cuh"
 
 namespace romk {
 
-template <typename T, int KI>
-static void* async_kernel_for(int cb) {
-    return cb == 1   ? (void*)&rank2_async_kernel<T, KI, 1>
-           : cb == 2 ? (void*)&rank2_async_kernel<T, KI, 2>
-                     : (void*)&rank2_async_kernel<T, KI, 4>;
-}
 template <typename T>
-static void* async_kernel(int KI, int cb) {
-    switch (KI) {
-        case 1: return async_kernel_for<T, 1>(cb);
-        case 2: return async_kernel_for<T, 2>(cb);
-        case 3: return async_kernel_for<T, 3>(cb);
-        case 4: return async_kernel_for<T, 4>(cb);
-        default: break;
-    }
-    if constexpr (sizeof(T) == 4) {
-        switch (KI) {
-            case 5: return async_kernel_for<T, 5>(cb);
-            case 6: return async_kernel_for<T, 6>(cb);
-            case 7: return async_kernel_for<T, 7>(cb);
-            case 8: return async_kernel_for<T, 8>(cb);
-            default: break;
-        }
-    }
-    return nullptr;
+static void* async_kernel(int KI, int cb) { return async_instance<T, false>(KI, cb); }
+
+// Does a run take its traces in tiles of receivers (rpc of them a CTA)?  us a step
+// with one dot product a warp at a time / in tiles, records on every step: rank-1
+// FP32 K = 512 16 receivers (1 a CTA) 1.35 / 1.39, 100 (7) 1.53 / 1.42, 1000 8.4
+// / 2.1; FP64 K = 256, M = 100 1000 receivers 174 / 110.  In FP64 a tile of few
+// receivers keeps one warp at it where several shared the dot products.
+static bool async_many(const Rank2Args& a, int cb, bool f64) {
+    return a.traces && (f64 ? a.rpc >= 32 : cb < 4 && a.rpc >= 6);
 }
 
 // The column group for w columns.  FP64 is bound by the FP64 units, so no
@@ -91,7 +76,8 @@ static cudaError_t launch_async(const Rank2Args& a_in, const Rank2Plan& p, cudaS
     a.Wa = p.Wa;
     a.rpc = (a.R + p.cs - 1) / p.cs;
     a.c_global = p.c_global ? 1 : 0;
-    void* fn = async_kernel<T>(p.KI, p.cb);
+    void* fn = async_many(a, p.cb, sizeof(T) == 8) ? async_many_kernel(sizeof(T) == 8, p.KI, p.cb)
+                                                   : async_kernel<T>(p.KI, p.cb);
     if (!fn || a.group) return cudaErrorInvalidValue;
     cudaError_t e = prepare_kernel<T>(fn, p.smem);
     if (e != cudaSuccess) return e;

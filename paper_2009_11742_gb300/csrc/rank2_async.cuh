@@ -163,16 +163,14 @@ __device__ __forceinline__ double async_wavelet(const Rank2Args& a, int n, const
 
 // Receiver traces of the first nc columns of group X for this CTA's nj rows of
 // C: one dot product per warp at a time, or with many of them (in FP32 with 4
-// columns: more than warps) a tile of 4 receivers x CB columns (the same values:
-// lanes sum the same stripes and meet in the same order).  1000 receivers on
-// every step, us a step one by one / in tiles: FP64 K = 256 M = 100 174 / 110,
-// rank-1 FP32 K = 512 8.5 / 2.2 (rows staged beyond 64 KB, too).
-template <typename T, int CB>
+// columns: more than warps; MANY) a tile of 4 receivers x CB columns (the same
+// values: lanes sum the same stripes and meet in the same order).
+template <typename T, int CB, bool MANY>
 __device__ __forceinline__ void async_traces(const T* C, const T* X, int Kp, int nj, int nc, int warp, int lane,
                                              T* out, int R) {
     using Lay = AsyncLayout<T, CB>;
     constexpr int kWarps = kThreads / 32;
-    if (sizeof(T) == 4 && CB == 4 ? nj * nc > kWarps : nj >= 4 * kWarps) {
+    if (MANY || (sizeof(T) == 4 && CB == 4 && nj * nc > kWarps)) {
         for (int j0 = 4 * warp; j0 < nj; j0 += 4 * kWarps) trace_group<T, CB>(C, X, Kp, j0, nj, nc, lane, out, R);
         return;
     }
@@ -192,7 +190,10 @@ __device__ __forceinline__ void async_traces(const T* C, const T* X, int Kp, int
     }
 }
 
-template <typename T, int KI, int CB>
+// MANY: the form for many receivers (async_many).  An instance of its own, since
+// the other trace code alone makes the compiler lay out the whole step
+// differently (K = 192, 28 columns, no traces: 0.86 -> 0.92 us a step).
+template <typename T, int KI, int CB, bool MANY>
 __global__ void __launch_bounds__(kThreads, 1) rank2_async_kernel(const Rank2Args a) {
     using Lay = AsyncLayout<T, CB>;
     constexpr int Kp = 64 * KI, NV = 2 * CB;
@@ -372,7 +373,7 @@ __global__ void __launch_bounds__(kThreads, 1) rank2_async_kernel(const Rank2Arg
                 const T y = state_add(y0, inc, carry);
                 if (sizeof(T) == 4 && active) *cp = carry;
                 if (record)  // before this warp's S lets V be overwritten
-                    async_traces<T, CB>(Crows, Vc, Kp, nj, min(CB, ncol - g * CB), warp, lane,
+                    async_traces<T, CB, MANY>(Crows, Vc, Kp, nj, min(CB, ncol - g * CB), warp, lane,
                                     traces + ((size_t)rec * a.Mtot + gc0 + g * CB) * a.R + jr0, a.R);
                 __syncwarp();
                 async_send<CB>(y, mS + (unsigned)g * kGroupBytes, mB + 8u * (unsigned)(G + g), zw, dpeer, lane, npeer);
