@@ -884,7 +884,7 @@ def bench_fom(args, torch, dev, inputs, rom):
                         "basis": f"{2 * es // spp} B per unknown per realization per step "
                                  f"(every state value read once and written once; {spp} steps a pass)"},
            "rank1": {"value": N / t1, "ms_per_step": 1e3 * t1 / N,
-                     "achieved_gbs": 2.0 * es * nun * N / t1 / 1e9},
+                     "achieved_gbs": 2.0 * es * nun * N / spp / t1 / 1e9},
            "rank2_over_rank1_per_realization": (M * N / t) / (N / t1)}
     print(json.dumps(out), flush=True)
     return 0
