@@ -150,24 +150,18 @@ __device__ __forceinline__ void stat_exchange(int (&x)[EPL], int* xb, int wcol, 
 template <int EPL, int W>
 __host__ __device__ constexpr int stat_blocks() { return EPL <= 16 ? 6 : (W == 1 ? 4 : 2); }
 
-// Rows p, p + step, .. of nr short records (M rows each, R values apart in src),
-// receiver jj of nj, to the tile.
-__device__ __noinline__ void stat_load_rows(float* tile, const float* src, int R, int M, int nr, int nj, int jj,
-                                            int p, int step, int TS) {
-    int m = p, c = jj;                             // row of the record, column of the tile
-#pragma unroll 4
-    for (; p < nr * M; p += step) {
-        if (m >= M) {
-            c += m / M * nj;
-            m %= M;
-        }
-        tile[m * TS + c] = src[(size_t)p * R];
-        m += step;
-    }
+// log2 of the threads that read a row of nj receivers side by side.
+__host__ __device__ inline int stat_row_lanes(int nj) {
+    int lg = 0;
+    while ((1 << lg) < nj) ++lg;
+    return lg;
 }
 
-// EPL values a lane, W warps a column (W > 1: EPL = 32).
-template <int EPL, int W>
+// EPL values a lane, W warps a column (W > 1: EPL = 32).  SHORT: the tile's
+// records are short, and their rows are read in one loop (the rows of a record
+// follow those of the last), whose bookkeeping costs long ones (1000 x 64 x 512:
+// 180 us, 215 with it), as does its mere presence beside the other (182).
+template <int EPL, int W, bool SHORT>
 __global__ void __launch_bounds__(kStatThreads, stat_blocks<EPL, W>()) trace_stats_kernel(const StatArgs a) {
     static_assert(W == 1 || EPL == 32, "wide columns hold 1024 values a warp");
     constexpr int B = EPL * 32 * W <= 512 ? 21 : 18;
@@ -184,16 +178,22 @@ __global__ void __launch_bounds__(kStatThreads, stat_blocks<EPL, W>()) trace_sta
     const int k0 = (int)(blockIdx.x / ntj) * a.nr, j0 = (int)(blockIdx.x % ntj) * a.nj;
     const int nr = min(a.nr, a.nrec - k0), nj = min(a.nj, a.R - j0);
     const int nc = nr * nj;                        // column c = rr nj + jj
-    // ---- the tile: consecutive threads on consecutive receivers.  Record by
-    // record while one gives every thread 4 loads in flight; of short records, all
-    // rows in one loop (the rows of a record follow those of the last), whose
-    // bookkeeping costs long ones (1000 x 64 x 512: 180 us, 215 with this loop).
+    // ---- the tile: consecutive threads on consecutive receivers
     {
-        int lg = 0;
-        while ((1 << lg) < nj) ++lg;
+        const int lg = stat_row_lanes(nj);
         const int jj = tid & ((1 << lg) - 1), step = kStatThreads >> lg;
-        if (nr > 1 && M < 4 * step) {
-            if (jj < nj) stat_load_rows(tile, a.traces + (size_t)k0 * M * a.R + j0 + jj, a.R, M, nr, nj, jj, tid >> lg, step, TS);
+        if constexpr (SHORT) {
+            const float* src = a.traces + (size_t)k0 * M * a.R + j0 + jj;
+            int m = tid >> lg, c = jj;             // row of the record, column of the tile
+#pragma unroll 4
+            for (int p = m; p < (jj < nj ? nr * M : 0); p += step) {
+                if (m >= M) {
+                    c += m / M * nj;
+                    m %= M;
+                }
+                tile[m * TS + c] = src[(size_t)p * a.R];
+                m += step;
+            }
         } else {
             for (int rr = 0; rr < nr; ++rr) {
                 const float* src = a.traces + (size_t)(k0 + rr) * M * a.R + j0 + jj;
@@ -343,6 +343,17 @@ static void stat_tiles(StatArgs& a, int W, long long* nblk) {
     cut(G);
 }
 
+template <bool SHORT>
+static const void* stat_kernel(int M) {
+    if (M <= 32) return (const void*)trace_stats_kernel<1, 1, SHORT>;
+    if (M <= 64) return (const void*)trace_stats_kernel<2, 1, SHORT>;
+    if (M <= 128) return (const void*)trace_stats_kernel<4, 1, SHORT>;
+    if (M <= 256) return (const void*)trace_stats_kernel<8, 1, SHORT>;
+    if (M <= 512) return (const void*)trace_stats_kernel<16, 1, SHORT>;
+    if (M <= 1024) return (const void*)trace_stats_kernel<32, 1, SHORT>;
+    return M <= 2048 ? (const void*)trace_stats_kernel<32, 2, false> : (const void*)trace_stats_kernel<32, 4, false>;
+}
+
 static bool device_pointer(const void* p) {
     cudaPointerAttributes at{};
     if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
@@ -386,14 +397,9 @@ extern "C" rom_status rom_trace_stats(const float* traces, int nrec, int R, int 
     long long nblk = 0;
     stat_tiles(a, W, &nblk);
     if ((long long)nrec * R > 0x7fffffffLL) return ROM_E_INVAL;
-    const void* fn = M <= 32     ? (const void*)trace_stats_kernel<1, 1>
-                     : M <= 64   ? (const void*)trace_stats_kernel<2, 1>
-                     : M <= 128  ? (const void*)trace_stats_kernel<4, 1>
-                     : M <= 256  ? (const void*)trace_stats_kernel<8, 1>
-                     : M <= 512  ? (const void*)trace_stats_kernel<16, 1>
-                     : M <= 1024 ? (const void*)trace_stats_kernel<32, 1>
-                     : M <= 2048 ? (const void*)trace_stats_kernel<32, 2>
-                                 : (const void*)trace_stats_kernel<32, 4>;
+    // several records a tile, too short to keep 3 loads a thread in flight each
+    const bool shrt = a.nr > 1 && M < 3 * (kStatThreads >> stat_row_lanes(a.nj));
+    const void* fn = shrt ? stat_kernel<true>(M) : stat_kernel<false>(M);
     const size_t smem = stat_smem_layout(M, a.G, nprobs, W).total;
     cudaError_t e = cudaSuccess;
     if (smem > 48 * 1024) e = allow_smem(fn, smem);
